@@ -219,8 +219,8 @@ vr_status vr_precompute_morphology(vr_ctx* ctx, int vol_id, const float* h_sigma
 vr_status vr_load_second_channel(vr_ctx* ctx, int vol_id, const void* data, int on_device, vr_dtype dtype);
 
 /* Set transfer-function and tissue uniforms (copied), then re-classify the
- * bricks (and, with derived bricks, the cells) for empty-space skipping: two
- * small kernels, tens of microseconds. Nothing else is recomputed (the uniform
+ * bricks and the cells for empty-space skipping: a few small kernels, tens of
+ * microseconds. Nothing else is recomputed (the uniform
  * buffers of the abstract and Sec. 4). Errors: INVALID_ARG (bad sizes or
  * values), NOT_READY (mode 2 without vesselness or a second channel), OOM, CUDA.
  * Argument errors change nothing; after an OOM or CUDA error the volume is
@@ -248,9 +248,8 @@ vr_status vr_set_normalized(vr_ctx* ctx, int vol_id, const float* d_norm);
 vr_status vr_get_bricks(vr_ctx* ctx, int vol_id, unsigned short* h_grid, unsigned char* h_empty, int* h_nb);
 
 /* Edge of the skip bricks of a volume, in interpolation cells: 4, 8 (the default)
- * or 16. The brick min/max grid, the empty-brick flags, the per-cell empty bits and
- * the derived bricks of the voxel-wise derivatives are kept per skip brick; empty
- * skip bricks are jumped a brick at a time. Rebuilds the grid at once; the volume
+ * or 16. The brick min/max grid, the empty-brick flags and the derived bricks of the
+ * voxel-wise derivatives are kept per skip brick. Rebuilds the grid at once; the volume
  * then needs vr_precompute_morphology again (NOT_READY until then), which also
  * re-classifies under the current tissue parameters. The images do not depend on
  * the size (skipping is bit-neutral); the evaluated-sample counter does. The

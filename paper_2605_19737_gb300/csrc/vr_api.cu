@@ -39,8 +39,8 @@ struct Volume {
     float* d_vessel = nullptr;
     float* d_vbricks = nullptr;
     float* d_dbricks = nullptr;  // derived bricks (voxel-wise I, gradient, Hessian) or nullptr
-    uint16_t* d_cellq = nullptr;     // after the morphology precompute: per-cell quantised min/max
-    uint32_t* d_cellmask = nullptr;  // and per-cell empty bits under the current transfer function
+    uint32_t* d_cellq = nullptr;  // after the morphology precompute: per-cell quantised min/max
+    uint8_t* d_skip = nullptr;    // and the skip field under the current transfer function, with its scratch
     float* d_smax = nullptr;  // per-scale max Hessian norm (8 floats)
     float* d_ch2 = nullptr;   // second channel: [0, 2) its I_min, I_max, [4, 8) its VolConst
     bool v_ready = false;     // d_vessel holds a complete second channel (vesselness or a modality)
@@ -166,7 +166,7 @@ void free_volume(vr_ctx* ctx, Volume* v) {
     dfree(ctx, v->d_vbricks);
     dfree(ctx, v->d_dbricks);
     dfree(ctx, v->d_cellq);
-    dfree(ctx, v->d_cellmask);
+    dfree(ctx, v->d_skip);
     dfree(ctx, v->d_smax);
     dfree(ctx, v->d_ch2);
     dfree(ctx, v->d_tf);
@@ -237,7 +237,9 @@ void fill_launch(RenderLaunch& L, const Volume* v, int W, int H, int skip) {
     L.vol.bricks = v->d_bricks;
     L.vol.vbricks = (v->tp.tf_mode == 2) ? v->d_vbricks : nullptr;
     L.vol.dbricks = v->d_dbricks;
-    L.vol.cellmask = v->d_cellmask;
+    L.vol.skipf = v->d_skip;  // the field comes first in its store
+    L.vol.skip_cx = v->n[0] - 1;
+    L.vol.skip_by = (v->n[1] - 1 + 3) >> 2;
     L.vol.empty = v->d_empty;
     L.vol.vc = v->d_vc;
     L.tp = v->tp;
@@ -252,18 +254,22 @@ vr_status rebuild_bricks(vr_ctx* ctx, Volume* v) {
     CK(launch_brick_minmax(v->d_norm, v->n, v->nb, v->bs, v->d_grid, ctx->stream), "brick min/max");
     if (v->d_dbricks)
         CK(launch_make_derived(v->d_norm, v->n, v->nb, v->bs, v->s, v->d_dbricks, ctx->stream), "derived bricks");
-    if (v->d_cellq) CK(launch_cell_minmax(v->d_norm, v->n, v->nb, v->bs, v->d_cellq, ctx->stream), "cell min/max");
+    if (v->d_cellq) CK(launch_cell_minmax(v->d_norm, v->n, v->d_cellq, ctx->stream), "cell min/max");
     return VR_OK;
 }
 
-// Brick skip flags and (once the morphology is precomputed) the per-cell empty bits
+// The classification scratch: tf_w + 1 prefix counts, then tf_w column limits.
+int* column_limits(const Volume* v) { return v->d_prefix + v->tp.tf_w + 1; }
+
+// Brick skip flags and (once the morphology is precomputed) the per-cell skip field
 // under the volume's current transfer function.
 vr_status classify_volume(vr_ctx* ctx, Volume* v) {
-    CK(launch_classify(v->d_grid, v->nbricks, v->d_tf, v->tp.tf_w, v->tp.tf_h, v->d_empty, v->d_prefix, ctx->stream),
+    CK(launch_classify(v->d_grid, v->nbricks, v->d_tf, v->tp.tf_w, v->tp.tf_h, v->d_empty, v->d_prefix,
+                       column_limits(v), ctx->stream),
        "classify");
-    if (v->d_cellmask)
-        CK(launch_classify_cells(v->d_cellq, v->nbricks, v->bs, v->d_prefix, v->tp.tf_w, v->d_cellmask, ctx->stream),
-           "classify cells");
+    if (v->d_skip)
+        CK(launch_skip_field(v->d_cellq, v->n, column_limits(v), v->tp.tf_w, skip_store(v->d_skip, v->n), ctx->stream),
+           "skip field");
     return VR_OK;
 }
 
@@ -476,14 +482,12 @@ vr_status vr_precompute_morphology(vr_ctx* ctx, int vol_id, const float* h_sigma
             v->d_dbricks = nullptr;  // fall back to the per-sample stencils
         }
     }
-    // per-cell min/max (4 B per cell) and per-cell empty bits, for either path
-    if (!v->d_cellq)
-        CK(dalloc(ctx, &v->d_cellq, (sizeof(uint16_t) * 2 * (size_t)v->nbricks) << (3 * v->bs)), "cell grid");
-    if (!v->d_cellmask)
-        CK(dalloc(ctx, &v->d_cellmask, sizeof(uint32_t) * (size_t)cell_words(v->bs) * v->nbricks), "cell flags");
+    // per-cell min/max (4 B per cell) and the skip field (1 B per cell + scratch), for either path
+    if (!v->d_cellq) CK(dalloc(ctx, &v->d_cellq, sizeof(uint32_t) * cellq_cells(v->n)), "cell grid");
+    if (!v->d_skip) CK(dalloc(ctx, &v->d_skip, skip_store_bytes(v->n)), "skip field");
     if (v->d_dbricks)
         CK(launch_make_derived(v->d_norm, v->n, v->nb, v->bs, v->s, v->d_dbricks, ctx->stream), "derived bricks");
-    CK(launch_cell_minmax(v->d_norm, v->n, v->nb, v->bs, v->d_cellq, ctx->stream), "cell min/max");
+    CK(launch_cell_minmax(v->d_norm, v->n, v->d_cellq, ctx->stream), "cell min/max");
     if (v->params_ready) {
         vr_status cs = classify_volume(ctx, v);
         if (cs != VR_OK) return cs;
@@ -552,7 +556,7 @@ vr_status vr_set_tissue_params(vr_ctx* ctx, int vol_id, const vr_tissue_params* 
         dfree(ctx, v->d_prefix);
         v->d_prefix = nullptr;
         v->prefix_cap = 0;
-        CK(dalloc(ctx, &v->d_prefix, sizeof(int) * (tp->tf_w + 1)), "classification scratch");
+        CK(dalloc(ctx, &v->d_prefix, sizeof(int) * (2 * (size_t)tp->tf_w + 1)), "classification scratch");
         v->prefix_cap = tp->tf_w + 1;
     }
     CK(cudaMemcpyAsync(v->d_tf, tp->tf, bytes, tp->tf_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -564,6 +568,7 @@ vr_status vr_set_tissue_params(vr_ctx* ctx, int vol_id, const vr_tissue_params* 
     d.gamma = tp->gamma, d.kappa_ref = tp->kappa_ref, d.w_max = tp->w_max;
     d.gk = (float)((double)tp->gamma / (double)tp->kappa_ref);
     d.inv_kref = (float)(1.0 / (double)tp->kappa_ref);
+    d.leap_per_cell = (float)((1.0 - 1e-6) / (double)tp->step_vox);
     d.ka = tp->ka, d.kd = tp->kd, d.ks = tp->ks;
     d.status = ctx->d_work + 1;
     d.opacity_scale = tp->opacity_scale, d.et_threshold = tp->et_threshold, d.step_vox = tp->step_vox;
@@ -694,15 +699,14 @@ vr_status vr_set_brick_size(vr_ctx* ctx, int vol_id, int cells) {
     if (bs == v->bs) return VR_OK;
     DeviceGuard g(ctx->device);
     CK(cudaStreamSynchronize(ctx->stream), "set_brick_size sync");
-    // the grid, flags, cells and derived bricks follow the new size; the derived
-    // bricks and the cell grid are rebuilt by the next vr_precompute_morphology
+    // the grid, flags and derived bricks follow the new size (the cell grid and the skip
+    // field do not depend on it); the derived bricks are rebuilt by the next
+    // vr_precompute_morphology
     v->morph_ready = false;
     dfree(ctx, v->d_grid);
     dfree(ctx, v->d_empty);
     dfree(ctx, v->d_dbricks);
-    dfree(ctx, v->d_cellq);
-    dfree(ctx, v->d_cellmask);
-    v->d_grid = nullptr, v->d_empty = nullptr, v->d_dbricks = nullptr, v->d_cellq = nullptr, v->d_cellmask = nullptr;
+    v->d_grid = nullptr, v->d_empty = nullptr, v->d_dbricks = nullptr;
     v->bs = bs;
     for (int a = 0; a < 3; ++a) v->nb[a] = (v->n[a] - 1 + (1 << bs) - 1) >> bs;
     v->nbricks = (long long)v->nb[0] * v->nb[1] * v->nb[2];

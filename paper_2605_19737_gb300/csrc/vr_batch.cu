@@ -13,7 +13,7 @@ namespace {
 // volume has derived bricks, so only that path is compiled in and the kernel is
 // held to 72 registers (measured: 110 Gsamples/s on the 256-view batch, against
 // 102 at 64 registers); otherwise each view takes its own path at run time.
-template <bool kAllDerived, int kBS>
+template <bool kAllDerived, bool kCount, int kBS>
 __device__ __forceinline__ void batch_body(const BatchLaunch& B) {
     const int lane = threadIdx.x & 31;
     unsigned rays_hit = 0, dense_tot = 0, eval_tot = 0, shade_tot = 0, interp_tot = 0;
@@ -43,60 +43,69 @@ __device__ __forceinline__ void batch_body(const BatchLaunch& B) {
         const bool hit = inside && setup_ray(vw.cam, vw.rc, i, j, v.n, v.s, r);
         float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
         unsigned dense = 0, evald = 0, shaded = 0, interp = 0;
-        if (hit) {
-            if (kAllDerived || v.dbricks)
-                march_gather<true, false, false, true, kBS>(v, vw.tp, reinterpret_cast<const float4*>(vw.tf), r,
-                                                             B.skip, inv_gmax, is, out, dense, evald, shaded, interp);
-            else
-                march_gather<false, false, false, true, kBS>(v, vw.tp, reinterpret_cast<const float4*>(vw.tf), r,
-                                                             B.skip, inv_gmax, is, out, dense, evald, shaded, interp);
-        }
+        if (!hit) r.ns = 0;
+        if (kAllDerived || v.dbricks)
+            march_gather<true, false, kCount, kBS>(v, vw.tp, reinterpret_cast<const float4*>(vw.tf), r, B.skip,
+                                                       inv_gmax, is, out, dense, evald, shaded, interp);
+        else
+            march_gather<false, false, kCount, kBS>(v, vw.tp, reinterpret_cast<const float4*>(vw.tf), r, B.skip,
+                                                        inv_gmax, is, out, dense, evald, shaded, interp);
         if (inside) reinterpret_cast<float4*>(vw.out)[(long long)j * vw.W + i] = out;
-        rays_hit += hit ? 1u : 0u;
-        dense_tot += dense;
-        eval_tot += evald;
-        shade_tot += shaded;
-        interp_tot += interp;
+        if (kCount) {
+            rays_hit += hit ? 1u : 0u;
+            dense_tot += dense;
+            eval_tot += evald;
+            shade_tot += shaded;
+            interp_tot += interp;
+        }
     }
-    if (B.counters) add_counters(B.counters, rays_hit, dense_tot, eval_tot, 0u, shade_tot, interp_tot);
+    if (kCount && B.counters) add_counters(B.counters, rays_hit, dense_tot, eval_tot, 0u, shade_tot, interp_tot);
 }
 
 // kBS: the skip-brick size shared by every view, or 0 when the views mix sizes.
-template <int kBS>
+template <bool kCount, int kBS>
 __global__ void __maxnreg__(72) k_render_batch_derived(const __grid_constant__ BatchLaunch B) {
-    batch_body<true, kBS>(B);
+    batch_body<true, kCount, kBS>(B);
 }
 
+template <bool kCount>
 __global__ void __launch_bounds__(256, 3) k_render_batch_mixed(const __grid_constant__ BatchLaunch B) {
-    batch_body<false, 0>(B);
+    batch_body<false, kCount, 0>(B);
 }
 
-template <int kBS>
-cudaError_t derived_ctas(int threads, int* per_sm) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_render_batch_derived<kBS>, threads, 0);
+template <bool kCount>
+void launch_derived(const BatchLaunch& B, int ctas, int threads, int bs, cudaStream_t st) {
+    if (bs == 2)
+        k_render_batch_derived<kCount, 2><<<ctas, threads, 0, st>>>(B);
+    else if (bs == 3)
+        k_render_batch_derived<kCount, 3><<<ctas, threads, 0, st>>>(B);
+    else if (bs == 4)
+        k_render_batch_derived<kCount, 4><<<ctas, threads, 0, st>>>(B);
+    else
+        k_render_batch_derived<kCount, 0><<<ctas, threads, 0, st>>>(B);
 }
 
 }  // namespace
 
 cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, int* per_sm) {
-    return all_derived ? derived_ctas<3>(warps_per_block * 32, per_sm)
-                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_render_batch_mixed,
+    // every variant of a family is held to the same registers, so one answers for all
+    return all_derived ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_render_batch_derived<false, 3>,
+                                                                       warps_per_block * 32, 0)
+                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_render_batch_mixed<false>,
                                                                        warps_per_block * 32, 0);
 }
 
 cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, bool all_derived, int bs,
                                 cudaStream_t st) {
     const int t = warps_per_block * 32;
-    if (!all_derived)
-        k_render_batch_mixed<<<ctas, t, 0, st>>>(B);
-    else if (bs == 2)
-        k_render_batch_derived<2><<<ctas, t, 0, st>>>(B);
-    else if (bs == 3)
-        k_render_batch_derived<3><<<ctas, t, 0, st>>>(B);
-    else if (bs == 4)
-        k_render_batch_derived<4><<<ctas, t, 0, st>>>(B);
+    if (all_derived && B.counters)
+        launch_derived<true>(B, ctas, t, bs, st);
+    else if (all_derived)
+        launch_derived<false>(B, ctas, t, bs, st);
+    else if (B.counters)
+        k_render_batch_mixed<true><<<ctas, t, 0, st>>>(B);
     else
-        k_render_batch_derived<0><<<ctas, t, 0, st>>>(B);
+        k_render_batch_mixed<false><<<ctas, t, 0, st>>>(B);
     return cudaGetLastError();
 }
 

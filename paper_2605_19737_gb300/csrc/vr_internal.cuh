@@ -40,8 +40,59 @@ __host__ __device__ __forceinline__ long long der_brick_floats(int bs) {
     const long long e = der_edge(bs);
     return e * e * e * kDerFloats;
 }
-// Per-cell empty bits of a skip brick: B^3 bits, in 32-bit words.
-__host__ __device__ __forceinline__ int cell_words(int bs) { return (1 << (3 * bs)) >> 5; }
+
+// Skip field: per interpolation cell one byte, the Chebyshev distance in cells to the
+// nearest cell that may hold opacity under the current transfer function, capped (0: the
+// cell itself may, so its samples are evaluated). Cells are stored in 4x4 columns of
+// (y, z), 16 bytes each, so that a 32-byte sector covers 2x4x4 cells and a line
+// 8x4x4: neighbouring rays and consecutive samples stay in a few sectors.
+struct SkipDims {
+    int cx, cy, cz;     // cells per axis, n - 1
+    int wx;             // 32-cell words per row of the cell bit grid
+    int bx, by, bz;     // 4^3-cell blocks per axis
+    int bwx;            // 32-block words per row of the block bit grid
+};
+__host__ __device__ __forceinline__ SkipDims skip_dims(const int n[3]) {
+    SkipDims d;
+    d.cx = n[0] - 1, d.cy = n[1] - 1, d.cz = n[2] - 1;
+    d.wx = (d.cx + 31) >> 5;
+    d.bx = (d.cx + 3) >> 2, d.by = (d.cy + 3) >> 2, d.bz = (d.cz + 3) >> 2;
+    d.bwx = (d.bx + 31) >> 5;
+    return d;
+}
+__host__ __device__ __forceinline__ size_t skip_index(int x, int y, int z, int cx, int by) {
+    return (size_t)(unsigned)(((z >> 2) * by + (y >> 2)) * cx + x) * 16 + (((y & 3) << 2) | (z & 3));
+}
+// One allocation holds the field and the scratch of its construction.
+struct SkipStore {
+    uint8_t* field;       // skip_index order
+    uint32_t* cell_bits;  // [cz][cy][wx], bit set = cell empty
+    uint32_t* block_bits; // [bz][by][bwx], bit set = 4^3 block empty
+    uint4* block_dist;    // [bz][by][bwx] distance in blocks to the nearest non-empty block, capped,
+                          // as four bit planes of 32 blocks
+};
+inline size_t skip_store_bytes(const int n[3]) {
+    const SkipDims d = skip_dims(n);
+    const size_t f = (size_t)d.bz * d.by * d.cx * 16;
+    const size_t c = ((size_t)d.cz * d.cy * d.wx * 4 + 15) & ~(size_t)15;
+    const size_t b = ((size_t)d.bz * d.by * d.bwx * 4 + 15) & ~(size_t)15;
+    return f + c + b + (size_t)d.bz * d.by * d.bwx * 16;
+}
+inline SkipStore skip_store(uint8_t* p, const int n[3]) {
+    const SkipDims d = skip_dims(n);
+    SkipStore s;
+    s.field = p;
+    p += (size_t)d.bz * d.by * d.cx * 16;
+    s.cell_bits = reinterpret_cast<uint32_t*>(p);
+    p += ((size_t)d.cz * d.cy * d.wx * 4 + 15) & ~(size_t)15;
+    s.block_bits = reinterpret_cast<uint32_t*>(p);
+    p += ((size_t)d.bz * d.by * d.bwx * 4 + 15) & ~(size_t)15;
+    s.block_dist = reinterpret_cast<uint4*>(p);
+    return s;
+}
+// Cells of the min/max grid per row, padded to whole warps.
+__host__ __device__ __forceinline__ int cellq_pitch(int nx) { return (nx - 1 + 31) & ~31; }
+inline size_t cellq_cells(const int n[3]) { return (size_t)cellq_pitch(n[0]) * (n[1] - 1) * (n[2] - 1); }
 constexpr size_t kDerivedBudgetBytes = (size_t)16 << 30;  // default: built only up to this size
 
 struct CamDev {
@@ -52,6 +103,12 @@ struct TissueDev {
     int tf_mode, tf_w, tf_h, grad_mod, shading;
     float gamma, kappa_ref, w_max, ka, kd, ks, opacity_scale, et_threshold, step_vox;
     float alpha_exp;  // dt / opacity_ref_step for the step-size opacity correction; 0 = off
+    // Samples per cell of leap: from a cell at distance d of the skip field, the d - 1
+    // layers of cells around it are empty and a sample moves no axis by more than step_vox
+    // cells, so the next floor((d - 1) leap_per_cell) samples are empty too and the one
+    // after is looked at. leap_per_cell = (1 - 1e-6) / step_vox: the margin exceeds the
+    // rounding of the step (2^-32 voxel per sample), so a leap never lands outside them.
+    float leap_per_cell;
     float gk, inv_kref;  // gamma / kappa_ref and 1 / kappa_ref (rounded from double on the host)
     unsigned* status;    // the context's device status word (debug builds report failed index checks there)
 };
@@ -90,9 +147,8 @@ struct VolumeDev {
     const float* vbricks;    // vesselness storage bricks (same layout) or nullptr
     const float* dbricks;    // derived skip bricks or nullptr (then the per-sample stencils are used)
     const uint8_t* empty;    // skip-brick flags, 1 = skip
-    const uint32_t* cellmask;  // skip bricks x cell_words(bs) words, bit (lz*B+ly)*B+lx set when that
-                               // cell is empty under the current transfer function (nullptr before
-                               // the precompute)
+    const uint8_t* skipf;    // skip field (nullptr before the precompute)
+    int skip_cx, skip_by;    // its cells per row and 4-cell blocks along y
     const VolConst* vc;
 };
 
@@ -211,11 +267,14 @@ cudaError_t launch_make_derived(const float* norm, const int n[3], const int nb[
                                 float* dbricks, cudaStream_t st);
 cudaError_t launch_gmax(const float* norm, const int n[3], const float s[3], VolConst* vc, cudaStream_t st);
 cudaError_t launch_classify(const uint16_t* grid, long long nbricks, const float* tf, int tf_w, int tf_h,
-                            uint8_t* empty, int* prefix_scratch /* tf_w + 1 ints */, cudaStream_t st);
-cudaError_t launch_cell_minmax(const float* norm, const int n[3], const int nb[3], int bs, uint16_t* cellq,
-                               cudaStream_t st);
-cudaError_t launch_classify_cells(const uint16_t* cellq, long long nbricks, int bs, const int* prefix, int tf_w,
-                                  uint32_t* cellmask, cudaStream_t st);
+                            uint8_t* empty, int* prefix_scratch /* tf_w + 1 ints */,
+                            int* limit /* nullable, tf_w: see k_tf_alpha_prefix */, cudaStream_t st);
+// Per interpolation cell the quantised (min, max) of its 8 corner voxels, low and high
+// 16 bits: [nz - 1][ny - 1][cellq_pitch(nx)].
+cudaError_t launch_cell_minmax(const float* norm, const int n[3], uint32_t* cellq, cudaStream_t st);
+// The skip field under the transfer function whose column limits are `limit`.
+cudaError_t launch_skip_field(const uint32_t* cellq, const int n[3], const int* limit, int tf_w, const SkipStore& s,
+                              cudaStream_t st);
 
 // Multi-scale vesselness of `norm` into V (both nvox floats); tmp_a and tmp_b are
 // nvox floats of scratch each, smax receives each scale's max Hessian norm.

@@ -35,8 +35,24 @@ __device__ __forceinline__ void add_counters(vr_counters* ctr, unsigned rays, un
     }
 }
 
-// Front-to-back march of one ray (Eqs. 4-6) over the bricked volume in HBM/L2,
-// skipping bricks classified empty. Shared by the single-view and batched kernels.
+// Front-to-back march of one ray (Eqs. 4-6) over the bricked volume in HBM/L2.
+// Shared by the single-view and batched kernels.
+// Empty space: a sample whose cell is empty under the transfer function has opacity
+// exactly 0 (its intensity lies in the range of the cell's 8 corners) and adds nothing.
+// The skip field holds, per cell, the distance to the nearest cell that may have
+// opacity, so one byte load both tests the cell and leaps over empty space; it needs no
+// brick state in registers.
+// The lanes of a warp walk in step: all at the same sample index k, advancing together
+// by the smallest leap any lane may take. Neighbouring rays then sit at the same
+// depth and their corner loads share cells; a lane that leapt alone would lose step for
+// the rest of its ray. Measured (1080p of the 181x217x181 head / vessel 256x256x176 at
+// 1080p / 540p of the head): single steps over empty cells inside bricks 2.15 / 0.367 /
+// 0.811 ms, each lane leaping for itself 2.16 / 0.134 / 0.90, warps in step 1.81 / 0.130
+// / 0.72. Bound by latency: ~0.45 issue slots used, two L1 round trips (byte, corners)
+// and the table's per sample.
+// kCount: the launch wants sample counters. Evaluated samples are defined by the
+// skip bricks (samples outside bricks classified empty), so this variant walks brick by
+// brick and sample by sample instead of leaping; the image is the same.
 // kHessianFirst: the derived path issues the Hessian loads before the table lookup,
 // so that they overlap it, or only after its zero-opacity test; the arithmetic, and
 // so the image, is the same. Every kernel now takes the first order (the batched
@@ -48,7 +64,9 @@ __device__ __forceinline__ void add_counters(vr_counters* ctr, unsigned rays, un
 // take the volume's at run time (batches that mix sizes); a fixed size keeps the
 // brick and cell index arithmetic in immediates (the run-time form measured 4-10 %
 // slower).
-template <bool kDerived, bool kState = false, bool kParity = false, bool kHessianFirst = true, int kBS = 3>
+// Called by whole warps; a lane without a ray passes r.ns = 0.
+constexpr unsigned kRayEnded = 0x7fffffffu;  // above any advance
+template <bool kDerived, bool kState, bool kCount, int kBS, bool kParity = false, bool kHessianFirst = true>
 __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
                                              const RayDev& r, int skip, float inv_gmax, const float is[3],
                                              float4& out, unsigned& dense, unsigned& evald, unsigned& shaded,
@@ -58,64 +76,63 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
     int klast = -1;      // kState: last evaluated sample
     int k1 = -1;         // kState: first sample with A >= 1 (where the adjoint sweep must start
     float T1 = 1.f;      // when early termination is off) and the transmittance in front of it
-    int k = 0, kstop = -1;
+    int k = 0;
     unsigned ne = 0, nsh = 0, nip = 0;
-    // The skip flag and the base pointers of the current brick are re-read only
-    // when the brick changes (about every 16 samples), keeping a dependent L1 round
-    // trip and the 64-bit address arithmetic off the path of every sample.
-    int cur_bi = -1;
-    bool cur_empty = false;
-    const float4* dbrick = nullptr;  // derived brick of cur_bi
     const int bs = kBS ? kBS : v.bs, B = 1 << bs, E = B + 1;
     // the position of sample k, u0 + k du, carried by exact integer additions
     long long U[3] = {r.u0[0], r.u0[1], r.u0[2]};
-    auto advance = [&](int k1) {
-        if (k1 == k + 1) {
+    auto step = [&]() {
 #pragma unroll
-            for (int q = 0; q < 3; ++q) U[q] += r.du[q];
-        } else {
-#pragma unroll
-            for (int q = 0; q < 3; ++q) U[q] += (long long)(k1 - k) * r.du[q];
-        }
-        k = k1;
+        for (int q = 0; q < 3; ++q) U[q] += r.du[q];
+        ++k;
     };
-    while (k < r.ns) {
-        int i0[3], bc[3];
+    auto leap = [&](int m) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            i0[q] = cell_index_at(U[q], v.n[q]);
-            bc[q] = i0[q] >> bs;
-        }
-        if (!VR_CHECK(tp.status, (unsigned)bc[0] < (unsigned)v.nb[0] && (unsigned)bc[1] < (unsigned)v.nb[1] &&
-                                     (unsigned)bc[2] < (unsigned)v.nb[2])) {
-            advance(k + 1);
-            continue;
-        }
-        const int bi = brick_index(v, bc);
-        if (bi != cur_bi) {
-            cur_bi = bi;
-            if (skip) cur_empty = __ldg(v.empty + bi) != 0;
-            if (kDerived)
-                dbrick = reinterpret_cast<const float4*>(
-                    v.dbricks + (size_t)bi * (kBS ? (size_t)der_brick_floats(kBS) : (size_t)v.der_stride));
-        }
-        if (skip && cur_empty) {
-            advance(brick_exit_k_at(r, U, bc, B, k, r.ns));
-            continue;
-        }
-        // local cell of (i0, j0, k0) within the skip brick: i0 - B bc = i0 & (B - 1)
-        const int lx = i0[0] & (B - 1), ly = i0[1] & (B - 1), lz = i0[2] & (B - 1);
-        if (skip && v.cellmask) {
-            // a cell classified empty holds only samples of opacity exactly 0 (their
-            // intensity lies in the range of its 8 corners): nothing to read or add
-            const int c = (((lz << bs) + ly) << bs) + lx;
-            if ((__ldg(v.cellmask + (size_t)bi * cell_words(bs) + (c >> 5)) >> (c & 31)) & 1u) {
-                ++ne;
-                advance(k + 1);
-                continue;
+        for (int q = 0; q < 3; ++q) U[q] += (long long)m * r.du[q];
+        k += m;
+    };
+    int ns = r.ns;  // samples of this ray, cut to the stopping one when it terminates early
+    while (true) {
+        int i0[3] = {0, 0, 0};
+        unsigned adv = kRayEnded;
+        if (k < ns) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) i0[q] = cell_index_at(U[q], v.n[q]);
+            adv = 0u;
+            if (!VR_CHECK(tp.status, (unsigned)i0[0] <= (unsigned)(v.n[0] - 2) &&
+                                         (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
+                                         (unsigned)i0[2] <= (unsigned)(v.n[2] - 2))) {
+                adv = 1u;
+            } else if (skip) {
+                bool out = false;
+                if (kCount || !v.skipf) {
+                    const int bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
+                    if (__ldg(v.empty + brick_index(v, bc))) {
+                        out = true;
+                        adv = (unsigned)(brick_exit_k_at(r, U, bc, B, k, ns) - k);
+                    }
+                }
+                if (!out && v.skipf) {
+                    adv = __ldg(v.skipf + skip_index(i0[0], i0[1], i0[2], v.skip_cx, v.skip_by));
+                    if (kCount && adv) {
+                        ++ne;
+                        adv = 1u;
+                    }
+                }
             }
         }
-        ++nip;
+        // without counters adv is a distance in cells (samples when there is no field)
+        const unsigned m = __reduce_min_sync(0xffffffffu, adv);
+        if (m) {
+            if (m == kRayEnded) break;
+            leap(kCount || !v.skipf ? (int)m : (int)((float)(m - 1u) * tp.leap_per_cell) + 1);
+            continue;
+        }
+        if (adv) {
+            step();
+            continue;
+        }
+        if (kCount) ++nip;
         // the sample's fractions, only for samples that are evaluated
         float f[3];
 #pragma unroll
@@ -126,6 +143,11 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
             v.vbricks ? value_eval(GlobalLoad{v.vbricks + (size_t)sbi * kBrickVox}, base, f[0], f[1], f[2]) : 0.0f;
         float fld[10], alpha, col[3];
         if (kDerived) {
+            // derived brick of the cell, and the cell's place in it
+            const int bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
+            const float4* dbrick = reinterpret_cast<const float4*>(
+                v.dbricks + (size_t)(unsigned)brick_index(v, bc) * (unsigned)(kBS ? der_brick_floats(kBS) : v.der_stride));
+            const int lx = i0[0] & (B - 1), ly = i0[1] & (B - 1), lz = i0[2] & (B - 1);
             // I and the gradient (one 16-byte load per corner) and the Hessian (two), then
             // the transfer function: a zero opacity entry makes alpha exactly 0 whatever
             // the Hessian, and the sample adds nothing (bit-neutral). The Hessian loads are
@@ -136,8 +158,8 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
             SampleOptics o;
             optics_tf(fld, vval, tp, tf, inv_gmax, o);
             if (o.c.w == 0.0f) {
-                ++ne;
-                advance(k + 1);
+                if (kCount) ++ne;
+                step();
                 continue;
             }
             if (!kHessianFirst) load_hessian<kParity>(tp, dbrick, E, lx, ly, lz, f, fld);
@@ -151,7 +173,7 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
             scale_field(fld, is);
             sample_optics(fld, vval, r.dir, tp, tf, inv_gmax, alpha, col);
         }
-        ++nsh;
+        if (kCount) ++nsh;
         const float wgt = (1.0f - A) * alpha;  // Eqs. 5-6
         fma2v(col[0], col[1], wgt, wgt, C0, C1);
         C2 = fmaf(col[2], wgt, C2);
@@ -164,15 +186,14 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
             k1 = k;
             T1 = 1.0f - A_prev;
         }
-        ++ne;
+        if (kCount) ++ne;
         if (A >= tp.et_threshold) {
-            kstop = k;
-            break;
+            ns = k + 1;
         }
-        advance(k + 1);
+        step();
     }
     out = make_float4(C0, C1, C2, A);
-    dense = kstop >= 0 ? (unsigned)(kstop + 1) : (unsigned)r.ns;
+    dense = (unsigned)ns;
     evald = ne;
     shaded = nsh;
     interp = nip;

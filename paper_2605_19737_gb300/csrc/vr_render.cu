@@ -7,8 +7,8 @@
 // bricks (voxel-wise I, gradient, Hessian: three 16-byte loads per corner) when
 // they were built, else the 56 weighted voxels of the 4x4x4 neighbourhood of the
 // intensity bricks with the separable stencils -- evaluates Eq. 4 and the
-// shading, and composites by Eqs. 5-6. Samples in bricks classified empty are
-// skipped a brick at a time (bit-neutral: their opacity is exactly zero).
+// shading, and composites by Eqs. 5-6. Empty cells are leapt over by the skip
+// field, the lanes of a warp in step (bit-neutral: their opacity is exactly zero).
 #include "vr_async.cuh"
 #include "vr_march.cuh"
 
@@ -20,7 +20,7 @@ namespace {
 // equal at 1080p, 2.5 % faster on the 8-view 512^2 workload than 72), 72 when it also
 // records the ray state (CTAs of at most 4 warps, 7 per SM: 1.5 % faster than 80 at 6;
 // 64 spills ~100 bytes), 80 for the stencils. CTAs of 2, 4 or 8 warps (tile_pixel).
-template <bool kDerived, bool kState, int kBS>
+template <bool kDerived, bool kState, bool kCount, int kBS>
 __global__ void __launch_bounds__(kState ? 128 : 256, kDerived ? (kState ? 7 : 4) : (kState ? 6 : 3))
     k_render_gather(const __grid_constant__ RenderLaunch L) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -42,19 +42,27 @@ __global__ void __launch_bounds__(kState ? 128 : 256, kDerived ? (kState ? 7 : 4
     unsigned dense = 0, evald = 0, shaded = 0, interp = 0;
     int kl = -1;
     float tl = 1.0f;
-    if (hit)
-        march_gather<kDerived, kState, false, true, kBS>(v, L.tp, tf, r, L.skip, inv_gmax, is, px, dense, evald,
-                                                         shaded, interp, &kl, &tl);
+    if (!hit) r.ns = 0;
+    march_gather<kDerived, kState, kCount, kBS>(v, L.tp, tf, r, L.skip, inv_gmax, is, px, dense, evald, shaded,
+                                                    interp, &kl, &tl);
     if (inside) {
         const long long pix = ((long long)(L.cam_offset + cam) * L.H + j) * L.W + i;
         reinterpret_cast<float4*>(L.out)[pix] = px;
         if (kState) L.ray_state[pix] = make_float2(__int_as_float(kl), tl);
-        if (L.ray_samples) {
+        if (kCount && L.ray_samples) {
             L.ray_samples[2 * pix] = dense;
             L.ray_samples[2 * pix + 1] = evald;
         }
     }
-    if (L.counters) add_counters(L.counters, hit ? 1u : 0u, dense, evald, 0u, shaded, interp);
+    if (kCount && L.counters) add_counters(L.counters, hit ? 1u : 0u, dense, evald, 0u, shaded, interp);
+}
+
+template <bool kDerived, bool kState, int kBS>
+void launch_gather_count(const RenderLaunch& L, dim3 grid, int threads, cudaStream_t st) {
+    if (L.counters || L.ray_samples)
+        k_render_gather<kDerived, kState, true, kBS><<<grid, threads, 0, st>>>(L);
+    else
+        k_render_gather<kDerived, kState, false, kBS><<<grid, threads, 0, st>>>(L);
 }
 
 }  // namespace
@@ -64,14 +72,14 @@ void launch_gather_bs(const RenderLaunch& L, dim3 grid, int threads, cudaStream_
     const bool state = L.ray_state != nullptr;
     if (L.vol.dbricks) {
         if (state)
-            k_render_gather<true, true, kBS><<<grid, threads, 0, st>>>(L);
+            launch_gather_count<true, true, kBS>(L, grid, threads, st);
         else
-            k_render_gather<true, false, kBS><<<grid, threads, 0, st>>>(L);
+            launch_gather_count<true, false, kBS>(L, grid, threads, st);
     } else {
         if (state)
-            k_render_gather<false, true, kBS><<<grid, threads, 0, st>>>(L);
+            launch_gather_count<false, true, kBS>(L, grid, threads, st);
         else
-            k_render_gather<false, false, kBS><<<grid, threads, 0, st>>>(L);
+            launch_gather_count<false, false, kBS>(L, grid, threads, st);
     }
 }
 
@@ -401,11 +409,8 @@ __global__ void __launch_bounds__(256, 3) k_render_staged_derived(const __grid_c
                     }
                     const int lx = i0[0] & (B - 1), ly = i0[1] & (B - 1), lz = i0[2] & (B - 1);
                     bool done_sample = false;
-                    if (L.skip && v.cellmask) {
-                        const int c = (((lz << kBS) + ly) << kBS) + lx;
-                        if ((__ldg(v.cellmask + (size_t)sel * cell_words(kBS) + (c >> 5)) >> (c & 31)) & 1u)
-                            done_sample = true;
-                    }
+                    if (L.skip && v.skipf)
+                        done_sample = __ldg(v.skipf + skip_index(i0[0], i0[1], i0[2], v.skip_cx, v.skip_by)) != 0;
                     if (!done_sample) {
                         ++nip;
                         float fld[10];
