@@ -187,6 +187,7 @@ struct RenderLaunch {
     int packet_w, packet_h;    // ray packet of a warp (packet_w * packet_h == 32); per-lane kernels: 4, 8 or 16 wide
     int tile_w, tile_h;        // per-lane kernels: CTA tile in pixels (tile_packets_x packets across)
     int tile_sx;               // log2 of the packets across the tile
+    int lanes;                 // k_render_lanes: lanes per ray
     unsigned* work_counter;    // staged kernel work queue (zeroed before launch)
     unsigned* status;          // device status word (kStatusTimeout on an expired wait)
     int n_packets_x, n_packets_y, n_work;

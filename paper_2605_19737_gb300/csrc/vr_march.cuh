@@ -35,6 +35,49 @@ __device__ __forceinline__ void add_counters(vr_counters* ctr, unsigned rays, un
     }
 }
 
+// Opacity and colour of the sample at position U in cell i0. False when its
+// transfer-function opacity is exactly zero (derived path): it adds nothing.
+// The Hessian loads are issued before that test so that they overlap the table lookup
+// (measured: equal at 1080p, 2-3 % faster on the 8-view and batched workloads than
+// loading them after it).
+template <bool kDerived, int kBS>
+__device__ __forceinline__ bool eval_sample(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
+                                            const long long U[3], const int i0[3], const float dir[3],
+                                            float inv_gmax, const float is[3], float& alpha, float col[3]) {
+    float f[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) f[q] = cell_frac_at(U[q], v.n[q]);
+    int base = 0, sbi = 0;
+    if (!kDerived || v.vbricks) sbi = storage_brick(v, i0, base);
+    const float vval =
+        v.vbricks ? value_eval(GlobalLoad{v.vbricks + (size_t)sbi * kBrickVox}, base, f[0], f[1], f[2]) : 0.0f;
+    float fld[10];
+    if (kDerived) {
+        // derived brick of the cell, and the cell's place in it; I and the gradient (one
+        // 16-byte load per corner), the Hessian (two), then the transfer function
+        const int bs = kBS ? kBS : v.bs, B = 1 << bs, E = B + 1;
+        const int bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
+        const float4* dbrick = reinterpret_cast<const float4*>(
+            v.dbricks + (size_t)(unsigned)brick_index(v, bc) * (unsigned)(kBS ? der_brick_floats(kBS) : v.der_stride));
+        const int lx = i0[0] & (B - 1), ly = i0[1] & (B - 1), lz = i0[2] & (B - 1);
+        derived_channels<false, 0, 4>(dbrick, E, lx, ly, lz, f[0], f[1], f[2], fld);
+        load_hessian<false>(tp, dbrick, E, lx, ly, lz, f, fld);
+        SampleOptics o;
+        optics_tf(fld, vval, tp, tf, inv_gmax, o);
+        if (o.c.w == 0.0f) return false;
+        optics_rest(fld, dir, tp, o);
+        alpha = o.alpha;
+        col[0] = o.col[0];
+        col[1] = o.col[1];
+        col[2] = o.col[2];
+    } else {
+        field_eval(GlobalLoad{v.bricks + (size_t)sbi * kBrickVox}, base, f[0], f[1], f[2], fld);
+        scale_field(fld, is);
+        sample_optics(fld, vval, dir, tp, tf, inv_gmax, alpha, col);
+    }
+    return true;
+}
+
 // Front-to-back march of one ray (Eqs. 4-6) over the bricked volume in HBM/L2.
 // Shared by the single-view and batched kernels.
 // Empty space: a sample whose cell is empty under the transfer function has opacity
@@ -53,11 +96,6 @@ __device__ __forceinline__ void add_counters(vr_counters* ctr, unsigned rays, un
 // kCount: the launch wants sample counters. Evaluated samples are defined by the
 // skip bricks (samples outside bricks classified empty), so this variant walks brick by
 // brick and sample by sample instead of leaping; the image is the same.
-// kHessianFirst: the derived path issues the Hessian loads before the table lookup,
-// so that they overlap it, or only after its zero-opacity test; the arithmetic, and
-// so the image, is the same. Every kernel now takes the first order (the batched
-// kernel measured 3 % faster with it once the packed arithmetic and incremental
-// positions were in; 1.4 % slower before).
 // With kState it also returns the ray's last sample index (kstop) and the
 // transmittance in front of that sample (t_last), which the adjoint sweep starts from.
 // kBS: log2 of the skip-brick edge in cells, fixed at compile time (2, 3, 4), or 0 to
@@ -66,7 +104,7 @@ __device__ __forceinline__ void add_counters(vr_counters* ctr, unsigned rays, un
 // slower).
 // Called by whole warps; a lane without a ray passes r.ns = 0.
 constexpr unsigned kRayEnded = 0x7fffffffu;  // above any advance
-template <bool kDerived, bool kState, bool kCount, int kBS, bool kParity = false, bool kHessianFirst = true>
+template <bool kDerived, bool kState, bool kCount, int kBS>
 __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
                                              const RayDev& r, int skip, float inv_gmax, const float is[3],
                                              float4& out, unsigned& dense, unsigned& evald, unsigned& shaded,
@@ -78,7 +116,7 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
     float T1 = 1.f;      // when early termination is off) and the transmittance in front of it
     int k = 0;
     unsigned ne = 0, nsh = 0, nip = 0;
-    const int bs = kBS ? kBS : v.bs, B = 1 << bs, E = B + 1;
+    const int bs = kBS ? kBS : v.bs;
     // the position of sample k, u0 + k du, carried by exact integer additions
     long long U[3] = {r.u0[0], r.u0[1], r.u0[2]};
     auto step = [&]() {
@@ -109,7 +147,7 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
                     const int bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
                     if (__ldg(v.empty + brick_index(v, bc))) {
                         out = true;
-                        adv = (unsigned)(brick_exit_k_at(r, U, bc, B, k, ns) - k);
+                        adv = (unsigned)(brick_exit_k_at(r, U, bc, 1 << bs, k, ns) - k);
                     }
                 }
                 if (!out && v.skipf) {
@@ -133,45 +171,11 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
             continue;
         }
         if (kCount) ++nip;
-        // the sample's fractions, only for samples that are evaluated
-        float f[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) f[q] = cell_frac_at(U[q], v.n[q]);
-        int base = 0, sbi = 0;
-        if (!kDerived || v.vbricks) sbi = storage_brick(v, i0, base);
-        const float vval =
-            v.vbricks ? value_eval(GlobalLoad{v.vbricks + (size_t)sbi * kBrickVox}, base, f[0], f[1], f[2]) : 0.0f;
-        float fld[10], alpha, col[3];
-        if (kDerived) {
-            // derived brick of the cell, and the cell's place in it
-            const int bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
-            const float4* dbrick = reinterpret_cast<const float4*>(
-                v.dbricks + (size_t)(unsigned)brick_index(v, bc) * (unsigned)(kBS ? der_brick_floats(kBS) : v.der_stride));
-            const int lx = i0[0] & (B - 1), ly = i0[1] & (B - 1), lz = i0[2] & (B - 1);
-            // I and the gradient (one 16-byte load per corner) and the Hessian (two), then
-            // the transfer function: a zero opacity entry makes alpha exactly 0 whatever
-            // the Hessian, and the sample adds nothing (bit-neutral). The Hessian loads are
-            // issued before that test so that they overlap the table lookup (measured:
-            // equal at 1080p, 2 % faster on the 8-view workload than loading them after it)
-            derived_channels<kParity, 0, 4>(dbrick, E, lx, ly, lz, f[0], f[1], f[2], fld);
-            if (kHessianFirst) load_hessian<kParity>(tp, dbrick, E, lx, ly, lz, f, fld);
-            SampleOptics o;
-            optics_tf(fld, vval, tp, tf, inv_gmax, o);
-            if (o.c.w == 0.0f) {
-                if (kCount) ++ne;
-                step();
-                continue;
-            }
-            if (!kHessianFirst) load_hessian<kParity>(tp, dbrick, E, lx, ly, lz, f, fld);
-            optics_rest(fld, r.dir, tp, o);
-            alpha = o.alpha;
-            col[0] = o.col[0];
-            col[1] = o.col[1];
-            col[2] = o.col[2];
-        } else {
-            field_eval(GlobalLoad{v.bricks + (size_t)sbi * kBrickVox}, base, f[0], f[1], f[2], fld);
-            scale_field(fld, is);
-            sample_optics(fld, vval, r.dir, tp, tf, inv_gmax, alpha, col);
+        float alpha, col[3];
+        if (!eval_sample<kDerived, kBS>(v, tp, tf, U, i0, r.dir, inv_gmax, is, alpha, col)) {
+            if (kCount) ++ne;
+            step();
+            continue;
         }
         if (kCount) ++nsh;
         const float wgt = (1.0f - A) * alpha;  // Eqs. 5-6
@@ -203,6 +207,84 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
         const int kl = (int)dense - 1;
         *klast_out = k1 >= 0 ? k1 : kl;
         *t_last = k1 >= 0 ? T1 : ((klast == kl) ? 1.0f - A_prev : 1.0f - A);  // samples after klast: alpha 0
+    }
+}
+
+// The same march with G lanes per ray (G a power of two up to 32, the lanes of a ray
+// consecutive): lane g evaluates sample kb + g, then the G samples are composited in
+// order, every lane of the ray repeating the one sequence of operations of
+// march_gather on the values it gets by shuffle -- the image is the same bit for bit.
+// For launches with too few rays to fill the chip the time is the serial chain of one
+// ray, and this shortens it by almost G (64^3 at 128x128: 90 -> 29 us at G = 8); a
+// filled chip gains nothing and pays the shuffles (4 per sample slot).
+template <bool kDerived, bool kState, int G>
+__device__ __forceinline__ void march_lanes(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
+                                            const RayDev& r, int skip, float inv_gmax, const float is[3],
+                                            float4& out, int* klast_out, float* t_last) {
+    const int lane = threadIdx.x & 31, g = lane & (G - 1), first = lane & ~(G - 1);
+    float C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f;
+    float A_prev = 0.f, T1 = 1.f;
+    int klast = -1, k1 = -1, kb = 0, ns = r.ns;
+    long long U[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) U[q] = r.u0[q] + (long long)g * r.du[q];
+    while (true) {
+        int i0[3] = {0, 0, 0};
+        unsigned adv = kRayEnded;
+        if (kb + g < ns) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) i0[q] = cell_index_at(U[q], v.n[q]);
+            adv = 0u;
+            if (!VR_CHECK(tp.status, (unsigned)i0[0] <= (unsigned)(v.n[0] - 2) &&
+                                         (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
+                                         (unsigned)i0[2] <= (unsigned)(v.n[2] - 2)))
+                adv = 1u;
+            else if (skip && v.skipf)
+                adv = __ldg(v.skipf + skip_index(i0[0], i0[1], i0[2], v.skip_cx, v.skip_by));
+        }
+        const unsigned m = __reduce_min_sync(0xffffffffu, adv);
+        int next = G;  // samples to move on
+        if (m) {
+            if (m == kRayEnded) break;
+            // every sample up to kb + G - 1 is empty, and from the last of them a leap follows
+            next = G - 1 + (int)((float)(m - 1u) * tp.leap_per_cell) + 1;
+        } else {
+            float alpha = 0.0f, col[3] = {0.f, 0.f, 0.f};
+            bool shaded = false;
+            if (adv == 0u) shaded = eval_sample<kDerived, 0>(v, tp, tf, U, i0, r.dir, inv_gmax, is, alpha, col);
+            const unsigned live = __ballot_sync(0xffffffffu, shaded);
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+                const int src = first + h;
+                const float a = __shfl_sync(0xffffffffu, alpha, src);
+                const float c0 = __shfl_sync(0xffffffffu, col[0], src), c1 = __shfl_sync(0xffffffffu, col[1], src),
+                            c2 = __shfl_sync(0xffffffffu, col[2], src);
+                if (((live >> src) & 1u) && kb + h < ns) {
+                    const float wgt = (1.0f - A) * a;  // Eqs. 5-6
+                    fma2v(c0, c1, wgt, wgt, C0, C1);
+                    C2 = fmaf(c2, wgt, C2);
+                    if (kState) {
+                        A_prev = A;
+                        klast = kb + h;
+                    }
+                    A += wgt;
+                    if (kState && k1 < 0 && A >= 1.0f) {
+                        k1 = kb + h;
+                        T1 = 1.0f - A_prev;
+                    }
+                    if (A >= tp.et_threshold) ns = kb + h + 1;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) U[q] += (long long)next * r.du[q];
+        kb += next;
+    }
+    out = make_float4(C0, C1, C2, A);
+    if (kState) {
+        const int kl = ns - 1;
+        *klast_out = k1 >= 0 ? k1 : kl;
+        *t_last = k1 >= 0 ? T1 : ((klast == kl) ? 1.0f - A_prev : 1.0f - A);
     }
 }
 

@@ -57,6 +57,48 @@ __global__ void __launch_bounds__(kState ? 128 : 256, kDerived ? (kState ? 7 : 4
     if (kCount && L.counters) add_counters(L.counters, hit ? 1u : 0u, dense, evald, 0u, shaded, interp);
 }
 
+// Several lanes per ray, for launches that would leave the chip idle (march_lanes): a
+// warp covers pw x ph rays of G lanes, a CTA four warps side by side. The fewer the rays,
+// the more registers pay (more loads in flight per lane): 128 at 8 and 16 lanes (128^2 of
+// the 181x217x181 head 142 -> 127 us against 80), 80 at 2 and 4 (256^2 121 -> 113 us
+// against 128); 64 were slower everywhere the chip is not full. The skip-brick size stays
+// a run-time value here: at latency-bound sizes its index arithmetic is hidden.
+template <bool kDerived, bool kState, int G>
+__global__ void __launch_bounds__(128, kDerived && G < 8 ? 6 : 4) k_render_lanes(const __grid_constant__ RenderLaunch L) {
+    const int w = threadIdx.x >> 5;
+    const int ray = (threadIdx.x & 31) / G, pw = L.packet_w;
+    const int i = (blockIdx.x * 4 + w) * pw + (ray & (pw - 1));
+    const int j = blockIdx.y * L.packet_h + ray / pw;
+    const int cam = blockIdx.z;
+    const bool inside = i < L.W && j < L.H;
+    const VolumeDev& v = L.vol;
+    const float gmax = __ldg(&v.vc->gmax);
+    const float inv_gmax = gmax > 0.0f ? 1.0f / gmax : 0.0f;
+    const float is[3] = {1.0f / v.s[0], 1.0f / v.s[1], 1.0f / v.s[2]};
+    RayDev r;
+    if (!(inside && setup_ray(L.cams[cam], L.rc, i, j, v.n, v.s, r))) r.ns = 0;
+    float4 px;
+    int kl = -1;
+    float tl = 1.0f;
+    march_lanes<kDerived, kState, G>(v, L.tp, reinterpret_cast<const float4*>(L.tf), r, L.skip, inv_gmax, is, px, &kl,
+                                     &tl);
+    if (inside && (threadIdx.x & (G - 1)) == 0) {
+        const long long pix = ((long long)(L.cam_offset + cam) * L.H + j) * L.W + i;
+        reinterpret_cast<float4*>(L.out)[pix] = px;
+        if (kState) L.ray_state[pix] = make_float2(__int_as_float(kl), tl);
+    }
+}
+
+template <bool kDerived, bool kState>
+void launch_lanes(const RenderLaunch& L, dim3 grid, cudaStream_t st) {
+    switch (L.lanes) {
+        case 2: k_render_lanes<kDerived, kState, 2><<<grid, 128, 0, st>>>(L); break;
+        case 4: k_render_lanes<kDerived, kState, 4><<<grid, 128, 0, st>>>(L); break;
+        case 8: k_render_lanes<kDerived, kState, 8><<<grid, 128, 0, st>>>(L); break;
+        default: k_render_lanes<kDerived, kState, 16><<<grid, 128, 0, st>>>(L); break;
+    }
+}
+
 template <bool kDerived, bool kState, int kBS>
 void launch_gather_count(const RenderLaunch& L, dim3 grid, int threads, cudaStream_t st) {
     if (L.counters || L.ray_samples)
@@ -83,8 +125,33 @@ void launch_gather_bs(const RenderLaunch& L, dim3 grid, int threads, cudaStream_
     }
 }
 
+// Lanes per ray of a launch with that many rays. One lane per ray fills the chip at
+// 152 SMs x 32 warps x 32 = 156 k rays; below that the time is one ray's serial chain.
+// Measured us at 1 / 2 / 4 / 8 / 16 lanes (128^3 head; 181x217x181 head, 2D table):
+//   64 x 64     226 / 100 /  59 /  37 /  29
+//   128 x 128   203 /  96 /  64 /  49 /  59      990 / 326 / 186 / 127 / 141
+//   256 x 256   180 / 121 / 113 / 129 / 170      678 / 367 / 316 / 301 / 333
+//   400 x 300                                    677 / 414 / 394 / 388 / 449
+//   384 x 384   201 / 192 / 208 / 266 / 369
+//   512 x 512   272 / 294 / 342 / 459 / 649      728 / 700 / 780 / 966 / 1207
+int render_lanes(long long rays) {
+    return rays <= 6000 ? 16 : rays <= 28000 ? 8 : rays <= 100000 ? 4 : rays <= 200000 ? 2 : 1;
+}
+
 cudaError_t launch_render_gather(const RenderLaunch& L0, int warps, cudaStream_t st) {
     RenderLaunch L = L0;
+    L.lanes = render_lanes((long long)L.W * L.H * L.n_cams);
+    if (L.lanes > 1 && !L.counters && !L.ray_samples && (!L.skip || L.vol.skipf)) {
+        const int rays = 32 / L.lanes;  // per warp: 16, 8, 4, 2
+        L.packet_w = rays >= 8 ? 4 : (rays >= 4 ? 2 : 1);
+        L.packet_h = rays / L.packet_w;
+        dim3 grid((L.W + 4 * L.packet_w - 1) / (4 * L.packet_w), (L.H + L.packet_h - 1) / L.packet_h, L.n_cams);
+        if (L.vol.dbricks)
+            L.ray_state ? launch_lanes<true, true>(L, grid, st) : launch_lanes<true, false>(L, grid, st);
+        else
+            L.ray_state ? launch_lanes<false, true>(L, grid, st) : launch_lanes<false, false>(L, grid, st);
+        return cudaGetLastError();
+    }
     // the state-recording kernels are built for CTAs of at most 4 warps (72 registers,
     // 7 CTAs per SM); the image and the state do not depend on the CTA shape
     if (L.ray_state && warps > 4) warps = 4;

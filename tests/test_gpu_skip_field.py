@@ -107,3 +107,37 @@ def test_leaps_are_neutral(torch, dims, spacing, step, width, blobs, derived):
         every[..., 3] = 0.01
         ctx.set_tissue_params(vid, every, grad_mod=0, step_vox=step)
         assert torch.equal(ctx.render(vid, cams, W, H), ctx.render(vid, cams, W, H, skip_empty=False))
+
+
+# images on both sides of every line between 16, 8, 4, 2 and 1 lanes per ray
+SIZES = [(16, 8), (61, 67), (100, 61), (150, 160), (190, 149), (300, 301), (330, 307), (420, 430), (470, 460)]
+
+
+@pytest.mark.parametrize("W,H", SIZES)
+@pytest.mark.parametrize("derived", [True, False])
+def test_lanes_per_ray_are_neutral(torch, W, H, derived):
+    """The image and the ray state of a small launch (several lanes per ray) equal those
+    of the one-lane kernel, which a render with counters always takes, bit for bit."""
+    import paper_2605_19737_gb300 as pkg
+    dims, sp = (61, 50, 43), (1.0, 1.0, 1.2)
+    cams = camera_array([orbit_camera(dims, sp, 40.0, 25.0, width=W, height=H)])
+    rng = np.random.default_rng(W)
+    vol = rng.random(dims[::-1], dtype=np.float32)
+    tf = _table(256)
+    with pkg.Context(0) as ctx:
+        if not derived:
+            ctx.set_derived_budget(0)
+        vid = ctx.load_volume(vol, sp)
+        ctx.precompute_morphology(vid, (1.0,))
+        for mode, et in ((0, 0.99), (0, 2.0), (2, 0.8)):
+            table = np.repeat(tf, 4, 0) if mode else tf
+            ctx.set_tissue_params(vid, table, tf_mode=mode, shading=1, grad_mod=0, gamma=0.4, kappa_ref=0.05,
+                                  et_threshold=et, opacity_scale=30.0 if et > 1 else 1.0)
+            st = [torch.zeros((1, H, W, 2), device="cuda") for _ in range(2)]
+            img = ctx.render(vid, cams, W, H, ray_state=st[0])
+            one = ctx.render(vid, cams, W, H, ray_state=st[1], counters=pkg.new_counters(0))
+            plain = ctx.render(vid, cams, W, H, skip_empty=False)
+            ctx.synchronize()
+            assert float(one[..., 3].max()) > 0.5
+            assert torch.equal(img, one) and torch.equal(plain, one)
+            assert torch.equal(st[0].view(torch.int32), st[1].view(torch.int32))
