@@ -258,18 +258,19 @@ vr_status rebuild_bricks(vr_ctx* ctx, Volume* v) {
     return VR_OK;
 }
 
-// The classification scratch: tf_w + 1 prefix counts, then tf_w column limits.
-int* column_limits(const Volume* v) { return v->d_prefix + v->tp.tf_w + 1; }
-
 // Brick skip flags and (once the morphology is precomputed) the per-cell skip field
-// under the volume's current transfer function.
+// under the volume's current transfer function. Scratch: tf_w + 1 prefix counts, then
+// tf_w column limits.
 vr_status classify_volume(vr_ctx* ctx, Volume* v) {
-    CK(launch_classify(v->d_grid, v->nbricks, v->d_tf, v->tp.tf_w, v->tp.tf_h, v->d_empty, v->d_prefix,
-                       column_limits(v), ctx->stream),
-       "classify");
+    int* limits = v->d_prefix + v->tp.tf_w + 1;
     if (v->d_skip)
-        CK(launch_skip_field(v->d_cellq, v->n, column_limits(v), v->tp.tf_w, skip_store(v->d_skip, v->n), ctx->stream),
-           "skip field");
+        CK(launch_skip_field(v->d_cellq, v->n, v->d_grid, v->nbricks, v->d_tf, v->tp.tf_w, v->tp.tf_h, v->d_prefix,
+                             limits, v->d_empty, skip_store(v->d_skip, v->n), ctx->stream),
+           "classify bricks and cells");
+    else
+        CK(launch_classify(v->d_grid, v->nbricks, v->d_tf, v->tp.tf_w, v->tp.tf_h, v->d_empty, v->d_prefix,
+                           ctx->stream),
+           "classify");
     return VR_OK;
 }
 

@@ -268,14 +268,15 @@ cudaError_t launch_make_derived(const float* norm, const int n[3], const int nb[
                                 float* dbricks, cudaStream_t st);
 cudaError_t launch_gmax(const float* norm, const int n[3], const float s[3], VolConst* vc, cudaStream_t st);
 cudaError_t launch_classify(const uint16_t* grid, long long nbricks, const float* tf, int tf_w, int tf_h,
-                            uint8_t* empty, int* prefix_scratch /* tf_w + 1 ints */,
-                            int* limit /* nullable, tf_w: see k_tf_alpha_prefix */, cudaStream_t st);
+                            uint8_t* empty, int* prefix_scratch /* tf_w + 1 ints */, cudaStream_t st);
 // Per interpolation cell the quantised (min, max) of its 8 corner voxels, low and high
 // 16 bits: [nz - 1][ny - 1][cellq_pitch(nx)].
 cudaError_t launch_cell_minmax(const float* norm, const int n[3], uint32_t* cellq, cudaStream_t st);
-// The skip field under the transfer function whose column limits are `limit`.
-cudaError_t launch_skip_field(const uint32_t* cellq, const int n[3], const int* limit, int tf_w, const SkipStore& s,
-                              cudaStream_t st);
+// The skip field, and the brick flags of launch_classify, under a transfer function
+// (scratch: tf_w + 1 and tf_w ints).
+cudaError_t launch_skip_field(const uint32_t* cellq, const int n[3], const uint16_t* grid, long long nbricks,
+                              const float* tf, int tf_w, int tf_h, int* prefix_scratch, int* limit_scratch,
+                              uint8_t* empty, const SkipStore& s, cudaStream_t st);
 
 // Multi-scale vesselness of `norm` into V (both nvox floats); tmp_a and tmp_b are
 // nvox floats of scratch each, smax receives each scale's max Hessian norm.

@@ -262,6 +262,11 @@ __global__ void __launch_bounds__(256) k_gmax(const float* __restrict__ I, int n
     }
 }
 
+// Largest upper code of a range that stays below the first opaque column f (w: none).
+__device__ __forceinline__ int column_limit(int f, int w) {
+    return f >= w ? 65535 : (f < 2 ? -1 : (f - 2) * 65535 / (w - 1));
+}
+
 // For every intensity column j of the transfer function: 1 if any row has a
 // non-zero opacity; then an exclusive prefix count, so that a brick's column
 // range can be tested in O(1), and (when `limit` is wanted) per lower column j the
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(1024) k_tf_alpha_prefix(const float* __restric
 #pragma unroll
         for (int q = 3; q >= 0; --q) {
             if (c[q]) nx = j0 + q;
-            if (j0 + q < w) limit[j0 + q] = nx >= w ? 65535 : (nx < 2 ? -1 : (nx - 2) * 65535 / (w - 1));
+            if (j0 + q < w) limit[j0 + q] = column_limit(nx, w);
         }
     }
 }
@@ -417,11 +422,67 @@ __global__ void __launch_bounds__(256) k_cell_minmax(const float* __restrict__ n
 // The rule is one division and one comparison with the lower column's limit from shared
 // memory (qlo (w - 1) < 2^29: 32-bit arithmetic); two lookups of a prefix table in global
 // memory bound this kernel by L1 wavefronts (181x217x181: 20.6 -> 15.9 us, the 30 MB of codes read from HBM).
+// The same launch classifies the skip bricks (grid layers past the cells').
+// A 1D table's limits are computed by every CTA for itself (one scan of w columns), which
+// saves the launch that reduces a 2D table's rows first.
+__device__ __forceinline__ int lower_column(unsigned ql, int w) {
+    return max((int)(ql * (unsigned)(w - 1) / 65535u) - 1, 0);
+}
+
+// lim[j], j < w: from `limit`, or from the columns of the 1D table `tf1` (w <= 1024).
+__device__ __forceinline__ void load_limits(const int* __restrict__ limit, const float* __restrict__ tf1, int w,
+                                            int* lim) {
+    if (!tf1) {
+        for (int j = threadIdx.x; j < w; j += 256) lim[j] = __ldg(limit + j);
+        __syncthreads();
+        return;
+    }
+    __shared__ int first[8];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, j0 = 4 * threadIdx.x;
+    bool c[4];
+    int f = w;
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+        c[q] = j0 + q < w && __ldg(tf1 + 4 * (j0 + q) + 3) != 0.0f;
+        if (c[q]) f = j0 + q;
+    }
+    int suf = f;  // suffix minimum of the first opaque columns
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int m = __shfl_down_sync(0xffffffffu, suf, o);
+        if (lane + o < 32) suf = min(suf, m);
+    }
+    if (lane == 0) first[wid] = suf;
+    __syncthreads();
+    int nx = __shfl_down_sync(0xffffffffu, suf, 1);
+    if (lane == 31) nx = w;
+    for (int q = wid + 1; q < 8; ++q) nx = min(nx, first[q]);
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+        if (c[q]) nx = j0 + q;
+        if (j0 + q < w) lim[j0 + q] = column_limit(nx, w);
+    }
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(256) k_cell_bits(const uint32_t* __restrict__ cellq, SkipDims d, int pitch,
-                                                   const int* __restrict__ limit, int w,
-                                                   uint32_t* __restrict__ cell_bits, uint8_t* __restrict__ block_bits) {
+                                                   const int* __restrict__ limit, const float* __restrict__ tf1, int w,
+                                                   uint32_t* __restrict__ cell_bits, uint8_t* __restrict__ block_bits,
+                                                   int cell_layers, const uint16_t* __restrict__ grid,
+                                                   long long nbricks, uint8_t* __restrict__ empty) {
     __shared__ uint32_t rows[64];  // [z 0..15][y 0..3]
     __shared__ int lim[4096];
+    if ((int)blockIdx.z >= cell_layers) {
+        load_limits(limit, tf1, w, lim);
+        const long long stride = (long long)(gridDim.z - cell_layers) * gridDim.y * gridDim.x * 256;
+        for (long long b = (((long long)(blockIdx.z - cell_layers) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) *
+                               256 + threadIdx.x;
+             b < nbricks; b += stride) {
+            const unsigned q = __ldg(reinterpret_cast<const unsigned*>(grid) + b);
+            empty[b] = (uint8_t)((int)(q >> 16) <= lim[lower_column(q & 0xffffu, w)]);
+        }
+        return;
+    }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int x = blockIdx.x * 32 + lane, y0 = blockIdx.y * 4, z0 = blockIdx.z * 16 + wid * 2;
     const long long r0 = (long long)z0 * d.cy + y0;  // the warp's rows: (z0, z0 + 1) x (y0 .. y0 + 3)
@@ -430,11 +491,10 @@ __global__ void __launch_bounds__(256) k_cell_bits(const uint32_t* __restrict__ 
 #pragma unroll
     for (int r = 0; r < 8; ++r)
         q[r] = (r & 3) < ny && (r >> 2) < nz ? __ldg(cellq + (r0 + (r >> 2) * d.cy + (r & 3)) * pitch + x) : 65535u;
-    for (int j = threadIdx.x; j < w; j += blockDim.x) lim[j] = __ldg(limit + j);
-    __syncthreads();
+    load_limits(limit, tf1, w, lim);
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-        const int jl = max((int)((q[r] & 0xffffu) * (unsigned)(w - 1) / 65535u) - 1, 0);
+        const int jl = lower_column(q[r] & 0xffffu, w);
         // cells past the volume hold the code pair (65535, 0), the only one with qlo > qhi
         const unsigned bits = __ballot_sync(0xffffffffu, (int)(q[r] >> 16) <= lim[jl] || q[r] == 65535u);
         if (lane == 0) {
@@ -572,14 +632,30 @@ __device__ __forceinline__ unsigned plane_count(const uint4& p, int x) {
 // own (up to 5) and what its block's promises: with the block at distance c, the
 // 4 (c - 1) layers of cells around the block are empty, so the cell is at 4 c - 3 at
 // least (up to 33).
+// kFused: the CTA erodes the blocks around its tile itself instead of reading
+// k_block_dist's result: three times the erosions, so only where the launch is too small
+// to fill the chip and the saved launch is worth more (64^3: 5 + 6.2 -> 9.4 us).
+template <bool kFused>
 __global__ void __launch_bounds__(256) k_skip_field(const uint32_t* __restrict__ bits, SkipDims d,
+                                                    const uint32_t* __restrict__ block_bits,
                                                     const uint4* __restrict__ block_dist,
                                                     uint8_t* __restrict__ field) {
     constexpr int kE = kCellErosions, T = 32 - 2 * kE, TB = T / 4;
     __shared__ EdgeRows sm;
-    __shared__ uint4 plane[T][T];  // [z][y] of the tile
+    __shared__ uint4 plane[T][T];       // [z][y] of the tile
+    __shared__ uint4 bplane[TB][TB];    // kFused: of its blocks
     const int xl = threadIdx.x & 31, x = blockIdx.x * 32 + xl;
     CountPlanes p;
+    if (kFused) {
+        constexpr int kB = kBlockErosions;
+        erode_tile<kB>(block_bits, d.bwx, d.by, d.bz, blockIdx.x >> 2, blockIdx.y * TB, blockIdx.z * TB, sm, p);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int z = (threadIdx.x >> 5) * 4 + r - kB, y = xl - kB;
+            if (z >= 0 && z < TB && y >= 0 && y < TB) bplane[z][y] = make_uint4(p.c0[r], p.c1[r], p.c2[r], p.c3[r]);
+        }
+        __syncthreads();  // the edge rows are used again
+    }
     erode_tile<kE>(bits, d.wx, d.cy, d.cz, blockIdx.x, blockIdx.y * T, blockIdx.z * T, sm, p);
     if (tile_row<kE>()) {
 #pragma unroll
@@ -592,7 +668,7 @@ __global__ void __launch_bounds__(256) k_skip_field(const uint32_t* __restrict__
     for (int c = threadIdx.x >> 5; c < TB * TB; c += 8) {
         const int yb = c % TB, zb = c / TB, by = blockIdx.y * TB + yb, bz = blockIdx.z * TB + zb;
         if (by >= d.by || bz >= d.bz) continue;
-        const uint4 far4 = __ldg(block_dist + ((long long)bz * d.by + by) * d.bwx + (x >> 7));
+        const uint4 far4 = kFused ? bplane[zb][yb] : __ldg(block_dist + ((long long)bz * d.by + by) * d.bwx + (x >> 7));
         const int far = 4 * (int)plane_count(far4, (x >> 2) & 31) - 3;
         uint32_t o[4];
 #pragma unroll
@@ -617,17 +693,27 @@ cudaError_t launch_cell_minmax(const float* norm, const int n[3], uint32_t* cell
     return cudaGetLastError();
 }
 
-cudaError_t launch_skip_field(const uint32_t* cellq, const int n[3], const int* limit, int tf_w, const SkipStore& s,
-                              cudaStream_t st) {
+cudaError_t launch_skip_field(const uint32_t* cellq, const int n[3], const uint16_t* grid, long long nbricks,
+                              const float* tf, int tf_w, int tf_h, int* prefix_scratch, int* limit_scratch,
+                              uint8_t* empty, const SkipStore& s, cudaStream_t st) {
     const SkipDims d = skip_dims(n);
     constexpr int TC = 32 - 2 * kCellErosions, TB = 32 - 2 * kBlockErosions;
-    k_cell_bits<<<dim3(d.wx, d.by, (d.cz + 15) / 16), 256, 0, st>>>(cellq, d, cellq_pitch(n[0]), limit, tf_w,
-                                                                    s.cell_bits,
-                                                                    reinterpret_cast<uint8_t*>(s.block_bits));
-    k_block_dist<<<dim3(d.bwx, (d.by + TB - 1) / TB, (d.bz + TB - 1) / TB), 256, 0, st>>>(s.block_bits, d,
-                                                                                        s.block_dist);
-    k_skip_field<<<dim3(d.wx, (d.cy + TC - 1) / TC, (d.cz + TC - 1) / TC), 256, 0, st>>>(s.cell_bits, d, s.block_dist,
-                                                                                       s.field);
+    const float* tf1 = tf_h == 1 && tf_w <= 1024 ? tf : nullptr;
+    if (!tf1) k_tf_alpha_prefix<<<1, 1024, 0, st>>>(tf, tf_w, tf_h, prefix_scratch, limit_scratch);
+    const int layers = (d.cz + 15) / 16;
+    const long long per_layer = (long long)d.wx * d.by * 256;
+    const long long more = (nbricks + per_layer - 1) / per_layer;
+    k_cell_bits<<<dim3(d.wx, d.by, layers + (unsigned)(more < 4 ? more : 4)), 256, 0, st>>>(
+        cellq, d, cellq_pitch(n[0]), limit_scratch, tf1, tf_w, s.cell_bits, reinterpret_cast<uint8_t*>(s.block_bits),
+        layers, grid, nbricks, empty);
+    const dim3 tiles(d.wx, (d.cy + TC - 1) / TC, (d.cz + TC - 1) / TC);
+    if ((long long)tiles.x * tiles.y * tiles.z <= kSMs) {
+        k_skip_field<true><<<tiles, 256, 0, st>>>(s.cell_bits, d, s.block_bits, nullptr, s.field);
+    } else {
+        k_block_dist<<<dim3(d.bwx, (d.by + TB - 1) / TB, (d.bz + TB - 1) / TB), 256, 0, st>>>(s.block_bits, d,
+                                                                                            s.block_dist);
+        k_skip_field<false><<<tiles, 256, 0, st>>>(s.cell_bits, d, nullptr, s.block_dist, s.field);
+    }
     return cudaGetLastError();
 }
 
@@ -693,8 +779,8 @@ cudaError_t launch_gmax(const float* norm, const int n[3], const float s[3], Vol
 }
 
 cudaError_t launch_classify(const uint16_t* grid, long long nbricks, const float* tf, int tf_w, int tf_h,
-                            uint8_t* empty, int* prefix_scratch, int* limit, cudaStream_t st) {
-    k_tf_alpha_prefix<<<1, 1024, 0, st>>>(tf, tf_w, tf_h, prefix_scratch, limit);
+                            uint8_t* empty, int* prefix_scratch, cudaStream_t st) {
+    k_tf_alpha_prefix<<<1, 1024, 0, st>>>(tf, tf_w, tf_h, prefix_scratch, nullptr);
     k_classify<<<(unsigned)((nbricks + 255) / 256), 256, 0, st>>>(grid, nbricks, prefix_scratch, tf_w, empty);
     return cudaGetLastError();
 }
@@ -818,8 +904,7 @@ extern "C" vr_status vr_classify_bricks_noalloc(const unsigned short* d_grid, lo
         prefix = g_static_prefix_ptr[dev];
     }
     const cudaError_t e = launch_classify(reinterpret_cast<const uint16_t*>(d_grid), nbricks, d_tf, tf_w, tf_h,
-                                          reinterpret_cast<uint8_t*>(d_empty), prefix, nullptr,
-                                          (cudaStream_t)cuda_stream);
+                                          reinterpret_cast<uint8_t*>(d_empty), prefix, (cudaStream_t)cuda_stream);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         put_msg(h_msg, msg_len, cudaGetErrorString(e));
