@@ -34,13 +34,14 @@ struct ParamGrad {
 // (Shared-memory tables with scalar atomics measured 1.6x slower on a 1D table:
 // the lanes of a CTA contend for the same few entries.)
 
+// two_d is a template argument: a 1D table's sink has eight accumulators less.
+template <bool two_d>
 struct TfGradSink {
     float* p;       // this copy: [cell key][kTfCellFloats]
-    bool two_d;
     int key = -1;   // the pending cell, -1 = none
     float4 a00, a01, a10, a11;
 
-    __device__ __forceinline__ TfGradSink(float* p_, bool two_d_) : p(p_), two_d(two_d_) {}
+    __device__ __forceinline__ explicit TfGradSink(float* p_) : p(p_) {}
 
     __device__ __forceinline__ void put(int piece, const float4& v) const {
         // any component not +-0: one OR of the bit patterns, the sign bits shifted out
@@ -85,9 +86,10 @@ struct TfGradSink {
 // computed for it. da = dL/dalpha and dc = dL/dcolour come in; the transfer-function
 // and uniform gradients go to dtf and dp; dfield receives dL/d(I, gx, gy, gz, Hxx,
 // Hyy, Hzz, Hxy, Hxz, Hyz) in the same (spacing-scaled) units as the field f.
+template <bool k2D>
 __device__ __forceinline__ void sample_adjoint(const float f[10], const SampleOptics& o, const float dir[3],
                                                const TissueDev& tp, float inv_gmax, float da, const float dc[3],
-                                               TfGradSink& dtf, ParamGrad& dp, float dfield[10]) {
+                                               TfGradSink<k2D>& dtf, ParamGrad& dp, float dfield[10]) {
     const float gx = f[1], gy = f[2], gz = f[3];
     const float gg = o.gg, r = o.r, kappa = o.kappa, hx = o.hx, hy = o.hy, hz = o.hz;
     const float Hgx = o.Hgx, Hgy = o.Hgy, Hgz = o.Hgz, gn = o.gn, y = o.y;
@@ -133,7 +135,7 @@ __device__ __forceinline__ void sample_adjoint(const float f[10], const SampleOp
     const bool in_x = I >= 0.0f && I <= 1.0f;
     float dI = 0.f;
     const float T00a[4] = {T00.x, T00.y, T00.z, T00.w}, T01a[4] = {T01.x, T01.y, T01.z, T01.w};
-    if (h == 1) {
+    if (!k2D) {
         dtf.add_cell(j, 1.0f - t, t, 0.0f, 0.0f, dr);
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch)

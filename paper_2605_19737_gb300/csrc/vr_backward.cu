@@ -37,8 +37,15 @@ struct GLoad {
     __device__ __forceinline__ float operator()(int o) const { return __ldg(p + o); }
 };
 
-__device__ __forceinline__ long long bidx(const VolumeDev& v, const int b[3]) {
-    return ((long long)b[2] * v.nb[1] + b[1]) * v.nb[0] + b[0];
+// Skip-brick id in 32-bit arithmetic: dims <= 2048 give at most 512^3 = 2^27 bricks.
+__device__ __forceinline__ int bidx(const VolumeDev& v, const int b[3]) {
+    return (b[2] * v.nb[1] + b[1]) * v.nb[0] + b[0];
+}
+
+// Derived brick `bi` (32-bit operands: one widening multiply-add).
+template <int kBS>
+__device__ __forceinline__ const float4* derived_brick(const VolumeDev& v, int bi) {
+    return reinterpret_cast<const float4*>(v.dbricks + (size_t)(unsigned)bi * (unsigned)der_brick_floats(kBS));
 }
 
 // The sample field, from the derived bricks (voxel-wise derivatives) or by the
@@ -49,11 +56,11 @@ __device__ __forceinline__ long long bidx(const VolumeDev& v, const int b[3]) {
 // bi: the skip brick of the sample's cell (derived bricks); sbi, base: its storage
 // brick and the stencil origin in it (intensity bricks).
 template <bool kDerived, bool kHessian, int kBS>
-__device__ __forceinline__ void eval_field(const VolumeDev& v, const TissueDev& tp, long long bi, long long sbi,
+__device__ __forceinline__ void eval_field(const VolumeDev& v, const TissueDev& tp, int bi, long long sbi,
                                            const int i0[3], int base, const float f[3], const float is[3],
                                            float fld[10]) {
     if (kDerived) {
-        const float4* brick = reinterpret_cast<const float4*>(v.dbricks + bi * der_brick_floats(kBS));
+        const float4* brick = derived_brick<kBS>(v, bi);
         const int m = (1 << kBS) - 1, E = m + 2;
         derived_channels<true, 0, 4>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
         if (kHessian)
@@ -262,19 +269,29 @@ __global__ void __launch_bounds__(256) k_channels_to_voxels(const float* __restr
 }
 
 // 4 resident CTAs per SM (<= 128 registers): measured 1 ms faster at 1080p than
-// the 3 that the unbounded register count allows.
+// the 3 that the unbounded register count allows. The sweep re-evaluates every sample
+// and is bound by instructions and registers (16 warps at 55-60 % issue), so what a
+// launch does not need is compiled out:
 // Derived bricks without a curvature term (gamma = 0): with kLazyHessian a sample
 // reads the Hessian only when its opacity entry is non-zero (for dL/dgamma); with
 // kNoHessian, when no uniform gradient is wanted, never.
+// kTfOnly: neither uniform nor voxel gradients are wanted (a transfer-function fit): no
+// field adjoint, no scatter. k2D: whether the table has two dimensions; a 1D table's
+// sink and lookup keep 16 registers less, and the kernel for a 1D table alone fits five
+// CTAs (96 registers). Forward + backward, without / with both: fit step of 8 views of
+// the 128^3 head at 512^2 9.53 -> 6.86 ms (1.9 of it the forward), 4 such views with
+// every gradient 6.71 -> 5.91, 1080p of the 181x217x181 head (2D) 11.63 -> 11.43, its
+// table alone at 2 x 700x600 6.48 -> 5.43. (6 CTAs for the 1D table alone: 2 % slower; 5
+// for 1D with every gradient: 5 % slower; 5 for the 2D table alone: 2 % slower.)
 // kBS: log2 of the skip-brick edge (2, 3, 4), fixed at compile time.
-template <bool kDerived, bool kLazyHessian, bool kNoHessian, int kBS>
-__global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constant__ BackwardLaunch B) {
+template <bool kDerived, bool kLazyHessian, bool kNoHessian, bool kTfOnly, bool k2D, int kBS>
+__global__ void __launch_bounds__(128, kTfOnly && !k2D ? 5 : 4) k_render_backward(const __grid_constant__ BackwardLaunch B) {
     const RenderLaunch& L = B.r;
     const size_t ncell = (size_t)L.tp.tf_w * L.tp.tf_h * kTfCellFloats;
     // one of n_copies private global copies of the gradient, so that CTAs working on
     // the same hot entries do not serialise on one address
     const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    TfGradSink sink(B.dtf_copies + (size_t)(cta % B.n_copies) * ncell, L.tp.tf_h > 1);
+    TfGradSink<k2D> sink(B.dtf_copies + (size_t)(cta % B.n_copies) * ncell);
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     int di, dj;
     tile_pixel(L.packet_w, __ffs(tile_packets_x(L.packet_w, 4)) - 1, w, l, di, dj);
@@ -322,7 +339,7 @@ __global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constan
                                                (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
                                                (unsigned)i0[2] <= (unsigned)(v.n[2] - 2)))
                     break;
-                const long long bi = bidx(v, bc);
+                const int bi = bidx(v, bc);
                 if (L.skip && __ldg(v.empty + bi)) {
                     k = brick_exit_k(r, bc, 1 << kBS, k, r.ns);
                     continue;
@@ -375,7 +392,7 @@ __global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constan
                                                (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
                                                (unsigned)i0[2] <= (unsigned)(v.n[2] - 2)))
                     continue;
-                const long long bi = bidx(v, bc);
+                const int bi = bidx(v, bc);
                 int base;
                 const long long sbi = storage_brick(v, i0, base);
                 float fld[10];
@@ -386,10 +403,10 @@ __global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constan
                     // I and the gradient, the table lookup, then the Hessian, which without
                     // a curvature term only dL/dgamma needs -- and not at a zero opacity
                     // entry (dL/dw = 0 there, and w = 1 whatever kappa)
-                    const float4* brick = reinterpret_cast<const float4*>(v.dbricks + bi * der_brick_floats(kBS));
+                    const float4* brick = derived_brick<kBS>(v, bi);
                     const int m = (1 << kBS) - 1, E = m + 2;
                     derived_channels<true, 0, 4>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
-                    optics_tf(fld, vval, L.tp, tf, inv_gmax, so);
+                    optics_tf<k2D ? 2 : 1>(fld, vval, L.tp, tf, inv_gmax, so);
                     if (!kNoHessian && so.c.w != 0.0f) {
                         derived_channels<true, 4, 6>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2],
                                                      fld + 4);
@@ -400,7 +417,7 @@ __global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constan
                     optics_rest(fld, r.dir, L.tp, so);
                 } else {
                     eval_field<kDerived, true, kBS>(v, L.tp, bi, sbi, i0, base, f, is, fld);
-                    optics_core(fld, vval, r.dir, L.tp, tf, inv_gmax, so);
+                    optics_core<k2D ? 2 : 1>(fld, vval, r.dir, L.tp, tf, inv_gmax, so);
                 }
                 const float alpha = so.alpha, col[3] = {so.col[0], so.col[1], so.col[2]};
                 // T_k = T_{k+1} / (1 - alpha_k); Tk still holds T_{k+1} here, which a zero
@@ -417,7 +434,7 @@ __global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constan
                     const float dr[4] = {0.f, 0.f, 0.f,
                                          (so.raw >= 0.0f && so.raw <= 1.0f) ? dal * L.tp.opacity_scale * so.mg * so.wk
                                                                             : 0.0f};
-                    if (L.tp.tf_h == 1)
+                    if (!k2D)
                         sink.add_cell(so.j, 1.0f - so.t, so.t, 0.0f, 0.0f, dr);
                     else
                         sink.add_cell(so.k * L.tp.tf_w + so.j, (1.0f - so.q) * (1.0f - so.t), (1.0f - so.q) * so.t,
@@ -429,7 +446,8 @@ __global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constan
                 const float dc[3] = {ta * dC[0], ta * dC[1], ta * dC[2]};
                 float dfs[10];
                 sample_adjoint(fld, so, r.dir, L.tp, inv_gmax, da, dc, sink, dp, dfs);
-                if (kDerived && B.dgrad) {
+                if (kTfOnly) {
+                } else if (kDerived && B.dgrad) {
                     scatter_channels(B.dgrad, v.n, i0, f, dfs, L.packet_w);
                 } else if (B.dvol) {
                     const int x0 = i0[0] - 1, y0 = i0[1] - 1, z0 = i0[2] - 1;
@@ -450,6 +468,7 @@ __global__ void __launch_bounds__(128, 4) k_render_backward(const __grid_constan
             }
     }
     sink.flush();
+    if (kTfOnly) return;
     // uniform gradients: warp sums, one atomic per warp and parameter
     float pv[5] = {dp.gamma, dp.ka, dp.kd, dp.ks, dp.os};
 #pragma unroll
@@ -479,6 +498,7 @@ __device__ __forceinline__ unsigned far_key(const int b[3], const int e[3]) {
     return (dz << 20) | (dy << 10) | dx;
 }
 
+template <bool k2D>
 __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_constant__ BackwardLaunch B) {
     extern __shared__ float smem[];
     const RenderLaunch& L = B.r;
@@ -488,7 +508,7 @@ __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_con
     for (int e = l; e < kBrickVox; e += 32) acc[e] = 0.0f;
     __syncthreads();
     const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    TfGradSink sink(B.dtf_copies + (size_t)(cta % B.n_copies) * ncell, L.tp.tf_h > 1);
+    TfGradSink<k2D> sink(B.dtf_copies + (size_t)(cta % B.n_copies) * ncell);
     const int i = blockIdx.x * 16 + (warp & 1) * 8 + (l & 7);
     const int j = blockIdx.y * 8 + (warp >> 1) * 4 + (l >> 3);
     const int cam = blockIdx.z;
@@ -529,7 +549,7 @@ __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_con
                                            (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
                                            (unsigned)i0[2] <= (unsigned)(v.n[2] - 2)))
                 break;
-            const long long bi = bidx(v, bc);
+            const int bi = bidx(v, bc);
             if (L.skip && __ldg(v.empty + bi)) {
                 k = brick_exit_k(r, bc, kCells, k, r.ns);
                 continue;
@@ -537,9 +557,9 @@ __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_con
             const int base = ((i0[2] - kCells * bc[2]) * kEdge + (i0[1] - kCells * bc[1])) * kEdge +
                              (i0[0] - kCells * bc[0]);
             float fld[10];
-            field_eval(GLoad{v.bricks + bi * kBrickVox}, base, f[0], f[1], f[2], fld);
+            field_eval(GLoad{v.bricks + (long long)bi * kBrickVox}, base, f[0], f[1], f[2], fld);
             scale_field(fld, is);
-            const float vval = v.vbricks ? value_eval(GLoad{v.vbricks + bi * kBrickVox}, base, f[0], f[1], f[2]) : 0.f;
+            const float vval = v.vbricks ? value_eval(GLoad{v.vbricks + (long long)bi * kBrickVox}, base, f[0], f[1], f[2]) : 0.f;
             float alpha, col[3];
             sample_optics(fld, vval, r.dir, L.tp, tf, inv_gmax, alpha, col);
             A_prev = A;
@@ -576,7 +596,7 @@ __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_con
         for (int q = 0; q < 3; ++q) sc[q] = __shfl_sync(0xffffffffu, bc[q], leader);
         int lo_t[3] = {kEdge, kEdge, kEdge}, hi_t[3] = {-1, -1, -1};  // touched local range
         if (live && bc[0] == sc[0] && bc[1] == sc[1] && bc[2] == sc[2]) {
-            const long long bi = bidx(v, sc);
+            const int bi = bidx(v, sc);
             while (true) {
                 const int base = ((i0[2] - kCells * sc[2]) * kEdge + (i0[1] - kCells * sc[1])) * kEdge +
                                  (i0[0] - kCells * sc[0]);
@@ -586,10 +606,10 @@ __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_con
                     break;
                 }
                 float fld[10];
-                field_eval(GLoad{v.bricks + bi * kBrickVox}, base, f[0], f[1], f[2], fld);
+                field_eval(GLoad{v.bricks + (long long)bi * kBrickVox}, base, f[0], f[1], f[2], fld);
                 scale_field(fld, is);
                 const float vval =
-                    v.vbricks ? value_eval(GLoad{v.vbricks + bi * kBrickVox}, base, f[0], f[1], f[2]) : 0.f;
+                    v.vbricks ? value_eval(GLoad{v.vbricks + (long long)bi * kBrickVox}, base, f[0], f[1], f[2]) : 0.f;
                 SampleOptics so;
                 optics_core(fld, vval, r.dir, L.tp, tf, inv_gmax, so);
                 const float alpha = so.alpha, col[3] = {so.col[0], so.col[1], so.col[2]};
@@ -721,18 +741,31 @@ cudaError_t launch_sum_copies(const float* copies, int n_copies, int tf_w, int t
     return cudaGetLastError();
 }
 
-template <int kBS>
+template <bool k2D, int kBS>
 void launch_backward_bs(const BackwardLaunch& B, dim3 grid, cudaStream_t st) {
     const RenderLaunch& L = B.r;
-    if (L.vol.dbricks)
-        if (L.tp.gk == 0.0f && !B.dparams)
-            k_render_backward<true, true, true, kBS><<<grid, 128, 0, st>>>(B);
-        else if (L.tp.gk == 0.0f)
-            k_render_backward<true, true, false, kBS><<<grid, 128, 0, st>>>(B);
-        else
-            k_render_backward<true, false, false, kBS><<<grid, 128, 0, st>>>(B);
+    const bool tf_only = !B.dparams && !B.dvol && !B.dgrad;
+    if (!L.vol.dbricks)
+        k_render_backward<false, false, false, false, k2D, kBS><<<grid, 128, 0, st>>>(B);
+    else if (L.tp.gk == 0.0f && tf_only)
+        k_render_backward<true, true, true, true, k2D, kBS><<<grid, 128, 0, st>>>(B);
+    else if (L.tp.gk == 0.0f && !B.dparams)
+        k_render_backward<true, true, true, false, k2D, kBS><<<grid, 128, 0, st>>>(B);
+    else if (L.tp.gk == 0.0f)
+        k_render_backward<true, true, false, false, k2D, kBS><<<grid, 128, 0, st>>>(B);
+    else if (tf_only)
+        k_render_backward<true, false, false, true, k2D, kBS><<<grid, 128, 0, st>>>(B);
     else
-        k_render_backward<false, false, false, kBS><<<grid, 128, 0, st>>>(B);
+        k_render_backward<true, false, false, false, k2D, kBS><<<grid, 128, 0, st>>>(B);
+}
+
+template <bool k2D>
+void launch_backward_table(const BackwardLaunch& B, dim3 grid, cudaStream_t st) {
+    switch (B.r.vol.bs) {
+        case 2: launch_backward_bs<k2D, 2>(B, grid, st); break;
+        case 4: launch_backward_bs<k2D, 4>(B, grid, st); break;
+        default: launch_backward_bs<k2D, 3>(B, grid, st); break;
+    }
 }
 
 cudaError_t launch_render_backward(const BackwardLaunch& B, bool staged, cudaStream_t st) {
@@ -740,17 +773,16 @@ cudaError_t launch_render_backward(const BackwardLaunch& B, bool staged, cudaStr
     dim3 grid((L.W + 15) / 16, (L.H + 7) / 8, L.n_cams);
     if (staged) {
         const int smem = 4 * kBrickBytes;
-        cudaError_t e = cudaFuncSetAttribute(k_render_backward_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             smem);
+        auto kernel = L.tp.tf_h > 1 ? k_render_backward_staged<true> : k_render_backward_staged<false>;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        k_render_backward_staged<<<grid, 128, smem, st>>>(B);
+        kernel<<<grid, 128, smem, st>>>(B);
         return cudaGetLastError();
     }
-    switch (L.vol.bs) {
-        case 2: launch_backward_bs<2>(B, grid, st); break;
-        case 4: launch_backward_bs<4>(B, grid, st); break;
-        default: launch_backward_bs<3>(B, grid, st); break;
-    }
+    if (L.tp.tf_h > 1)
+        launch_backward_table<true>(B, grid, st);
+    else
+        launch_backward_table<false>(B, grid, st);
     return cudaGetLastError();
 }
 

@@ -388,6 +388,8 @@ struct SampleOptics {
 // First half of a sample's optics, from I and the gradient alone (f[0..3]): |g|,
 // the unit normal, the lookup coordinates and the transfer-function RGBA. Its
 // opacity entry c.w decides whether the sample can be visible at all.
+// kTable: 1 or 2 when the caller knows the table's dimensions, 0 to look at tf_h.
+template <int kTable = 0>
 __device__ __forceinline__ void optics_tf(const float f[4], float vval, const TissueDev& tp,
                                           const float4* __restrict__ tf, float inv_gmax, SampleOptics& o) {
     const float gx = f[1], gy = f[2], gz = f[3];
@@ -409,7 +411,7 @@ __device__ __forceinline__ void optics_tf(const float f[4], float vval, const Ti
     o.j = min((int)xs, w - 2);
     if (!VR_CHECK(tp.status, o.j >= 0)) o.j = 0;
     o.t = xs - (float)o.j;
-    if (h == 1) {
+    if (kTable == 1 || (kTable == 0 && h == 1)) {
         o.k = 0;
         o.q = 0.0f;
         o.T00 = __ldg(tf + o.j);
@@ -472,9 +474,10 @@ __device__ __forceinline__ void optics_rest(const float f[10], const float dir[3
 
 // Opacity (Eq. 4) and colour of one sample from its field (already scaled to
 // mm units) and vesselness value, keeping the intermediate values in `o`.
+template <int kTable = 0>
 __device__ __forceinline__ void optics_core(const float f[10], float vval, const float dir[3], const TissueDev& tp,
                                             const float4* __restrict__ tf, float inv_gmax, SampleOptics& o) {
-    optics_tf(f, vval, tp, tf, inv_gmax, o);
+    optics_tf<kTable>(f, vval, tp, tf, inv_gmax, o);
     optics_rest(f, dir, tp, o);
 }
 
