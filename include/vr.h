@@ -352,7 +352,8 @@ vr_status vr_render(vr_ctx* ctx, int vol_id, const vr_camera* h_cams, int n_cams
  * opts: NULL or as vr_render: skip_empty applies to the forward re-march only,
  * where it is exact; a non-NULL ray_state (written by the vr_render of this image)
  * replaces the re-march: each ray's reverse sweep starts from its recorded last
- * sample and transmittance (per-lane kernels only); kernel VR_KERNEL_STAGED sweeps brick by brick and sums voxel
+ * sample and transmittance (per-lane kernels only; launches of up to 122880 rays then
+ * give each ray several lanes, whatever packet_w says); kernel VR_KERNEL_STAGED sweeps brick by brick and sums voxel
  * gradients in shared memory before global atomics (per-sample stencils), any
  * other value (default) sweeps each lane independently and adds voxel gradients
  * with global atomics, evaluating samples from the derived bricks when they exist

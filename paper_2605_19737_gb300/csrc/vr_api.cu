@@ -65,6 +65,8 @@ struct Batch {
 
 }  // namespace
 
+constexpr int kParamSums = 32;  // words into vr_ctx::d_work (64 words, 8-byte aligned)
+
 struct vr_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -81,7 +83,8 @@ struct vr_ctx {
     size_t tfgrad_cap = 0;
     float* d_dgrad = nullptr;     // per-voxel derived-channel gradients (backward on derived bricks)
     size_t dgrad_cap = 0;
-    unsigned* d_work = nullptr;   // [0]: staged-kernel work counter, [1]: status word
+    unsigned* d_work = nullptr;   // [0]: staged-kernel work counter, [1]: status word, [kParamSums..]:
+                                  // five doubles, the uniform gradients' sums of a backward
     int staged_ctas[2][17] = {};   // resident CTAs per SM by (vesselness, warps per block)
     int batch_ctas[2][17] = {};    // resident batch-kernel CTAs per SM by (all derived, warps per block)
     size_t derived_budget = kDerivedBudgetBytes;  // largest derived-brick store precompute builds
@@ -932,7 +935,8 @@ vr_status vr_render_backward(vr_ctx* ctx, int vol_id, const vr_camera* h_cams, i
         return fail(ctx, VR_ERR_INVALID_ARG, "render_backward: bad kernel choice");
     const size_t ntf = (size_t)v->tp.tf_w * v->tp.tf_h * 4;
     CK(cudaMemsetAsync(d_dtf, 0, sizeof(float) * ntf, ctx->stream), "render_backward: zero dtf");
-    if (d_dparams) CK(cudaMemsetAsync(d_dparams, 0, sizeof(float) * 5, ctx->stream), "render_backward: zero dparams");
+    double* psum = d_dparams ? reinterpret_cast<double*>(ctx->d_work + kParamSums) : nullptr;
+    if (psum) CK(cudaMemsetAsync(psum, 0, sizeof(double) * 5, ctx->stream), "render_backward: zero dparams");
     BackwardLaunch B;
     memset(&B, 0, sizeof B);
     fill_launch(B.r, v, W, H, skip);
@@ -968,7 +972,7 @@ vr_status vr_render_backward(vr_ctx* ctx, int vol_id, const vr_camera* h_cams, i
     }
     B.dl_drgba = d_dl_drgba;
     B.dtf = d_dtf;
-    B.dparams = d_dparams;
+    B.dparams = psum;
     B.dvol = d_dvolume;
     {
         // private copies of the transfer-function gradient (a 16-float record per
@@ -1004,7 +1008,7 @@ vr_status vr_render_backward(vr_ctx* ctx, int vol_id, const vr_camera* h_cams, i
     if (channels)
         CK(launch_channels_to_voxels(ctx->d_dgrad, v->n, v->s, d_dvolume, ctx->stream),
            "render_backward: channel gradients to voxels");
-    CK(launch_sum_copies(ctx->d_tfgrad, B.n_copies, v->tp.tf_w, v->tp.tf_h, d_dtf, ctx->stream),
+    CK(launch_sum_copies(ctx->d_tfgrad, B.n_copies, v->tp.tf_w, v->tp.tf_h, d_dtf, psum, d_dparams, ctx->stream),
        "render_backward: sum gradient copies");
     return VR_OK;
 }

@@ -45,7 +45,8 @@ __device__ __forceinline__ int bidx(const VolumeDev& v, const int b[3]) {
 // Derived brick `bi` (32-bit operands: one widening multiply-add).
 template <int kBS>
 __device__ __forceinline__ const float4* derived_brick(const VolumeDev& v, int bi) {
-    return reinterpret_cast<const float4*>(v.dbricks + (size_t)(unsigned)bi * (unsigned)der_brick_floats(kBS));
+    return reinterpret_cast<const float4*>(
+        v.dbricks + (size_t)(unsigned)bi * (unsigned)(kBS ? der_brick_floats(kBS) : v.der_stride));
 }
 
 // The sample field, from the derived bricks (voxel-wise derivatives) or by the
@@ -61,7 +62,7 @@ __device__ __forceinline__ void eval_field(const VolumeDev& v, const TissueDev& 
                                            float fld[10]) {
     if (kDerived) {
         const float4* brick = derived_brick<kBS>(v, bi);
-        const int m = (1 << kBS) - 1, E = m + 2;
+        const int m = (1 << (kBS ? kBS : v.bs)) - 1, E = m + 2;
         derived_channels<true, 0, 4>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
         if (kHessian)
             derived_channels<true, 4, 6>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
@@ -268,6 +269,106 @@ __global__ void __launch_bounds__(256) k_channels_to_voxels(const float* __restr
     }
 }
 
+// The sample of the reverse sweep at fractions f of cell i0: its field and optics. No
+// skipping: a sample in empty space has alpha = 0, but its lookup still gives the opacity
+// entries it reads a non-zero gradient. bs: log2 of the skip-brick edge.
+template <bool kDerived, bool kLazyHessian, bool kNoHessian, bool k2D, int kBS>
+__device__ __forceinline__ void sweep_eval(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
+                                           const int i0[3], const float f[3], const float dir[3], const float is[3],
+                                           float inv_gmax, float fld[10], SampleOptics& so) {
+    const int bs = kBS ? kBS : v.bs, bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
+    const int bi = bidx(v, bc);
+    int base;
+    const long long sbi = storage_brick(v, i0, base);
+    const float vval = v.vbricks ? value_eval(GLoad{v.vbricks + sbi * kBrickVox}, base, f[0], f[1], f[2]) : 0.f;
+    if (kLazyHessian) {
+        // I and the gradient, the table lookup, then the Hessian, which without
+        // a curvature term only dL/dgamma needs -- and not at a zero opacity
+        // entry (dL/dw = 0 there, and w = 1 whatever kappa)
+        const float4* brick = derived_brick<kBS>(v, bi);
+        const int m = (1 << bs) - 1, E = m + 2;
+        derived_channels<true, 0, 4>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
+        optics_tf<k2D ? 2 : 1>(fld, vval, tp, tf, inv_gmax, so);
+        if (!kNoHessian && so.c.w != 0.0f) {
+            derived_channels<true, 4, 6>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
+        } else {
+#pragma unroll
+            for (int q = 4; q < 10; ++q) fld[q] = 0.0f;
+        }
+        optics_rest(fld, dir, tp, so);
+    } else {
+        eval_field<kDerived, true, kBS>(v, tp, bi, sbi, i0, base, f, is, fld);
+        optics_core<k2D ? 2 : 1>(fld, vval, dir, tp, tf, inv_gmax, so);
+    }
+}
+
+// dL/dalpha of a sample with transmittance Tk in front of it, the colour R and
+// transmittance P of everything behind it.
+__device__ __forceinline__ float sweep_dalpha(const SampleOptics& so, const float4& g4, float Tk, float R0, float R1,
+                                              float R2, float P) {
+    return Tk * (fmaf(g4.x, so.col[0] - R0, fmaf(g4.y, so.col[1] - R1, g4.z * (so.col[2] - R2))) + g4.w * P);
+}
+
+// Zero opacity entry: alpha = 0 exactly, so only the table's opacity entries at the
+// lookup receive a gradient (the one-sided derivative of the clamp at 0); colour, uniforms
+// and field gradients are all zero.
+template <bool k2D>
+__device__ __forceinline__ void sweep_apply_empty(const TissueDev& tp, const SampleOptics& so, float da,
+                                                  TfGradSink<k2D>& sink) {
+    if (tp.alpha_exp > 0.0f) da *= tp.alpha_exp;
+    const float dr[4] = {0.f, 0.f, 0.f,
+                         (so.raw >= 0.0f && so.raw <= 1.0f) ? da * tp.opacity_scale * so.mg * so.wk : 0.0f};
+    if (!k2D)
+        sink.add_cell(so.j, 1.0f - so.t, so.t, 0.0f, 0.0f, dr);
+    else
+        sink.add_cell(so.k * tp.tf_w + so.j, (1.0f - so.q) * (1.0f - so.t), (1.0f - so.q) * so.t,
+                      so.q * (1.0f - so.t), so.q * so.t, dr);
+}
+
+// Any other sample: table, uniform and (unless kTfOnly) voxel gradients. `pair`: the lane
+// distance whose lane the channel scatter tries to merge with after its neighbour.
+template <bool kDerived, bool kTfOnly, bool k2D>
+__device__ __forceinline__ void sweep_apply(const BackwardLaunch& B, const float fld[10], const SampleOptics& so,
+                                            const int i0[3], const float f[3], const float dir[3], const float is[3],
+                                            float inv_gmax, float da, float Tk, const float4& g4, int pair,
+                                            TfGradSink<k2D>& sink, ParamGrad& dp) {
+    const VolumeDev& v = B.r.vol;
+    const float ta = Tk * so.alpha;
+    const float dc[3] = {ta * g4.x, ta * g4.y, ta * g4.z};
+    float dfs[10];
+    sample_adjoint(fld, so, dir, B.r.tp, inv_gmax, da, dc, sink, dp, dfs);
+    if (kTfOnly) return;
+    if (kDerived && B.dgrad) {
+        scatter_channels(B.dgrad, v.n, i0, f, dfs, pair);
+    } else if (B.dvol) {
+        const int x0 = i0[0] - 1, y0 = i0[1] - 1, z0 = i0[2] - 1;
+        const int nx = v.n[0], ny = v.n[1], nz = v.n[2];
+        float* dv = B.dvol;
+        field_adjoint_scatter(dfs, is, f[0], f[1], f[2], [&](int a, int b, int c, float g) {
+            if (g == 0.0f) return;
+            const int x = min(max(x0 + a, 0), nx - 1), y = min(max(y0 + b, 0), ny - 1),
+                      z = min(max(z0 + c, 0), nz - 1);
+            atomicAdd(dv + ((long long)z * ny + y) * nx + x, g);
+        });
+    }
+}
+
+// Uniform gradients of a warp: one double-precision addition per warp and parameter
+// (float additions of thousands of warps lost 1e-6 of the sum).
+__device__ __forceinline__ void add_param_grads(const ParamGrad& dp, double* __restrict__ dparams) {
+    float pv[5] = {dp.gamma, dp.ka, dp.kd, dp.ks, dp.os};
+#pragma unroll
+    for (int e = 0; e < 5; ++e) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) pv[e] += __shfl_xor_sync(0xffffffffu, pv[e], o);
+    }
+    if ((threadIdx.x & 31) == 0 && dparams) {
+#pragma unroll
+        for (int e = 0; e < 5; ++e)
+            if (pv[e] != 0.0f) atomicAdd(dparams + e, (double)pv[e]);
+    }
+}
+
 // 4 resident CTAs per SM (<= 128 registers): measured 1 ms faster at 1080p than
 // the 3 that the unbounded register count allows. The sweep re-evaluates every sample
 // and is bound by instructions and registers (16 warps at 55-60 % issue), so what a
@@ -368,7 +469,6 @@ __global__ void __launch_bounds__(128, kTfOnly && !k2D ? 5 : 4) k_render_backwar
     }
     {
             float Tk1 = Tk, R0 = 0.f, R1 = 0.f, R2 = 0.f, P = 1.0f;
-            const float dC[3] = {g4.x, g4.y, g4.z};
             // 2. reverse sweep, the lanes of a warp in step: at iteration kr every lane
             // whose ray reaches that far works on its sample kr, so neighbouring rays sit
             // at nearly the same depth and their reads and reductions hit the same cells
@@ -379,108 +479,135 @@ __global__ void __launch_bounds__(128, kTfOnly && !k2D ? 5 : 4) k_render_backwar
             for (int q = 0; q < 3; ++q) U[q] = hit ? r.u0[q] + (long long)kmax * r.du[q] : 0ll;
             for (int kr = kmax; kr >= 0; --kr, U[0] -= r.du[0], U[1] -= r.du[1], U[2] -= r.du[2]) {
                 if (kr > kstop) continue;
-                int i0[3], bc[3];
+                int i0[3];
                 float f[3];
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    cell_at(U[q], v.n[q], i0[q], f[q]);
-                    bc[q] = i0[q] >> kBS;
-                }
-                // No skipping here: a sample in an empty brick has alpha = 0, but its lookup
-                // still gives the opacity entries it reads a non-zero gradient.
+                for (int q = 0; q < 3; ++q) cell_at(U[q], v.n[q], i0[q], f[q]);
                 if (!VR_CHECK(L.tp.status, (unsigned)i0[0] <= (unsigned)(v.n[0] - 2) &&
                                                (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
                                                (unsigned)i0[2] <= (unsigned)(v.n[2] - 2)))
                     continue;
-                const int bi = bidx(v, bc);
-                int base;
-                const long long sbi = storage_brick(v, i0, base);
                 float fld[10];
-                const float vval =
-                    v.vbricks ? value_eval(GLoad{v.vbricks + sbi * kBrickVox}, base, f[0], f[1], f[2]) : 0.f;
                 SampleOptics so;
-                if (kLazyHessian) {
-                    // I and the gradient, the table lookup, then the Hessian, which without
-                    // a curvature term only dL/dgamma needs -- and not at a zero opacity
-                    // entry (dL/dw = 0 there, and w = 1 whatever kappa)
-                    const float4* brick = derived_brick<kBS>(v, bi);
-                    const int m = (1 << kBS) - 1, E = m + 2;
-                    derived_channels<true, 0, 4>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
-                    optics_tf<k2D ? 2 : 1>(fld, vval, L.tp, tf, inv_gmax, so);
-                    if (!kNoHessian && so.c.w != 0.0f) {
-                        derived_channels<true, 4, 6>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2],
-                                                     fld + 4);
-                    } else {
-#pragma unroll
-                        for (int q = 4; q < 10; ++q) fld[q] = 0.0f;
-                    }
-                    optics_rest(fld, r.dir, L.tp, so);
-                } else {
-                    eval_field<kDerived, true, kBS>(v, L.tp, bi, sbi, i0, base, f, is, fld);
-                    optics_core<k2D ? 2 : 1>(fld, vval, r.dir, L.tp, tf, inv_gmax, so);
-                }
-                const float alpha = so.alpha, col[3] = {so.col[0], so.col[1], so.col[2]};
+                sweep_eval<kDerived, kLazyHessian, kNoHessian, k2D, kBS>(v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld,
+                                                                         so);
+                const float alpha = so.alpha;
                 // T_k = T_{k+1} / (1 - alpha_k); Tk still holds T_{k+1} here, which a zero
                 // alpha leaves unchanged (x / 1 = x), so the division is skipped then
                 if (kr != kstop && alpha != 0.0f) Tk = Tk1 / (1.0f - alpha);
-                const float da = Tk * (fmaf(dC[0], col[0] - R0, fmaf(dC[1], col[1] - R1, dC[2] * (col[2] - R2))) +
-                                       g4.w * P);
+                const float da = sweep_dalpha(so, g4, Tk, R0, R1, R2, P);
                 if (so.c.w == 0.0f) {
-                    // zero opacity entry: alpha = 0 exactly, so only the table's opacity
-                    // entries at the lookup receive a gradient (the one-sided derivative of
-                    // the clamp at 0); colour, uniforms and field gradients are all zero
-                    float dal = da;
-                    if (L.tp.alpha_exp > 0.0f) dal *= L.tp.alpha_exp;
-                    const float dr[4] = {0.f, 0.f, 0.f,
-                                         (so.raw >= 0.0f && so.raw <= 1.0f) ? dal * L.tp.opacity_scale * so.mg * so.wk
-                                                                            : 0.0f};
-                    if (!k2D)
-                        sink.add_cell(so.j, 1.0f - so.t, so.t, 0.0f, 0.0f, dr);
-                    else
-                        sink.add_cell(so.k * L.tp.tf_w + so.j, (1.0f - so.q) * (1.0f - so.t), (1.0f - so.q) * so.t,
-                                      so.q * (1.0f - so.t), so.q * so.t, dr);
+                    sweep_apply_empty(L.tp, so, da, sink);
                     Tk1 = Tk;
                     continue;
                 }
-                const float ta = Tk * alpha;
-                const float dc[3] = {ta * dC[0], ta * dC[1], ta * dC[2]};
-                float dfs[10];
-                sample_adjoint(fld, so, r.dir, L.tp, inv_gmax, da, dc, sink, dp, dfs);
-                if (kTfOnly) {
-                } else if (kDerived && B.dgrad) {
-                    scatter_channels(B.dgrad, v.n, i0, f, dfs, L.packet_w);
-                } else if (B.dvol) {
-                    const int x0 = i0[0] - 1, y0 = i0[1] - 1, z0 = i0[2] - 1;
-                    const int nx = v.n[0], ny = v.n[1], nz = v.n[2];
-                    float* dv = B.dvol;
-                    field_adjoint_scatter(dfs, is, f[0], f[1], f[2], [&](int a, int b, int c, float g) {
-                        if (g == 0.0f) return;
-                        const int x = min(max(x0 + a, 0), nx - 1), y = min(max(y0 + b, 0), ny - 1),
-                                  z = min(max(z0 + c, 0), nz - 1);
-                        atomicAdd(dv + ((long long)z * ny + y) * nx + x, g);
-                    });
-                }
-                R0 = fmaf(alpha, col[0], (1.0f - alpha) * R0);
-                R1 = fmaf(alpha, col[1], (1.0f - alpha) * R1);
-                R2 = fmaf(alpha, col[2], (1.0f - alpha) * R2);
+                sweep_apply<kDerived, kTfOnly>(B, fld, so, i0, f, r.dir, is, inv_gmax, da, Tk, g4, L.packet_w, sink,
+                                               dp);
+                R0 = fmaf(alpha, so.col[0], (1.0f - alpha) * R0);
+                R1 = fmaf(alpha, so.col[1], (1.0f - alpha) * R1);
+                R2 = fmaf(alpha, so.col[2], (1.0f - alpha) * R2);
                 P *= (1.0f - alpha);
                 Tk1 = Tk;
             }
     }
     sink.flush();
     if (kTfOnly) return;
-    // uniform gradients: warp sums, one atomic per warp and parameter
-    float pv[5] = {dp.gamma, dp.ka, dp.kd, dp.ks, dp.os};
-#pragma unroll
-    for (int e = 0; e < 5; ++e) {
-#pragma unroll
-        for (int o = 16; o; o >>= 1) pv[e] += __shfl_xor_sync(0xffffffffu, pv[e], o);
+    add_param_grads(dp, B.dparams);
+}
+
+// The sweep with G lanes per ray (G = L.lanes, a power of two up to 16), for launches
+// with too few rays to fill the chip and a recorded ray state: lane g evaluates sample
+// kb - g, every lane of the ray then repeats the recurrences of T, R and P over the G
+// samples in the sweep's order on shuffled opacities and colours, keeping the values at
+// its own sample, and applies its sample's adjoint. Time falls with the serial chain
+// (backward_lanes has the figures). 3 CTAs per SM (168 registers) where the field's
+// adjoint is wanted: up to 10 % faster than 4 with their spills; 4 for the table alone.
+template <bool kLazyHessian, bool kNoHessian, bool kTfOnly, bool k2D>
+__global__ void __launch_bounds__(128, kTfOnly ? 4 : 3) k_backward_lanes(const __grid_constant__ BackwardLaunch B) {
+    const RenderLaunch& L = B.r;
+    const size_t ncell = (size_t)L.tp.tf_w * L.tp.tf_h * kTfCellFloats;
+    const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    TfGradSink<k2D> sink(B.dtf_copies + (size_t)(cta % B.n_copies) * ncell);
+    const int G = L.lanes, lane = threadIdx.x & 31, g = lane & (G - 1), first = lane & ~(G - 1);
+    const int ray = lane / G, pw = L.packet_w;
+    const int i = (blockIdx.x * 4 + (threadIdx.x >> 5)) * pw + (ray & (pw - 1));
+    const int j = blockIdx.y * L.packet_h + ray / pw;
+    const int cam = blockIdx.z;
+    const VolumeDev& v = L.vol;
+    const float4* tf = reinterpret_cast<const float4*>(L.tf);
+    const float gmax = __ldg(&v.vc->gmax);
+    const float inv_gmax = gmax > 0.0f ? 1.0f / gmax : 0.0f;
+    const float is[3] = {1.0f / v.s[0], 1.0f / v.s[1], 1.0f / v.s[2]};
+    ParamGrad dp{0.f, 0.f, 0.f, 0.f, 0.f};
+    RayDev r;
+    float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    int kstop = -1;
+    float Tk = 1.0f;
+    const bool hit = i < L.W && j < L.H && setup_ray(L.cams[cam], L.rc, i, j, v.n, v.s, r);
+    if (hit) {
+        const long long pix = ((long long)(L.cam_offset + cam) * L.H + j) * L.W + i;
+        g4 = __ldg(reinterpret_cast<const float4*>(B.dl_drgba) + pix);
+        const float2 st = __ldg(L.ray_state + pix);
+        kstop = __float_as_int(st.x);
+        Tk = st.y;
+        if (!VR_CHECK(L.tp.status, kstop >= -1 && kstop < r.ns)) kstop = -1;  // a state of another image
     }
-    if (l == 0 && B.dparams) {
+    const int kmax = __reduce_max_sync(0xffffffffu, kstop);
+    long long U[3];
 #pragma unroll
-        for (int e = 0; e < 5; ++e)
-            if (pv[e] != 0.0f) atomicAdd(B.dparams + e, pv[e]);
+    for (int q = 0; q < 3; ++q) U[q] = hit ? r.u0[q] + (long long)(kmax - g) * r.du[q] : 0ll;
+    float Tk1 = Tk, R0 = 0.f, R1 = 0.f, R2 = 0.f, P = 1.0f;
+    for (int kb = kmax; kb >= 0; kb -= G) {
+        const int kr = kb - g;
+        bool on = kr >= 0 && kr <= kstop;
+        int i0[3] = {0, 0, 0};
+        float f[3] = {0.f, 0.f, 0.f}, fld[10];
+        SampleOptics so;
+        so.alpha = so.c.w = so.col[0] = so.col[1] = so.col[2] = 0.0f;
+        if (on) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) cell_at(U[q], v.n[q], i0[q], f[q]);
+            on = VR_CHECK(L.tp.status, (unsigned)i0[0] <= (unsigned)(v.n[0] - 2) &&
+                                           (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
+                                           (unsigned)i0[2] <= (unsigned)(v.n[2] - 2));
+            if (on)
+                sweep_eval<true, kLazyHessian, kNoHessian, k2D, 0>(v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld, so);
+        }
+        const unsigned shaded = __ballot_sync(0xffffffffu, on && so.c.w != 0.0f);
+        // the recurrences over the samples kb, kb - 1, ...; a sample of zero opacity entry
+        // leaves T, R and P as they are
+        float myT = 1.0f, myR0 = 0.f, myR1 = 0.f, myR2 = 0.f, myP = 1.0f;
+        for (int h = 0; h < G; ++h) {
+            const int src = first + h;
+            const float a = __shfl_sync(0xffffffffu, so.alpha, src);
+            const float c0 = __shfl_sync(0xffffffffu, so.col[0], src), c1 = __shfl_sync(0xffffffffu, so.col[1], src),
+                        c2 = __shfl_sync(0xffffffffu, so.col[2], src);
+            const bool sh = (shaded >> src) & 1u;
+            if (sh && kb - h != kstop && a != 0.0f) Tk = Tk1 / (1.0f - a);
+            if (h == g) {
+                myT = Tk;
+                myR0 = R0, myR1 = R1, myR2 = R2, myP = P;
+            }
+            if (sh) {
+                R0 = fmaf(a, c0, (1.0f - a) * R0);
+                R1 = fmaf(a, c1, (1.0f - a) * R1);
+                R2 = fmaf(a, c2, (1.0f - a) * R2);
+                P *= (1.0f - a);
+                Tk1 = Tk;
+            }
+        }
+        if (on) {
+            const float da = sweep_dalpha(so, g4, myT, myR0, myR1, myR2, myP);
+            if (so.c.w == 0.0f)
+                sweep_apply_empty(L.tp, so, da, sink);
+            else
+                sweep_apply<true, kTfOnly>(B, fld, so, i0, f, r.dir, is, inv_gmax, da, myT, g4, G, sink, dp);
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) U[q] -= (long long)G * r.du[q];
     }
+    sink.flush();
+    if (!kTfOnly) add_param_grads(dp, B.dparams);
 }
 
 // Brick-synchronous variant of the reverse sweep. Phase 1 (the forward
@@ -676,17 +803,7 @@ __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_con
         }
     }
     sink.flush();
-    float pv[5] = {dp.gamma, dp.ka, dp.kd, dp.ks, dp.os};
-#pragma unroll
-    for (int e = 0; e < 5; ++e) {
-#pragma unroll
-        for (int o = 16; o; o >>= 1) pv[e] += __shfl_xor_sync(0xffffffffu, pv[e], o);
-    }
-    if (l == 0 && B.dparams) {
-#pragma unroll
-        for (int e = 0; e < 5; ++e)
-            if (pv[e] != 0.0f) atomicAdd(B.dparams + e, pv[e]);
-    }
+    add_param_grads(dp, B.dparams);
 }
 
 // dtf[e] += the sum over copies [16 g, 16 g + 16) of entry e's share of the cells
@@ -696,8 +813,11 @@ __global__ void __launch_bounds__(128) k_render_backward_staged(const __grid_con
 // cell's j < w - 1 and, in a 2D table, k < h - 1); in a cell record the opacity of
 // corner q is float q, its RGB floats 4 + 3 q .. 6 + 3 q (1D: 2 + 3 q .. 4 + 3 q).
 constexpr int kCopiesPerThread = 16;
+// The first five threads also round the uniform gradients' double sums.
 __global__ void __launch_bounds__(256) k_sum_copies(const float* __restrict__ copies, int n_copies, int w, int h,
-                                                   float* __restrict__ out) {
+                                                   float* __restrict__ out, const double* __restrict__ dparams,
+                                                   float* __restrict__ out_params) {
+    if (out_params && blockIdx.x == 0 && threadIdx.x < 5) out_params[threadIdx.x] = (float)dparams[threadIdx.x];
     const long long n = 4ll * w * h;
     const long long stride = (long long)w * h * kTfCellFloats;
     const long long groups = (n_copies + kCopiesPerThread - 1) / kCopiesPerThread;
@@ -733,11 +853,12 @@ cudaError_t launch_channels_to_voxels(const float* dgrad, const int n[3], const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_sum_copies(const float* copies, int n_copies, int tf_w, int tf_h, float* dtf, cudaStream_t st) {
+cudaError_t launch_sum_copies(const float* copies, int n_copies, int tf_w, int tf_h, float* dtf,
+                              const double* dparams, float* out_params, cudaStream_t st) {
     const long long n = 4ll * tf_w * tf_h;
     const long long blocks = (n * ((n_copies + kCopiesPerThread - 1) / kCopiesPerThread) + 255) / 256;
     k_sum_copies<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, st>>>(copies, n_copies, tf_w, tf_h,
-                                                                               dtf);
+                                                                               dtf, dparams, out_params);
     return cudaGetLastError();
 }
 
@@ -768,8 +889,53 @@ void launch_backward_table(const BackwardLaunch& B, dim3 grid, cudaStream_t st) 
     }
 }
 
+template <bool k2D>
+void launch_backward_lanes(const BackwardLaunch& B, dim3 grid, cudaStream_t st) {
+    const bool tf_only = !B.dparams && !B.dvol && !B.dgrad;
+    if (B.r.tp.gk == 0.0f && tf_only)
+        k_backward_lanes<true, true, true, k2D><<<grid, 128, 0, st>>>(B);
+    else if (B.r.tp.gk == 0.0f && !B.dparams)
+        k_backward_lanes<true, true, false, k2D><<<grid, 128, 0, st>>>(B);
+    else if (B.r.tp.gk == 0.0f)
+        k_backward_lanes<true, false, false, k2D><<<grid, 128, 0, st>>>(B);
+    else if (tf_only)
+        k_backward_lanes<false, false, true, k2D><<<grid, 128, 0, st>>>(B);
+    else
+        k_backward_lanes<false, false, false, k2D><<<grid, 128, 0, st>>>(B);
+}
+
+// Lanes per ray of a backward launch with that many rays. One lane per ray fills the
+// chip at 152 SMs x 16 warps x 32 = 78 k rays. Forward + backward with every gradient,
+// measured us at 1 / 2 / 4 / 8 / 16 lanes (128^3 head, 1D table; 181x217x181 head, 2D):
+//    64 x 64    1017 / 541 / 366 / 285 / 252     96 x 96   1886 / 1095 /  834 /  739 /  732
+//   128 x 128    854 / 522 / 393 / 387 / 412    160 x 160  1870 / 1233 / 1102 / 1023 / 1058
+//   256 x 256    864 / 820 / 800 / 886 / 1069   256 x 256  2394 / 1850 / 1694 / 1716 / 1889
+//   384 x 384   1217 / 1370 / 1462 / 1679       400 x 300  2621 / 2118 / 2018 / 2126
+int backward_lanes(long long rays) {
+    return rays <= 6000 ? 16 : rays <= 28000 ? 8 : rays <= 90000 ? 4 : rays <= 122880 ? 2 : 1;
+}
+
+// Shape of a launch with several lanes per ray: rays per warp across and down.
+dim3 lanes_shape(RenderLaunch& L, int lanes) {
+    const int rays = 32 / lanes;
+    L.lanes = lanes;
+    L.packet_w = rays >= 8 ? 4 : (rays >= 4 ? 2 : 1);
+    L.packet_h = rays / L.packet_w;
+    return dim3((L.W + 4 * L.packet_w - 1) / (4 * L.packet_w), (L.H + L.packet_h - 1) / L.packet_h, L.n_cams);
+}
+
 cudaError_t launch_render_backward(const BackwardLaunch& B, bool staged, cudaStream_t st) {
     const RenderLaunch& L = B.r;
+    const int lanes = backward_lanes((long long)L.W * L.H * L.n_cams);
+    if (lanes > 1 && !staged && L.ray_state && L.vol.dbricks) {
+        BackwardLaunch C = B;
+        const dim3 shape = lanes_shape(C.r, lanes);
+        if (L.tp.tf_h > 1)
+            launch_backward_lanes<true>(C, shape, st);
+        else
+            launch_backward_lanes<false>(C, shape, st);
+        return cudaGetLastError();
+    }
     dim3 grid((L.W + 15) / 16, (L.H + 7) / 8, L.n_cams);
     if (staged) {
         const int smem = 4 * kBrickBytes;

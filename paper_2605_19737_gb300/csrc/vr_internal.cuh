@@ -217,7 +217,7 @@ struct BackwardLaunch {
     RenderLaunch r;
     const float* dl_drgba;  // [n_cams][H][W][4] upstream gradient
     float* dtf;             // [tf_h][tf_w][4], zeroed by the caller
-    float* dparams;         // gamma, ka, kd, ks, opacity_scale, zeroed by the caller
+    double* dparams;        // sums for gamma, ka, kd, ks, opacity_scale, zeroed by the caller, or nullptr
     float* dvol;            // nvox or nullptr, zeroed by the caller
     float* dtf_copies;      // n_copies zeroed private copies of the transfer-function gradient, one
                             // 16-float record per lookup cell (TfGradSink); CTA c adds into copy c % n_copies
@@ -295,8 +295,10 @@ cudaError_t launch_gauss3d(const float* in, float* out, float* tmp, const int n[
 // warps: warps per CTA (2, 4 or 8), tiled by tile_pixel.
 cudaError_t launch_render_gather(const RenderLaunch& L, int warps, cudaStream_t st);
 cudaError_t launch_render_backward(const BackwardLaunch& B, bool staged, cudaStream_t st);
-// dtf += the entries' shares of the cell records of every copy
-cudaError_t launch_sum_copies(const float* copies, int n_copies, int tf_w, int tf_h, float* dtf, cudaStream_t st);
+// dtf += the entries' shares of the cell records of every copy; out_params (nullable) =
+// the uniform gradients' sums rounded to float
+cudaError_t launch_sum_copies(const float* copies, int n_copies, int tf_w, int tf_h, float* dtf,
+                              const double* dparams, float* out_params, cudaStream_t st);
 cudaError_t launch_fma_peak(float* out, int blocks, int iters, cudaStream_t st);
 cudaError_t launch_wait_probe(unsigned* status, long long budget_cycles, cudaStream_t st);
 // One thread fails one index check (debug builds record it; release builds do nothing).

@@ -67,3 +67,25 @@ def test_fewer_gradients_same_values(torch, mode, gamma, derived, brick, stated)
             assert _rel(other[0], full[0]) <= 2e-5
         assert _rel(no_vol[1], full[1]) <= 2e-5
         assert _rel(no_par[2], full[2]) <= 2e-5
+
+
+# both sides of every line between 16, 8, 4, 2 and 1 lanes per ray
+@pytest.mark.parametrize("W,H", [(9, 5), (75, 80), (95, 64), (160, 175), (180, 160), (300, 300), (303, 300),
+                                 (384, 320), (390, 320)])
+@pytest.mark.parametrize("mode,gamma,corr", [(0, 0.0, 0.0), (1, 0.6, 0.0), (2, 0.6, 0.8)])
+def test_lanes_per_ray(torch, W, H, mode, gamma, corr):
+    """With a recorded ray state a small launch gives each ray several lanes; without one
+    it re-marches with one lane per ray. Same terms, another order."""
+    import paper_2605_19737_gb300 as pkg
+    with pkg.Context(0) as ctx:
+        vid, cams, g = _scene(ctx, torch, mode, gamma, True, 8, W, H, 1, corr)
+        st = torch.empty((1, H, W, 2), device="cuda")
+        ctx.render(vid, cams, W, H, ray_state=st)
+        lanes = ctx.render_backward(vid, cams, W, H, g, ray_state=st)
+        tf_only = ctx.render_backward(vid, cams, W, H, g, ray_state=st, want_params=False, want_volume=False)
+        one = ctx.render_backward(vid, cams, W, H, g)
+        ctx.synchronize()
+        assert float(one[2].abs().max()) > 0
+        for a, b in zip(lanes, one):
+            assert _rel(a, b) <= 2e-5
+        assert _rel(tf_only[0], one[0]) <= 2e-5
