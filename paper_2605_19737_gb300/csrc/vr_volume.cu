@@ -138,52 +138,66 @@ __global__ void k_normalize(const T* __restrict__ raw, long long n, const float*
     for (long long i = tid; i < n; i += stride) out[i] = __fdiv_rn(__fsub_rn((float)__ldg(raw + i), imin), range);
 }
 
-// One CTA per brick: copy voxels [8b-1, 8b+11) per axis (clamped) into the
-// brick's 12^3 block. Reads are row-contiguous in x, writes fully contiguous.
+// Voxels [8b-1, 8b+11) per axis (clamped) of each brick into its 12^3 block: a thread per
+// 16-byte piece of the output (432 per brick), so that stores are whole vectors and the
+// index arithmetic is paid once per four voxels (181x217x181: 44 us with one voxel per
+// thread -> 36 us, 99 MB written).
+constexpr int kBrickPieces = kBrickVox / 4;
 __global__ void __launch_bounds__(256) k_make_bricks(const float* __restrict__ norm, int nx, int ny, int nz, int nbx,
-                                                     int nby, float* __restrict__ bricks) {
-    const long long b = blockIdx.x;
-    const int bx = (int)(b % nbx), by = (int)((b / nbx) % nby), bz = (int)(b / ((long long)nbx * nby));
-    float* dst = bricks + b * kBrickVox;
-#pragma unroll
-    for (int q = 0; q < (kBrickVox + 255) / 256; ++q) {  // 256 threads: the loads issue back to back
-        const int e = threadIdx.x + 256 * q;
-        if (e >= kBrickVox) break;
-        const int lx = e % kEdge, ly = (e / kEdge) % kEdge, lz = e / (kEdge * kEdge);
-        const int x = min(max(kCells * bx - 1 + lx, 0), nx - 1);
-        const int y = min(max(kCells * by - 1 + ly, 0), ny - 1);
-        const int z = min(max(kCells * bz - 1 + lz, 0), nz - 1);
-        dst[e] = __ldg(norm + ((long long)z * ny + y) * nx + x);
-    }
+                                                     int nby, long long npieces, float4* __restrict__ bricks) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= npieces) return;
+    const int b = (int)(i / kBrickPieces), e = (int)(i - (long long)b * kBrickPieces);
+    const int bx = b % nbx, by = (b / nbx) % nby, bz = b / (nbx * nby);
+    const int px = e % 3, ly = (e / 3) % kEdge, lz = e / (3 * kEdge);
+    const int x = kCells * bx - 1 + 4 * px;
+    const int y = min(max(kCells * by - 1 + ly, 0), ny - 1);
+    const int z = min(max(kCells * bz - 1 + lz, 0), nz - 1);
+    const float* row = norm + ((long long)z * ny + y) * nx;
+    float4 v;
+    v.x = __ldg(row + min(max(x, 0), nx - 1));
+    v.y = __ldg(row + min(x + 1, nx - 1));
+    v.z = __ldg(row + min(x + 2, nx - 1));
+    v.w = __ldg(row + min(x + 3, nx - 1));
+    bricks[i] = v;
 }
 
 // One CTA per skip brick: the voxel-wise intensity, central-difference gradient
 // (Eq. 2) and second/mixed differences (Sec. 2.3) of the brick's (B+1)^3 corner
 // voxels, with clamp-to-edge neighbours, divided by the spacing -- the per-voxel
 // morphology the paper's compute shader produces, laid out for 16-byte loads.
+// A warp passes its 32 corners' records (48 bytes each) through shared memory and stores
+// them as 1536 consecutive bytes: stored straight from the threads that computed them, a
+// warp's store wrote 16 of every 48 bytes
+// (181x217x181 at B = 8, 518 MB: 136 -> 116 us; 256x256x176, 788 MB: 213 -> 192 us). kBS
+// (log2 B) at compile time keeps the divisions by the edges out.
+template <int kBS>
 __global__ void __launch_bounds__(256) k_make_derived(const float* __restrict__ norm, int nx, int ny, int nz, int nbx,
-                                                      int nby, int bs, float hx, float hy, float hz,
-                                                      float* __restrict__ out) {
+                                                      int nby, float hx, float hy, float hz, float* __restrict__ out) {
     // the brick's corner voxels and their neighbours, [Bb - 1, Bb + B + 2) per axis,
     // clamped to the volume (so neighbour i +- 1 of a corner is tile entry t +- 1)
-    constexpr int kTMax = (1 << kMaxBrickShift) + 3;
-    __shared__ float tile[kTMax * kTMax * kTMax];
-    const int B = 1 << bs, E = B + 1, T = B + 3;
-    const long long b = blockIdx.x;
-    const int bx = (int)(b % nbx), by = (int)((b / nbx) % nby), bz = (int)(b / ((long long)nbx * nby));
+    constexpr int B = 1 << kBS, E = B + 1, T = B + 3;
+    __shared__ float tile[T * T * T];
+    __shared__ float4 stage[8][96];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int b = blockIdx.x;
+    const int bx = b % nbx, by = (b / nbx) % nby, bz = b / (nbx * nby);
     const int x0 = B * bx - 1, y0 = B * by - 1, z0 = B * bz - 1;
-    for (int e = threadIdx.x; e < T * T * T; e += blockDim.x) {
+    for (int e = threadIdx.x; e < T * T * T; e += 256) {
         const int tx = e % T, ty = (e / T) % T, tz = e / (T * T);
         const int x = min(max(x0 + tx, 0), nx - 1), y = min(max(y0 + ty, 0), ny - 1), z = min(max(z0 + tz, 0), nz - 1);
         tile[e] = __ldg(norm + ((long long)z * ny + y) * nx + x);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < E * E * E; e += blockDim.x) {
+    float4* dst = reinterpret_cast<float4*>(out + (size_t)(unsigned)b * (unsigned)der_brick_floats(kBS));
+    for (int e0 = wid * 32; e0 < E * E * E; e0 += 256) {
+        const int e = min(e0 + lane, E * E * E - 1);
         const int lx = e % E, ly = (e / E) % E, lz = e / (E * E);
         // the corner voxel (clamped as in the per-voxel definition) in tile coordinates
         const int tx = min(B * bx + lx, nx - 1) - x0, ty = min(B * by + ly, ny - 1) - y0,
                   tz = min(B * bz + lz, nz - 1) - z0;
-        auto at = [&](int dx, int dy, int dz) { return tile[((tz + dz) * T + (ty + dy)) * T + (tx + dx)]; };
+        const float* t0 = tile + (tz * T + ty) * T + tx;
+        auto at = [&](int dx, int dy, int dz) { return t0[(dz * T + dy) * T + dx]; };
         const float c = at(0, 0, 0), c2 = 2.0f * c;
         float4 a, m, t;
         a.x = c;
@@ -198,35 +212,62 @@ __global__ void __launch_bounds__(256) k_make_derived(const float* __restrict__ 
         t.y = ((at(0, 1, 1) - at(0, 1, -1)) - (at(0, -1, 1) - at(0, -1, -1))) * (0.25f * hy * hz);
         t.z = 0.0f;
         t.w = 0.0f;
-        float4* o = reinterpret_cast<float4*>(out + b * der_brick_floats(bs)) + 3 * e;
-        o[0] = a;
-        o[1] = m;
-        o[2] = t;
+        float4* sp = stage[wid];
+        sp[3 * lane] = a;
+        sp[3 * lane + 1] = m;
+        sp[3 * lane + 2] = t;
+        __syncwarp();
+        const int left = 3 * (E * E * E - e0);  // pieces from e0 on
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (lane + 32 * q < left) dst[3 * e0 + lane + 32 * q] = sp[lane + 32 * q];
+        __syncwarp();
     }
 }
 
-// One warp per skip brick: min/max of I_norm over the brick's corner voxels
-// [Bb, min(Bb+B, N-1)] per axis, quantised to qlo = floor(min*65535),
-// qhi = ceil(max*65535) (float32 round-to-nearest products).
+// Min/max of I_norm over each skip brick's corner voxels [Bb, min(Bb+B, N-1)] per axis,
+// quantised to qlo = floor(min*65535), qhi = ceil(max*65535) (float32 round-to-nearest
+// products). A CTA owns 32/B bricks along x at one (y, z): its eight warps share the
+// (B+1)^2 voxel rows, each read as 32 consecutive values plus one, reduced over the B
+// lanes of a brick, whose last corner is the next brick's first lane (181x217x181, one
+// warp per brick with divisions per voxel: 28 -> 16 us).
+template <int kBS>
 __global__ void __launch_bounds__(256) k_brick_minmax(const float* __restrict__ norm, int nx, int ny, int nz, int nbx,
-                                                      int nby, int bs, long long nbricks, uint16_t* __restrict__ grid) {
-    const long long b = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (b >= nbricks) return;
-    const int B = 1 << bs;
-    const int bx = (int)(b % nbx), by = (int)((b / nbx) % nby), bz = (int)(b / ((long long)nbx * nby));
-    const int x0 = B * bx, y0 = B * by, z0 = B * bz;
-    const int ex = min(x0 + B, nx - 1) - x0 + 1;
-    const int ey = min(y0 + B, ny - 1) - y0 + 1;
-    const int ez = min(z0 + B, nz - 1) - z0 + 1;
-    float lo = INFINITY, hi = -INFINITY;
-    const int cnt = ex * ey * ez;
-    for (int e = lane; e < cnt; e += 32) {
-        const int lx = e % ex, ly = (e / ex) % ey, lz = e / (ex * ey);
-        acc(__ldg(norm + ((long long)(z0 + lz) * ny + (y0 + ly)) * nx + (x0 + lx)), lo, hi);
+                                                      uint16_t* __restrict__ grid) {
+    constexpr int B = 1 << kBS, E = B + 1;
+    __shared__ float slo[8][32], shi[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * B, z0 = blockIdx.z * B;
+    const int xa = min(x0 + lane, nx - 1), xb = min(x0 + 32, nx - 1);
+    float lo = INFINITY, hi = -INFINITY, elo = INFINITY, ehi = -INFINITY;  // own column; lane 31: the 33rd
+#pragma unroll 4
+    for (int r = wid; r < E * E; r += 8) {
+        const int y = min(y0 + r % E, ny - 1), z = min(z0 + r / E, nz - 1);
+        const float* row = norm + ((long long)z * ny + y) * nx;
+        acc(__ldg(row + xa), lo, hi);
+        if (lane == 31) acc(__ldg(row + xb), elo, ehi);
     }
-    warp_minmax(lo, hi);
-    if (lane == 0) {
+    // the brick's columns are its B lanes and the lane after them
+    float nlo = __shfl_down_sync(0xffffffffu, lo, 1), nhi = __shfl_down_sync(0xffffffffu, hi, 1);
+    if (lane == 31) nlo = elo, nhi = ehi;
+    lo = fminf(lo, nlo);
+    hi = fmaxf(hi, nhi);
+#pragma unroll
+    for (int o = B / 2; o; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    slo[wid][lane] = lo;
+    shi[wid][lane] = hi;
+    __syncthreads();
+    const int bx = blockIdx.x * (32 / B) + lane / B;
+    if (wid == 0 && (lane & (B - 1)) == 0 && bx < nbx) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) {
+            lo = fminf(lo, slo[w][lane]);
+            hi = fmaxf(hi, shi[w][lane]);
+        }
+        const long long b = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * nbx + bx;
         // codes clamp to [0, 65535]: intensities set outside [0, 1] (vr_set_normalized)
         // look up the transfer function's end entries, which the clamped range covers
         grid[2 * b] = (uint16_t)fminf(fmaxf(floorf(__fmul_rn(lo, 65535.0f)), 0.0f), 65535.0f);
@@ -237,19 +278,34 @@ __global__ void __launch_bounds__(256) k_brick_minmax(const float* __restrict__ 
 // |grad I|_max: largest voxel-wise central-difference gradient magnitude
 // (Eq. 2 with clamp-to-edge neighbours), reduced per block then combined with
 // an integer atomicMax on the (non-negative) float's bit pattern.
+// A thread walks kGmaxPlanes planes along z with the centre values of the planes below and
+// above in registers: four in-plane neighbour loads and one new centre per voxel instead of
+// seven loads (256x256x176: 53 -> 30 us).
+constexpr int kGmaxPlanes = 8;
 __global__ void __launch_bounds__(256) k_gmax(const float* __restrict__ I, int nx, int ny, int nz, float hx, float hy,
                                               float hz, VolConst* __restrict__ vc) {
     const int i = blockIdx.x * 32 + (threadIdx.x & 31);
     const int j = blockIdx.y * 8 + (threadIdx.x >> 5);
-    const int k = blockIdx.z;
+    const int k0 = blockIdx.z * kGmaxPlanes;
     float m = 0.0f;
     if (i < nx && j < ny) {
         const long long row = (long long)ny * nx;
-        const float* c = I + (long long)k * row + (long long)j * nx + i;
-        const float gx = (__ldg(c + (i + 1 < nx ? 1 : 0)) - __ldg(c - (i > 0 ? 1 : 0))) * hx;
-        const float gy = (__ldg(c + (j + 1 < ny ? nx : 0)) - __ldg(c - (j > 0 ? nx : 0))) * hy;
-        const float gz = (__ldg(c + (k + 1 < nz ? row : 0)) - __ldg(c - (k > 0 ? row : 0))) * hz;
-        m = sqrtf(gx * gx + gy * gy + gz * gz);
+        const float* c = I + (long long)k0 * row + (long long)j * nx + i;
+        const int xp = i + 1 < nx ? 1 : 0, xm = i > 0 ? -1 : 0, yp = j + 1 < ny ? nx : 0, ym = j > 0 ? -nx : 0;
+        float zm = __ldg(c - (k0 > 0 ? row : 0)), z0 = __ldg(c);
+#pragma unroll
+        for (int q = 0; q < kGmaxPlanes; ++q) {
+            const int k = k0 + q;
+            if (k >= nz) break;
+            const float zp = k + 1 < nz ? __ldg(c + row) : z0;
+            const float gx = (__ldg(c + xp) - __ldg(c + xm)) * hx;
+            const float gy = (__ldg(c + yp) - __ldg(c + ym)) * hy;
+            const float gz = (zp - zm) * hz;
+            m = fmaxf(m, sqrtf(gx * gx + gy * gy + gz * gz));
+            zm = z0;
+            z0 = zp;
+            c += row;
+        }
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -749,31 +805,41 @@ cudaError_t launch_normalize(const void* raw, vr_dtype dt, long long n, const fl
 }
 
 cudaError_t launch_make_bricks(const float* norm, const int n[3], const int nb[3], float* bricks, cudaStream_t st) {
-    const long long nbr = (long long)nb[0] * nb[1] * nb[2];
-    k_make_bricks<<<(unsigned)nbr, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], nb[1], bricks);
+    // nb: storage bricks, at most 256^3 = 2^24, so pieces / 256 fits the grid
+    const long long pieces = (long long)nb[0] * nb[1] * nb[2] * kBrickPieces;
+    k_make_bricks<<<(unsigned)((pieces + 255) / 256), 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], nb[1], pieces,
+                                                                    reinterpret_cast<float4*>(bricks));
     return cudaGetLastError();
 }
 
 cudaError_t launch_brick_minmax(const float* norm, const int n[3], const int nb[3], int bs, uint16_t* grid,
                                 cudaStream_t st) {
-    const long long nbr = (long long)nb[0] * nb[1] * nb[2];
-    const unsigned blocks = (unsigned)((nbr + 7) / 8);
-    k_brick_minmax<<<blocks, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], nb[1], bs, nbr, grid);
+    const dim3 ctas((nb[0] + (32 >> bs) - 1) / (32 >> bs), nb[1], nb[2]);
+    switch (bs) {
+        case 2: k_brick_minmax<2><<<ctas, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], grid); break;
+        case 4: k_brick_minmax<4><<<ctas, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], grid); break;
+        default: k_brick_minmax<3><<<ctas, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], grid); break;
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_make_derived(const float* norm, const int n[3], const int nb[3], int bs, const float s[3],
                                 float* dbricks, cudaStream_t st) {
     const long long nbr = (long long)nb[0] * nb[1] * nb[2];
-    k_make_derived<<<(unsigned)nbr, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], nb[1], bs, 1.0f / s[0],
-                                                  1.0f / s[1], 1.0f / s[2], dbricks);
+    const float hx = 1.0f / s[0], hy = 1.0f / s[1], hz = 1.0f / s[2];
+    const unsigned ctas = (unsigned)nbr;  // <= 512^3
+    switch (bs) {
+        case 2: k_make_derived<2><<<ctas, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], nb[1], hx, hy, hz, dbricks); break;
+        case 4: k_make_derived<4><<<ctas, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], nb[1], hx, hy, hz, dbricks); break;
+        default: k_make_derived<3><<<ctas, 256, 0, st>>>(norm, n[0], n[1], n[2], nb[0], nb[1], hx, hy, hz, dbricks); break;
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_gmax(const float* norm, const int n[3], const float s[3], VolConst* vc, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(&vc->gmax, 0, sizeof(float), st);
     if (e != cudaSuccess) return e;
-    dim3 grid((n[0] + 31) / 32, (n[1] + 7) / 8, n[2]);
+    dim3 grid((n[0] + 31) / 32, (n[1] + 7) / 8, (n[2] + kGmaxPlanes - 1) / kGmaxPlanes);
     k_gmax<<<grid, 256, 0, st>>>(norm, n[0], n[1], n[2], 0.5f / s[0], 0.5f / s[1], 0.5f / s[2], vc);
     return cudaGetLastError();
 }
