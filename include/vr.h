@@ -469,7 +469,10 @@ vr_status vr_debug_check_probe(vr_ctx* ctx);
 
 /* Device memory held by the context: every buffer the library allocates for it
  * (volumes, derived bricks, cell grids, vesselness, batches, scratch) is counted
- * in *bytes; caller-owned buffers (images, counters, ray state) are not. */
+ * in *bytes; caller-owned buffers (images, counters, ray state) are not, nor are freed
+ * buffers that the library keeps for later allocations of the same size by any context on
+ * the device (at most 2 GiB per device; given back when the device is out of memory and
+ * when the last context on it is destroyed; a context with a memory limit keeps none). */
 vr_status vr_memory_used(vr_ctx* ctx, unsigned long long* bytes);
 
 /* Cap on vr_memory_used (0, the default: no cap beyond the device's memory). An

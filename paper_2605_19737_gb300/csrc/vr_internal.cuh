@@ -250,6 +250,10 @@ struct BatchLaunch {
 // Record `msg` as the context's last error and return `status`.
 vr_status set_error(vr_ctx* ctx, vr_status status, const char* msg);
 
+// Process-unique id of the calling thread's current CUDA context, 0 when there is none or
+// the driver cannot tell.
+unsigned long long current_cuda_context();
+
 // ---------------------------------------------------------------- launchers
 // All return cudaSuccess or the launch error; all enqueue on `st`.
 cudaError_t launch_minmax_partials(const void* data, vr_dtype dt, long long n, float* partials, int nblocks,

@@ -889,12 +889,11 @@ typedef int (*CtxGetCurrentFn)(void**);
 typedef int (*CtxGetIdFn)(void*, unsigned long long*);
 CtxGetCurrentFn g_ctx_get_current = nullptr;
 CtxGetIdFn g_ctx_get_id = nullptr;
-bool g_ctx_fns_resolved = false;
+std::once_flag g_ctx_fns_once;
 
 // Id of the calling thread's current CUDA context, 0 when it cannot be told.
 unsigned long long current_ctx_id() {
-    if (!g_ctx_fns_resolved) {
-        g_ctx_fns_resolved = true;
+    std::call_once(g_ctx_fns_once, [] {
         void* f = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
@@ -905,7 +904,7 @@ unsigned long long current_ctx_id() {
             q == cudaDriverEntryPointSuccess)
             g_ctx_get_id = reinterpret_cast<CtxGetIdFn>(f);
         (void)cudaGetLastError();
-    }
+    });
     if (!g_ctx_get_current || !g_ctx_get_id) return 0;
     void* cu = nullptr;
     unsigned long long id = 0;
@@ -921,6 +920,9 @@ void put_msg(char* buf, int len, const char* msg) {
 }
 
 }  // namespace
+
+unsigned long long current_cuda_context() { return current_ctx_id(); }
+
 }  // namespace vr
 
 extern "C" vr_status vr_classify_bricks_noalloc(const unsigned short* d_grid, long long nbricks, const float* d_tf,
