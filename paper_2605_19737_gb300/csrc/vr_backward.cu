@@ -196,76 +196,82 @@ __device__ __forceinline__ void scatter_channels(float* __restrict__ dgrad, cons
     }
 }
 
-// Voxel p's channels read I at clamp(p +- 1) per axis. For voxel v, the p whose
-// "+1" (s = 0) or "-1" (s = 1) neighbour along an axis of size nn clamps to v.
-__device__ __forceinline__ int clamp_sources(int v, int nn, int sgn, int out[2]) {
-    int m = 0;
-    if (sgn == 0) {  // clamp(p + 1) == v
-        if (v >= 1) out[m++] = v - 1;
-        if (v == nn - 1) out[m++] = v;
-    } else {  // clamp(p - 1) == v
-        if (v <= nn - 2) out[m++] = v + 1;
-        if (v == 0) out[m++] = v;
-    }
-    return m;
-}
-
-// dL/dI[v] from the channel gradients: the transpose of the derived channels'
-// clamp-to-edge difference stencils (I; g_a = (I[p+a] - I[p-a]) / (2 s_a);
-// H_aa = (I[p+a] - 2 I[p] + I[p-a]) / s_a^2; H_ab = the four (p +- a +- b)
-// corners / (4 s_a s_b)), gathered per voxel (no atomics).
+// dL/dI from the channel gradients: the transpose of the derived channels' clamp-to-edge
+// difference stencils (I; g_a = (I[p+a] - I[p-a]) / (2 s_a); H_aa = (I[p+a] - 2 I[p] +
+// I[p-a]) / s_a^2; H_ab = the four (p +- a +- b) corners / (4 s_a s_b)).
+// Along one axis the transposed first difference of a channel G at voxel v is
+// d(G)[v] = G[v-1] - G[v+1] and the transposed second difference s(G)[v] = G[v-1] - 2 G[v]
+// + G[v+1], where at the ends, whose clamped neighbour is the end voxel itself, a missing
+// G[v-1] reads -G[v] in d and G[v] in s (and a missing G[v+1] likewise): the sources of
+// voxel 0 are p = 0 (its "-1" neighbour) and p = 1.
+// Separably, with the planes' sums
+//   A = I + d_x(gx) / 2sx + d_y(gy) / 2sy + s_x(Hxx) / sx^2 + s_y(Hyy) / sy^2 + d_x d_y(Hxy) / 4 sx sy
+//   D = gz / 2sz + d_x(Hxz) / 4 sx sz + d_y(Hyz) / 4 sy sz,    S = Hzz / sz^2
+// the voxel is A + d_z(D) + s_z(S). A CTA owns 32 x 8 columns and walks a run of planes: the
+// ten channels of a plane (with their one-voxel border) go through shared memory once and D
+// and S of three planes stay in registers, so every channel is read from memory about 1.3
+// times instead of through 28 scattered loads per voxel (181x217x181: 291 -> 117 us, 312 MB).
+constexpr int kVoxTileY = 8, kVoxPlanes = 12;
 __global__ void __launch_bounds__(256) k_channels_to_voxels(const float* __restrict__ G, int nx, int ny, int nz,
                                                             float sx, float sy, float sz, float* __restrict__ dvol) {
-    const long long nvox = (long long)nx * ny * nz;
-    const int nn[3] = {nx, ny, nz};
-    const float sp[3] = {sx, sy, sz};
-    const int hidx[3][3] = {{4, 7, 8}, {7, 5, 9}, {8, 9, 6}};  // channel of H_ab
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nvox;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int v[3] = {(int)(e % nx), (int)((e / nx) % ny), (int)(e / ((long long)nx * ny))};
-        auto at = [&](const int p[3], int ch) {
-            return __ldg(G + chan_index(((long long)p[2] * ny + p[1]) * nx + p[0], nvox, ch));
-        };
-        float acc = at(v, 0);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const float cg = 0.5f / sp[a], ch = 1.0f / (sp[a] * sp[a]);
-            acc -= 2.0f * ch * at(v, 4 + a);
-#pragma unroll
-            for (int sg = 0; sg < 2; ++sg) {
-                int src[2];
-                const int m = clamp_sources(v[a], nn[a], sg, src);
-                for (int u = 0; u < m; ++u) {
-                    int p[3] = {v[0], v[1], v[2]};
-                    p[a] = src[u];
-                    acc += (sg == 0 ? cg : -cg) * at(p, 1 + a) + ch * at(p, 4 + a);
-                }
-            }
+    constexpr int kW = 34, kH = kVoxTileY + 2, kAll = kW * kH;
+    // per plane: (I, gx, gy, gz), (Hxx, Hyy, Hzz, Hxy), (Hxz, Hyz)
+    __shared__ float4 t0[kAll], t1[kAll];
+    __shared__ float2 t2[kAll];
+    const long long nvox = (long long)nx * ny * nz, plane = (long long)nx * ny;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int x = blockIdx.x * 32 + tx, y = blockIdx.y * kVoxTileY + ty;
+    const int z0 = blockIdx.z * kVoxPlanes, z1 = min(z0 + kVoxPlanes, nz);
+    const bool in = x < nx && y < ny;
+    const float4* G0 = reinterpret_cast<const float4*>(G);
+    const float4* G1 = reinterpret_cast<const float4*>(G + 4 * nvox);
+    const float2* G2 = reinterpret_cast<const float2*>(G + 8 * nvox);
+    const float cx = 0.5f / sx, cy = 0.5f / sy, cz = 0.5f / sz;
+    const float qx = 1.0f / (sx * sx), qy = 1.0f / (sy * sy), qz = 1.0f / (sz * sz);
+    const float mxy = 0.25f / (sx * sy), mxz = 0.25f / (sx * sz), myz = 0.25f / (sy * sz);
+    const int c = (ty + 1) * kW + tx + 1;
+    // the entries this thread stages, clamped into the volume (a clamped border value is
+    // replaced by the end rules below)
+    auto place = [&](int e) {
+        const int gx = min(max((int)blockIdx.x * 32 - 1 + e % kW, 0), nx - 1);
+        const int gy = min(max((int)blockIdx.y * kVoxTileY - 1 + e / kW, 0), ny - 1);
+        return (long long)gy * nx + gx;
+    };
+    const int e1 = threadIdx.x, e2 = threadIdx.x + 256;
+    const long long o1 = place(e1), o2 = e2 < kAll ? place(e2) : 0;
+    // end rules: the clamped border entry is the end voxel's own value, wanted as it is in
+    // s and with the opposite sign in d
+    const float lx = x > 0 ? 1.0f : -1.0f, rx = x < nx - 1 ? 1.0f : -1.0f;
+    const float ly = y > 0 ? 1.0f : -1.0f, ry = y < ny - 1 ? 1.0f : -1.0f;
+    float Am = 0.0f, Dp = 0.0f, Dm = 0.0f, Sp = 0.0f, Sm = 0.0f;  // A, D, S of plane z - 1; D, S of plane z - 2
+    for (int z = z0 - 1; z <= z1; ++z) {
+        const long long zo = (long long)min(max(z, 0), nz - 1) * plane;
+        __syncthreads();
+        t0[e1] = __ldg(G0 + zo + o1);
+        t1[e1] = __ldg(G1 + zo + o1);
+        t2[e1] = __ldg(G2 + zo + o1);
+        if (e2 < kAll) {
+            t0[e2] = __ldg(G0 + zo + o2);
+            t1[e2] = __ldg(G1 + zo + o2);
+            t2[e2] = __ldg(G2 + zo + o2);
         }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-#pragma unroll
-            for (int b = a + 1; b < 3; ++b) {
-                const float cm = 0.25f / (sp[a] * sp[b]);
-#pragma unroll
-                for (int sa = 0; sa < 2; ++sa) {
-#pragma unroll
-                    for (int sb = 0; sb < 2; ++sb) {
-                        int pa[2], pb[2];
-                        const int ma = clamp_sources(v[a], nn[a], sa, pa), mb = clamp_sources(v[b], nn[b], sb, pb);
-                        const float sgn = (sa == sb) ? cm : -cm;
-                        for (int ua = 0; ua < ma; ++ua)
-                            for (int ub = 0; ub < mb; ++ub) {
-                                int p[3] = {v[0], v[1], v[2]};
-                                p[a] = pa[ua];
-                                p[b] = pb[ub];
-                                acc += sgn * at(p, hidx[a][b]);
-                            }
-                    }
-                }
-            }
-        }
-        dvol[e] = acc;
+        __syncthreads();
+        const float4 a = t0[c], h = t1[c];
+        const float hxx = t1[c - 1].x - 2.0f * h.x + t1[c + 1].x, hyy = t1[c - kW].y - 2.0f * h.y + t1[c + kW].y;
+        const float gx = lx * t0[c - 1].y - rx * t0[c + 1].y, gy = ly * t0[c - kW].z - ry * t0[c + kW].z;
+        const float xy = ly * (lx * t1[c - kW - 1].w - rx * t1[c - kW + 1].w) -
+                         ry * (lx * t1[c + kW - 1].w - rx * t1[c + kW + 1].w);
+        const float A = a.x + cx * gx + cy * gy + qx * hxx + qy * hyy + mxy * xy;
+        float D = cz * a.w + mxz * (lx * t2[c - 1].x - rx * t2[c + 1].x) + myz * (ly * t2[c - kW].y - ry * t2[c + kW].y);
+        const float S = qz * h.z;
+        if (z < 0 || z > nz - 1) D = -D;  // the plane past an end is the end plane, with d's sign
+        // voxel z - 1: A + (D[z-2] - D[z]) + (S[z-2] - 2 S[z-1] + S[z])
+        if (z > z0 && in) dvol[(long long)(z - 1) * plane + (long long)y * nx + x] = Am + (Dm - D) + (Sm - 2.0f * Sp + S);
+        Am = A;
+        Dm = Dp;
+        Dp = D;
+        Sm = Sp;
+        Sp = S;
     }
 }
 
@@ -846,10 +852,8 @@ __global__ void __launch_bounds__(256) k_sum_copies(const float* __restrict__ co
 
 cudaError_t launch_channels_to_voxels(const float* dgrad, const int n[3], const float s[3], float* dvol,
                                       cudaStream_t st) {
-    const long long nvox = (long long)n[0] * n[1] * n[2];
-    const long long blocks = (nvox + 255) / 256;
-    k_channels_to_voxels<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, st>>>(dgrad, n[0], n[1], n[2],
-                                                                                          s[0], s[1], s[2], dvol);
+    const dim3 grid((n[0] + 31) / 32, (n[1] + kVoxTileY - 1) / kVoxTileY, (n[2] + kVoxPlanes - 1) / kVoxPlanes);
+    k_channels_to_voxels<<<grid, 256, 0, st>>>(dgrad, n[0], n[1], n[2], s[0], s[1], s[2], dvol);
     return cudaGetLastError();
 }
 
