@@ -211,9 +211,10 @@ __device__ __forceinline__ void scatter_channels(float* __restrict__ dgrad, cons
 // ten channels of a plane (with their one-voxel border) go through shared memory once and D
 // and S of three planes stay in registers, so every channel is read from memory about 1.3
 // times instead of through 28 scattered loads per voxel (181x217x181: 291 -> 117 us, 312 MB).
-constexpr int kVoxTileY = 8, kVoxPlanes = 12;
+constexpr int kVoxTileY = 8;
 __global__ void __launch_bounds__(256) k_channels_to_voxels(const float* __restrict__ G, int nx, int ny, int nz,
-                                                            float sx, float sy, float sz, float* __restrict__ dvol) {
+                                                            float sx, float sy, float sz, int planes,
+                                                            float* __restrict__ dvol) {
     constexpr int kW = 34, kH = kVoxTileY + 2, kAll = kW * kH;
     // per plane: (I, gx, gy, gz), (Hxx, Hyy, Hzz, Hxy), (Hxz, Hyz)
     __shared__ float4 t0[kAll], t1[kAll];
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(256) k_channels_to_voxels(const float* __restr
     const long long nvox = (long long)nx * ny * nz, plane = (long long)nx * ny;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int x = blockIdx.x * 32 + tx, y = blockIdx.y * kVoxTileY + ty;
-    const int z0 = blockIdx.z * kVoxPlanes, z1 = min(z0 + kVoxPlanes, nz);
+    const int z0 = blockIdx.z * planes, z1 = min(z0 + planes, nz);
     const bool in = x < nx && y < ny;
     const float4* G0 = reinterpret_cast<const float4*>(G);
     const float4* G1 = reinterpret_cast<const float4*>(G + 4 * nvox);
@@ -852,8 +853,10 @@ __global__ void __launch_bounds__(256) k_sum_copies(const float* __restrict__ co
 
 cudaError_t launch_channels_to_voxels(const float* dgrad, const int n[3], const float s[3], float* dvol,
                                       cudaStream_t st) {
-    const dim3 grid((n[0] + 31) / 32, (n[1] + kVoxTileY - 1) / kVoxTileY, (n[2] + kVoxPlanes - 1) / kVoxPlanes);
-    k_channels_to_voxels<<<grid, 256, 0, st>>>(dgrad, n[0], n[1], n[2], s[0], s[1], s[2], dvol);
+    const unsigned tx = (n[0] + 31) / 32, ty = (n[1] + kVoxTileY - 1) / kVoxTileY;
+    const int planes = march_planes((long long)tx * ty, n[2], 4, 12);
+    k_channels_to_voxels<<<dim3(tx, ty, (n[2] + planes - 1) / planes), 256, 0, st>>>(dgrad, n[0], n[1], n[2], s[0],
+                                                                                   s[1], s[2], planes, dvol);
     return cudaGetLastError();
 }
 
@@ -861,7 +864,7 @@ cudaError_t launch_sum_copies(const float* copies, int n_copies, int tf_w, int t
                               const double* dparams, float* out_params, cudaStream_t st) {
     const long long n = 4ll * tf_w * tf_h;
     const long long blocks = (n * ((n_copies + kCopiesPerThread - 1) / kCopiesPerThread) + 255) / 256;
-    k_sum_copies<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, st>>>(copies, n_copies, tf_w, tf_h,
+    k_sum_copies<<<(unsigned)(blocks < kSMs * 8 ? blocks : kSMs * 8), 256, 0, st>>>(copies, n_copies, tf_w, tf_h,
                                                                                dtf, dparams, out_params);
     return cudaGetLastError();
 }

@@ -44,7 +44,8 @@ constexpr int kGaussCol = 64;   // y / z passes: outputs per column, 32 columns 
 // each of which adds its taps in the order t = -R .. R with one fmaf each (one LDS per
 // output and tap bound these passes before: x / y / z pass of 256x256x176 at R = 12 56 /
 // 47 / 47 -> 21 / 26 / 26 us). kR > 0 is the radius known at compile time (the loop unrolls, weights
-// become constant operands); kR = 0 reads it from G.R.
+// become constant operands); kR = 0 reads it from G.R and keeps the kN values in a ring
+// of registers, so that a tap is one LDS, one constant load and kN fmaf.
 template <int kR, int kN, class At>
 __device__ __forceinline__ void gauss_taps(const At& at, const GaussParams& G, float acc[kN]) {
 #pragma unroll
@@ -58,11 +59,20 @@ __device__ __forceinline__ void gauss_taps(const At& at, const GaussParams& G, f
                 if (i - n >= 0 && i - n <= 2 * kR) acc[n] = fmaf(G.w[i - n], v, acc[n]);
         }
     } else {
-        for (int i = 0; i < kN + 2 * G.R; ++i) {
-            const float v = at(i);
+        const int last = 2 * G.R;
+        float v[kN];  // v[i % kN] = value i, i in [t, t + kN)
 #pragma unroll
-            for (int n = 0; n < kN; ++n)
-                if (i - n >= 0 && i - n <= 2 * G.R) acc[n] = fmaf(G.w[i - n], v, acc[n]);
+        for (int i = 0; i < kN; ++i) v[i] = at(i);
+        for (int t0 = 0; t0 <= last; t0 += kN) {
+#pragma unroll
+            for (int q = 0; q < kN; ++q) {
+                const int t = t0 + q;
+                if (t > last) break;
+                const float w = G.w[t];
+#pragma unroll
+                for (int n = 0; n < kN; ++n) acc[n] = fmaf(w, v[(q + n) % kN], acc[n]);
+                if (t < last) v[q] = at(t + kN);
+            }
         }
     }
 }
@@ -161,8 +171,10 @@ void gauss_passes(const float* in, float* out, float* tmp, const int n[3], const
 // reads the nine in-plane neighbours it needs and keeps those of the planes below and
 // above in registers: 9 shared reads and 1.3 global loads per voxel instead of 19 loads
 // (pass A of 256x256x176: 64 -> 36 us).
-// f(z, H) is called by every thread of the CTA for every plane.
-constexpr int kTileX = 32, kTileY = 8, kTileZ = 16;
+// emit(z, H) is called by every thread of the CTA for every plane.
+// A short volume gets shorter walks (march_planes): with 16 planes per CTA 42x41x62 had 48
+// CTAs, each a chain of 18 plane loads, and took 162 us for two scales (now 94).
+constexpr int kTileX = 32, kTileY = 8;
 struct PlaneTile {
     float v[2][kTileY + 2][kTileX + 2];
 };
@@ -282,13 +294,13 @@ __device__ __forceinline__ void eig3_sorted(const float H[6], float l[3]) {
 // Pass A of a scale: the maximum over voxels of S = ||H|| (block maxima folded
 // into smax with an integer atomicMax on the non-negative float bits).
 __global__ void __launch_bounds__(256) k_frangi_smax(const float* __restrict__ sm, int nx, int ny, int nz, float s2,
-                                                     float* __restrict__ smax) {
+                                                     int planes, float* __restrict__ smax) {
     __shared__ PlaneTile tile;
     const int x = blockIdx.x * kTileX + (threadIdx.x & 31), y = blockIdx.y * kTileY + (threadIdx.x >> 5);
     const bool in = x < nx && y < ny;
-    const int z0 = blockIdx.z * kTileZ;
+    const int z0 = blockIdx.z * planes;
     float S = 0.0f;
-    march_hessians(sm, nx, ny, nz, s2, z0, min(z0 + kTileZ, nz), tile, [&](int, const float H[6]) {
+    march_hessians(sm, nx, ny, nz, s2, z0, min(z0 + planes, nz), tile, [&](int, const float H[6]) {
         if (in) S = fmaxf(S, hessian_norm(H));
     });
 #pragma unroll
@@ -326,7 +338,8 @@ __device__ __forceinline__ float vessel_response(const float H[6], float c) {
 // is left is bound by the special-function pipe, five operations per rotation). The others leave V
 // as it is (V starts at zero and only grows).
 __global__ void __launch_bounds__(256) k_frangi_v(const float* __restrict__ sm, int nx, int ny, int nz, float s2,
-                                                  const float* __restrict__ smax, float* __restrict__ V) {
+                                                  int planes, const float* __restrict__ smax,
+                                                  float* __restrict__ V) {
     __shared__ PlaneTile tile;
     __shared__ float qh[6][512];
     __shared__ int qpos[512];  // z - z0 and thread of the queued voxel
@@ -334,7 +347,7 @@ __global__ void __launch_bounds__(256) k_frangi_v(const float* __restrict__ sm, 
     const int lane = threadIdx.x & 31;
     const int x = blockIdx.x * kTileX + lane, y = blockIdx.y * kTileY + (threadIdx.x >> 5);
     const bool in = x < nx && y < ny;
-    const int z0 = blockIdx.z * kTileZ;
+    const int z0 = blockIdx.z * planes;
     const float c = 0.5f * __ldg(smax);
     if (!(c > 0.0f)) return;
     if (threadIdx.x == 0) tail = 0;
@@ -348,7 +361,7 @@ __global__ void __launch_bounds__(256) k_frangi_v(const float* __restrict__ sm, 
             *o = fmaxf(*o, v);
         }
     };
-    march_hessians(sm, nx, ny, nz, s2, z0, min(z0 + kTileZ, nz), tile, [&](int z, const float H[6]) {
+    march_hessians(sm, nx, ny, nz, s2, z0, min(z0 + planes, nz), tile, [&](int z, const float H[6]) {
         const bool take = in && H[0] + H[1] + H[2] < 0.0f;
         const unsigned m = __ballot_sync(0xffffffffu, take);
         int at = 0;
@@ -390,7 +403,10 @@ cudaError_t launch_frangi(const float* norm, const int n[3], const float* sigmas
     cudaError_t e = cudaMemsetAsync(V, 0, sizeof(float) * nvox, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(smax, 0, sizeof(float) * n_sigmas, st);
     if (e != cudaSuccess) return e;
-    const dim3 grid((n[0] + kTileX - 1) / kTileX, (n[1] + kTileY - 1) / kTileY, (n[2] + kTileZ - 1) / kTileZ);
+    const unsigned tx = (n[0] + kTileX - 1) / kTileX, ty = (n[1] + kTileY - 1) / kTileY;
+    // at most 16 planes: more leave the last wave uneven
+    const int planes = march_planes((long long)tx * ty, n[2], 8, 16);
+    const dim3 grid(tx, ty, (n[2] + planes - 1) / planes);
     for (int si = 0; si < n_sigmas; ++si) {
         const double sg = sigmas[si];
         GaussParams G;
@@ -401,8 +417,8 @@ cudaError_t launch_frangi(const float* norm, const int n[3], const float* sigmas
         for (int i = 0; i <= 2 * G.R; ++i) G.w[i] = (float)(w[i] / sum);
         gauss_passes(norm, tmp_a, tmp_b, n, G, st);
         const float s2 = (float)(sg * sg);
-        k_frangi_smax<<<grid, 256, 0, st>>>(tmp_a, n[0], n[1], n[2], s2, smax + si);
-        k_frangi_v<<<grid, 256, 0, st>>>(tmp_a, n[0], n[1], n[2], s2, smax + si, V);
+        k_frangi_smax<<<grid, 256, 0, st>>>(tmp_a, n[0], n[1], n[2], s2, planes, smax + si);
+        k_frangi_v<<<grid, 256, 0, st>>>(tmp_a, n[0], n[1], n[2], s2, planes, smax + si, V);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

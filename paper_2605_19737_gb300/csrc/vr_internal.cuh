@@ -90,6 +90,15 @@ inline SkipStore skip_store(uint8_t* p, const int n[3]) {
     s.block_dist = reinterpret_cast<uint4*>(p);
     return s;
 }
+constexpr int kSMs = 152;
+// Planes that a CTA of a kernel marching along z walks, `columns` CTAs covering a plane:
+// as many as keep `resident` CTAs for every SM, from 1 to `most`. Long walks read the two
+// border planes once for more planes of output; but a walk is a serial chain of plane
+// loads, so a launch that does not fill the chip takes the time of one walk.
+inline int march_planes(long long columns, int nz, int resident, int most) {
+    const long long p = columns * nz / ((long long)kSMs * resident);
+    return p < 1 ? 1 : p > most ? most : (int)p;
+}
 // Cells of the min/max grid per row, padded to whole warps.
 __host__ __device__ __forceinline__ int cellq_pitch(int nx) { return (nx - 1 + 31) & ~31; }
 inline size_t cellq_cells(const int n[3]) { return (size_t)cellq_pitch(n[0]) * (n[1] - 1) * (n[2] - 1); }

@@ -83,13 +83,13 @@ __device__ __forceinline__ int median_of_rows(const int L[9], const int M[9], co
 // comparisons took 478 us for 181x217x181, this 76 us.
 // With 14 or more NaNs among the 27 there is no 14th smallest number: the result is then
 // the (-1, -1, -1) neighbour.
-constexpr int kMedRows = 4, kMedPlanes = 16;
+constexpr int kMedRows = 4;
 __global__ void __launch_bounds__(128) k_median3(const float* __restrict__ in, float* __restrict__ out, int nx, int ny,
-                                                 int nz) {
+                                                 int nz, int planes) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int x = blockIdx.x * 30 - 1 + lane;
     const int y0 = (blockIdx.y * 4 + wid) * kMedRows;
-    const int z0 = blockIdx.z * kMedPlanes, z1 = min(z0 + kMedPlanes, nz);
+    const int z0 = blockIdx.z * planes, z1 = min(z0 + planes, nz);
     if (y0 >= ny) return;
     const long long plane = (long long)nx * ny;
     int off[kMedRows + 2];  // clamped rows, from the start of a plane
@@ -157,8 +157,9 @@ __global__ void __launch_bounds__(128) k_median3(const float* __restrict__ in, f
 }  // namespace
 
 cudaError_t launch_median3(const float* in, float* out, const int n[3], cudaStream_t st) {
-    dim3 grid((n[0] + 29) / 30, (n[1] + 4 * kMedRows - 1) / (4 * kMedRows), (n[2] + kMedPlanes - 1) / kMedPlanes);
-    k_median3<<<grid, 128, 0, st>>>(in, out, n[0], n[1], n[2]);
+    const unsigned tx = (n[0] + 29) / 30, ty = (n[1] + 4 * kMedRows - 1) / (4 * kMedRows);
+    const int planes = march_planes((long long)tx * ty, n[2], 8, 16);
+    k_median3<<<dim3(tx, ty, (n[2] + planes - 1) / planes), 128, 0, st>>>(in, out, n[0], n[1], n[2], planes);
     return cudaGetLastError();
 }
 

@@ -16,7 +16,6 @@ namespace vr {
 namespace {
 
 constexpr int kReduceThreads = 256;
-constexpr int kSMs = 152;
 
 __device__ __forceinline__ void warp_minmax(float& lo, float& hi) {
 #pragma unroll
