@@ -345,6 +345,7 @@ void fill_launch(RenderLaunch& L, const Volume* v, int W, int H, int skip) {
     }
     L.vol.bs = v->bs;
     L.vol.der_stride = (int)der_brick_floats(v->bs);
+    L.vol.der = der_layout(v->bs);
     L.vol.bricks = v->d_bricks;
     L.vol.vbricks = (v->tp.tf_mode == 2) ? v->d_vbricks : nullptr;
     L.vol.dbricks = v->d_dbricks;

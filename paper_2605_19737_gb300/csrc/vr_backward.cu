@@ -62,12 +62,13 @@ __device__ __forceinline__ void eval_field(const VolumeDev& v, const TissueDev& 
                                            float fld[10]) {
     if (kDerived) {
         const float4* brick = derived_brick<kBS>(v, bi);
-        const int m = (1 << (kBS ? kBS : v.bs)) - 1, E = m + 2;
-        derived_channels<true, 0, 4>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
+        const int m = (1 << (kBS ? kBS : v.bs)) - 1;
+        const DerLayout d = kBS ? der_layout(kBS) : v.der;
+        derived_channels<kBS == 2, 0, 4>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
         if (kHessian)
-            derived_channels<true, 4, 6>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
+            derived_channels<kBS == 2, 4, 6>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
         else
-            load_hessian<true>(tp, brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f, fld);
+            load_hessian<kBS == 2>(tp, brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f, fld);
     } else {
         field_eval(GLoad{v.bricks + sbi * kBrickVox}, base, f[0], f[1], f[2], fld);
         scale_field(fld, is);
@@ -293,11 +294,12 @@ __device__ __forceinline__ void sweep_eval(const VolumeDev& v, const TissueDev& 
         // a curvature term only dL/dgamma needs -- and not at a zero opacity
         // entry (dL/dw = 0 there, and w = 1 whatever kappa)
         const float4* brick = derived_brick<kBS>(v, bi);
-        const int m = (1 << bs) - 1, E = m + 2;
-        derived_channels<true, 0, 4>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
+        const int m = (1 << bs) - 1;
+        const DerLayout d = kBS ? der_layout(kBS) : v.der;
+        derived_channels<kBS == 2, 0, 4>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
         optics_tf<k2D ? 2 : 1>(fld, vval, tp, tf, inv_gmax, so);
         if (!kNoHessian && so.c.w != 0.0f) {
-            derived_channels<true, 4, 6>(brick, E, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
+            derived_channels<kBS == 2, 4, 6>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
         } else {
 #pragma unroll
             for (int q = 4; q < 10; ++q) fld[q] = 0.0f;
@@ -529,7 +531,7 @@ __global__ void __launch_bounds__(128, kTfOnly && !k2D ? 5 : 4) k_render_backwar
 // its own sample, and applies its sample's adjoint. Time falls with the serial chain
 // (backward_lanes has the figures). 3 CTAs per SM (168 registers) where the field's
 // adjoint is wanted: up to 10 % faster than 4 with their spills; 4 for the table alone.
-template <bool kLazyHessian, bool kNoHessian, bool kTfOnly, bool k2D>
+template <bool kLazyHessian, bool kNoHessian, bool kTfOnly, bool k2D, int kBS>
 __global__ void __launch_bounds__(128, kTfOnly ? 4 : 3) k_backward_lanes(const __grid_constant__ BackwardLaunch B) {
     const RenderLaunch& L = B.r;
     const size_t ncell = (size_t)L.tp.tf_w * L.tp.tf_h * kTfCellFloats;
@@ -578,7 +580,7 @@ __global__ void __launch_bounds__(128, kTfOnly ? 4 : 3) k_backward_lanes(const _
                                            (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
                                            (unsigned)i0[2] <= (unsigned)(v.n[2] - 2));
             if (on)
-                sweep_eval<true, kLazyHessian, kNoHessian, k2D, 0>(v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld, so);
+                sweep_eval<true, kLazyHessian, kNoHessian, k2D, kBS>(v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld, so);
         }
         const unsigned shaded = __ballot_sync(0xffffffffu, on && so.c.w != 0.0f);
         // the recurrences over the samples kb, kb - 1, ...; a sample of zero opacity entry
@@ -896,19 +898,28 @@ void launch_backward_table(const BackwardLaunch& B, dim3 grid, cudaStream_t st) 
     }
 }
 
-template <bool k2D>
-void launch_backward_lanes(const BackwardLaunch& B, dim3 grid, cudaStream_t st) {
+template <bool k2D, int kBS>
+void launch_backward_lanes_bs(const BackwardLaunch& B, dim3 grid, cudaStream_t st) {
     const bool tf_only = !B.dparams && !B.dvol && !B.dgrad;
     if (B.r.tp.gk == 0.0f && tf_only)
-        k_backward_lanes<true, true, true, k2D><<<grid, 128, 0, st>>>(B);
+        k_backward_lanes<true, true, true, k2D, kBS><<<grid, 128, 0, st>>>(B);
     else if (B.r.tp.gk == 0.0f && !B.dparams)
-        k_backward_lanes<true, true, false, k2D><<<grid, 128, 0, st>>>(B);
+        k_backward_lanes<true, true, false, k2D, kBS><<<grid, 128, 0, st>>>(B);
     else if (B.r.tp.gk == 0.0f)
-        k_backward_lanes<true, false, false, k2D><<<grid, 128, 0, st>>>(B);
+        k_backward_lanes<true, false, false, k2D, kBS><<<grid, 128, 0, st>>>(B);
     else if (tf_only)
-        k_backward_lanes<false, false, true, k2D><<<grid, 128, 0, st>>>(B);
+        k_backward_lanes<false, false, true, k2D, kBS><<<grid, 128, 0, st>>>(B);
     else
-        k_backward_lanes<false, false, false, k2D><<<grid, 128, 0, st>>>(B);
+        k_backward_lanes<false, false, false, k2D, kBS><<<grid, 128, 0, st>>>(B);
+}
+
+template <bool k2D>
+void launch_backward_lanes(const BackwardLaunch& B, dim3 grid, cudaStream_t st) {
+    switch (B.r.vol.bs) {
+        case 2: launch_backward_lanes_bs<k2D, 2>(B, grid, st); break;
+        case 4: launch_backward_lanes_bs<k2D, 4>(B, grid, st); break;
+        default: launch_backward_lanes_bs<k2D, 3>(B, grid, st); break;
+    }
 }
 
 // Lanes per ray of a backward launch with that many rays. One lane per ray fills the

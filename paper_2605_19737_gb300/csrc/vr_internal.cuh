@@ -29,17 +29,46 @@ constexpr int kBrickBytes = kBrickVox * 4;         // 6912 bytes
 constexpr int kMaxCamsPerLaunch = 64;
 
 // Derived bricks: per skip brick the (B+1)^3 corner voxels [Bb, Bb+B] (clamped) of
-// its cells, each as 12 floats = I, gx, gy, gz, Hxx, Hyy, Hzz, Hxy, Hxz, Hyz (mm
-// units), 0, 0: the voxel-wise derivatives of Sec. 2.3, three 16-byte loads per
-// corner (B = 8: 9^3 corners, 34,992 B).
+// its cells, the voxel-wise derivatives of Sec. 2.3 in mm units: (I, gx, gy, gz), (Hxx, Hyy,
+// Hzz, Hxy) and (Hxz, Hyz) of every corner, read by a 16-, a 16- and an 8-byte load. A
+// brick's place in the store is 12 floats per corner (B = 8: 9^3 corners, 34,992 B).
 constexpr int kDerFloats = 12;
 constexpr int kMinBrickShift = 2, kMaxBrickShift = 4;  // skip bricks of 4^3 .. 16^3 cells
 
-__host__ __device__ __forceinline__ int der_edge(int bs) { return (1 << bs) + 1; }
-__host__ __device__ __forceinline__ long long der_brick_floats(int bs) {
+__host__ __device__ __forceinline__ constexpr int der_edge(int bs) { return (1 << bs) + 1; }
+__host__ __device__ __forceinline__ constexpr long long der_brick_floats(int bs) {
     const long long e = der_edge(bs);
     return e * e * e * kDerFloats;
 }
+
+// Where a corner's three pieces lie in its brick. The raymarch kernels are bound by the L1
+// data stage (68-70 % of its passes in the 540p frame and its backward): the 16-byte loads
+// of a quarter warp go through in one pass only if they meet different 16-byte columns of
+// the 128-byte lines. In records of 48 bytes in rows of B + 1, a corner's neighbours along
+// x, y and z all lie 3 columns on; a load took 5.1 passes (4 without conflicts). For B = 8
+// and 16 the pieces are therefore three planes, and what they leave of the brick's place
+// pads their rows and slices so that neighbours lie x 1, y 2, z 4 columns on: the corners
+// of a cell, or one corner of eight neighbouring cells, on eight columns. Without a
+// curvature term only the first plane is read, 16 of 16 bytes instead of 16 of 48.
+// Measured, records -> planes: 1080p frame of the 181x217x181 head 1.88 -> 1.82 ms, its
+// 540p at B = 16 0.84 -> 0.77, 32 views without curvature 8.88 -> 8.27, fit step of 8 views
+// 6.90 -> 6.07, 1080p gradient 11.55 -> 11.41. B = 4 has no room for the padding (planes:
+// 700x600 0.78 -> 0.81 ms) and keeps the records. Kernels take the layout of a fixed B: as
+// run-time values it cost the launches of several lanes per ray 3 %.
+struct DerLayout {
+    int row, slice;  // records to a corner's neighbours along y and z
+    int rec, m;      // float4 per record, and from its first to its second piece
+    int t, trec;     // float2 from the brick's start to record 0's third piece, and per record
+};
+__host__ __device__ __forceinline__ constexpr DerLayout der_planes(int row, int slice, int B) {
+    const int n = B * (slice + row + 1) + 1;  // records of a padded plane
+    return DerLayout{row, slice, 1, n, 4 * n, 1};
+}
+__host__ __device__ __forceinline__ constexpr DerLayout der_layout(int bs) {
+    return bs == 2 ? DerLayout{5, 25, 3, 1, 4, 6} : bs == 3 ? der_planes(10, 92, 8) : der_planes(18, 308, 16);
+}
+static_assert(10 * der_layout(3).m <= der_brick_floats(3) && 10 * der_layout(4).m <= der_brick_floats(4),
+              "the planes fit a brick's place");
 
 // Skip field: per interpolation cell one byte, the Chebyshev distance in cells to the
 // nearest cell that may hold opacity under the current transfer function, capped (0: the
@@ -151,6 +180,7 @@ struct VolumeDev {
     int nsb[3];     // storage bricks per axis = ceil((n-1)/8)
     int bs;         // log2 B, cells per skip-brick edge
     int der_stride; // floats per derived brick, der_brick_floats(bs)
+    DerLayout der;  // der_layout(bs)
     float s[3];     // spacing (mm)
     const float* bricks;     // storage bricks x kBrickVox
     const float* vbricks;    // vesselness storage bricks (same layout) or nullptr

@@ -54,14 +54,15 @@ __device__ __forceinline__ bool eval_sample(const VolumeDev& v, const TissueDev&
     float fld[10];
     if (kDerived) {
         // derived brick of the cell, and the cell's place in it; I and the gradient (one
-        // 16-byte load per corner), the Hessian (two), then the transfer function
-        const int bs = kBS ? kBS : v.bs, B = 1 << bs, E = B + 1;
+        // load per corner), the Hessian (two), then the transfer function
+        const int bs = kBS ? kBS : v.bs, B = 1 << bs;
+        const DerLayout dl = kBS ? der_layout(kBS) : v.der;
         const int bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
         const float4* dbrick = reinterpret_cast<const float4*>(
             v.dbricks + (size_t)(unsigned)brick_index(v, bc) * (unsigned)(kBS ? der_brick_floats(kBS) : v.der_stride));
         const int lx = i0[0] & (B - 1), ly = i0[1] & (B - 1), lz = i0[2] & (B - 1);
-        derived_channels<false, 0, 4>(dbrick, E, lx, ly, lz, f[0], f[1], f[2], fld);
-        load_hessian<false>(tp, dbrick, E, lx, ly, lz, f, fld);
+        derived_channels<false, 0, 4>(dbrick, dl, lx, ly, lz, f[0], f[1], f[2], fld);
+        load_hessian<false>(tp, dbrick, dl, lx, ly, lz, f, fld);
         SampleOptics o;
         optics_tf(fld, vval, tp, tf, inv_gmax, o);
         if (o.c.w == 0.0f) return false;
@@ -217,7 +218,7 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
 // For launches with too few rays to fill the chip the time is the serial chain of one
 // ray, and this shortens it by almost G (64^3 at 128x128: 90 -> 29 us at G = 8); a
 // filled chip gains nothing and pays the shuffles (4 per sample slot).
-template <bool kDerived, bool kState, int G>
+template <bool kDerived, bool kState, int G, int kBS>
 __device__ __forceinline__ void march_lanes(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
                                             const RayDev& r, int skip, float inv_gmax, const float is[3],
                                             float4& out, int* klast_out, float* t_last) {
@@ -251,7 +252,7 @@ __device__ __forceinline__ void march_lanes(const VolumeDev& v, const TissueDev&
         } else {
             float alpha = 0.0f, col[3] = {0.f, 0.f, 0.f};
             bool shaded = false;
-            if (adv == 0u) shaded = eval_sample<kDerived, 0>(v, tp, tf, U, i0, r.dir, inv_gmax, is, alpha, col);
+            if (adv == 0u) shaded = eval_sample<kDerived, kBS>(v, tp, tf, U, i0, r.dir, inv_gmax, is, alpha, col);
             const unsigned live = __ballot_sync(0xffffffffu, shaded);
 #pragma unroll
             for (int h = 0; h < G; ++h) {

@@ -61,9 +61,9 @@ __global__ void __launch_bounds__(kState ? 128 : 256, kDerived ? (kState ? 7 : 4
 // warp covers pw x ph rays of G lanes, a CTA four warps side by side. The fewer the rays,
 // the more registers pay (more loads in flight per lane): 128 at 8 and 16 lanes (128^2 of
 // the 181x217x181 head 142 -> 127 us against 80), 80 at 2 and 4 (256^2 121 -> 113 us
-// against 128); 64 were slower everywhere the chip is not full. The skip-brick size stays
-// a run-time value here: at latency-bound sizes its index arithmetic is hidden.
-template <bool kDerived, bool kState, int G>
+// against 128); 64 were slower everywhere the chip is not full. kBS: log2 of the skip-brick
+// edge (any value without derived bricks).
+template <bool kDerived, bool kState, int G, int kBS>
 __global__ void __launch_bounds__(128, kDerived && G < 8 ? 6 : 4) k_render_lanes(const __grid_constant__ RenderLaunch L) {
     const int w = threadIdx.x >> 5;
     const int ray = (threadIdx.x & 31) / G, pw = L.packet_w;
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(128, kDerived && G < 8 ? 6 : 4) k_render_lanes
     float4 px;
     int kl = -1;
     float tl = 1.0f;
-    march_lanes<kDerived, kState, G>(v, L.tp, reinterpret_cast<const float4*>(L.tf), r, L.skip, inv_gmax, is, px, &kl,
+    march_lanes<kDerived, kState, G, kBS>(v, L.tp, reinterpret_cast<const float4*>(L.tf), r, L.skip, inv_gmax, is, px, &kl,
                                      &tl);
     if (inside && (threadIdx.x & (G - 1)) == 0) {
         const long long pix = ((long long)(L.cam_offset + cam) * L.H + j) * L.W + i;
@@ -89,13 +89,22 @@ __global__ void __launch_bounds__(128, kDerived && G < 8 ? 6 : 4) k_render_lanes
     }
 }
 
-template <bool kDerived, bool kState>
+template <bool kDerived, bool kState, int kBS>
 void launch_lanes(const RenderLaunch& L, dim3 grid, cudaStream_t st) {
     switch (L.lanes) {
-        case 2: k_render_lanes<kDerived, kState, 2><<<grid, 128, 0, st>>>(L); break;
-        case 4: k_render_lanes<kDerived, kState, 4><<<grid, 128, 0, st>>>(L); break;
-        case 8: k_render_lanes<kDerived, kState, 8><<<grid, 128, 0, st>>>(L); break;
-        default: k_render_lanes<kDerived, kState, 16><<<grid, 128, 0, st>>>(L); break;
+        case 2: k_render_lanes<kDerived, kState, 2, kBS><<<grid, 128, 0, st>>>(L); break;
+        case 4: k_render_lanes<kDerived, kState, 4, kBS><<<grid, 128, 0, st>>>(L); break;
+        case 8: k_render_lanes<kDerived, kState, 8, kBS><<<grid, 128, 0, st>>>(L); break;
+        default: k_render_lanes<kDerived, kState, 16, kBS><<<grid, 128, 0, st>>>(L); break;
+    }
+}
+
+template <bool kState>
+void launch_lanes_derived(const RenderLaunch& L, dim3 grid, cudaStream_t st) {
+    switch (L.vol.bs) {
+        case 2: launch_lanes<true, kState, 2>(L, grid, st); break;
+        case 4: launch_lanes<true, kState, 4>(L, grid, st); break;
+        default: launch_lanes<true, kState, 3>(L, grid, st); break;
     }
 }
 
@@ -147,9 +156,9 @@ cudaError_t launch_render_gather(const RenderLaunch& L0, int warps, cudaStream_t
         L.packet_h = rays / L.packet_w;
         dim3 grid((L.W + 4 * L.packet_w - 1) / (4 * L.packet_w), (L.H + L.packet_h - 1) / L.packet_h, L.n_cams);
         if (L.vol.dbricks)
-            L.ray_state ? launch_lanes<true, true>(L, grid, st) : launch_lanes<true, false>(L, grid, st);
+            L.ray_state ? launch_lanes_derived<true>(L, grid, st) : launch_lanes_derived<false>(L, grid, st);
         else
-            L.ray_state ? launch_lanes<false, true>(L, grid, st) : launch_lanes<false, false>(L, grid, st);
+            L.ray_state ? launch_lanes<false, true, 3>(L, grid, st) : launch_lanes<false, false, 3>(L, grid, st);
         return cudaGetLastError();
     }
     // the state-recording kernels are built for CTAs of at most 4 warps (72 registers,
@@ -481,9 +490,9 @@ __global__ void __launch_bounds__(256, 3) k_render_staged_derived(const __grid_c
                     if (!done_sample) {
                         ++nip;
                         float fld[10];
-                        derived_channels_smem<0, 4>(sbrick, E, lx, ly, lz, f[0], f[1], f[2], fld);
+                        derived_channels_smem<0, 4>(sbrick, der_layout(kBS), lx, ly, lz, f[0], f[1], f[2], fld);
                         if (tp.gk != 0.0f) {
-                            derived_channels_smem<4, 6>(sbrick, E, lx, ly, lz, f[0], f[1], f[2], fld + 4);
+                            derived_channels_smem<4, 6>(sbrick, der_layout(kBS), lx, ly, lz, f[0], f[1], f[2], fld + 4);
                         } else {
 #pragma unroll
                             for (int q = 4; q < 10; ++q) fld[q] = 0.0f;

@@ -209,24 +209,30 @@ __device__ __forceinline__ void field_eval(const Load& load, int base, float fx,
 // Sample field from derived bricks: trilinear interpolation of voxel-wise channels
 // (already in mm units) over the cell's 8 corners; (lx, ly, lz) is the cell's corner
 // voxel (i0, j0, k0) local to the brick's E^3 block (E = B + 1 corners per edge). Channels [kFirst, kFirst +
-// kCount): kFirst = 0, kCount = 4 reads (I, gx, gy, gz) -- the first 16-byte vector
-// of each corner; kFirst = 4, kCount = 6 the Hessian (Hxx, Hyy, Hzz, Hxy, Hxz, Hyz)
+// kCount): kFirst = 0, kCount = 4 reads (I, gx, gy, gz) -- the first piece;
+// kFirst = 4, kCount = 6 the Hessian (Hxx, Hyy, Hzz, Hxy, Hxz, Hyz)
 // -- the second and third. Each channel sums its 8 corners in the same order, so
 // split and whole evaluations agree bit for bit.
 // kParity: the 8 corner loads are issued in order of the corners' parity (even/odd
 // voxel index per axis) rather than of their offset from the cell, so that lanes in
-// neighbouring cells read the same record in the same instruction and their loads
-// coalesce; each lane picks the matching weight. That costs ~30 instructions per
-// sample; measured, the adjoint sweep gains 3 %, the 1080p forward frame loses
-// 1.3 % (512^2 views gain 3 %). The forward kernels keep the offset order, so that
-// single-view and batched renders stay bit-identical; the adjoint uses parity order.
-// Read-only 16-byte load that asks L2 to fetch the surrounding 256 bytes from DRAM
-// (neighbouring corner records of the same brick row).
+// neighbouring cells read the same record in the same instruction; each lane picks the
+// matching weight, ~30 instructions per sample. The adjoint sweep gained 3 % by it while
+// neighbouring corners shared L1 columns, and still takes it with skip bricks of edge 4
+//; with the padded planes it costs 1-9 % (fit step of 8 views 6.08 ms in
+// offset order, 6.64 in parity order). The forward kernels keep the offset order
+// everywhere, so that single-view and batched renders stay bit-identical.
+// Read-only 16- and 8-byte loads that ask L2 to fetch the surrounding 256 bytes from DRAM
+// (neighbouring corner records of the same brick rows).
 __device__ __forceinline__ float4 ldg_l2_256(const float4* p) {
     float4 v;
     asm("ld.global.nc.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];"
         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
         : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ldg_l2_256(const float2* p) {
+    float2 v;
+    asm("ld.global.nc.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
     return v;
 }
 
@@ -281,10 +287,14 @@ __device__ __forceinline__ void corner_weights(float fx, float fy, float fz, flo
 }
 
 template <bool kParity, int kFirst, int kCount>
-__device__ __forceinline__ void derived_channels(const float4* __restrict__ brick, int E, int lx, int ly, int lz,
+__device__ __forceinline__ void derived_channels(const float4* __restrict__ brick, const DerLayout& d, int lx, int ly, int lz,
                                                  float fx, float fy, float fz, float* out) {
     const int px = kParity ? lx & 1 : 0, py = kParity ? ly & 1 : 0, pz = kParity ? lz & 1 : 0;
-    const int base = (lz * E + ly) * E + lx;
+    const int c0 = lz * d.slice + ly * d.row + lx;
+    const float4* p0 = brick + d.rec * c0;
+    // (in the records the third piece is reached from the first: one address)
+    const float2* t0 = d.rec == 3 ? reinterpret_cast<const float2*>(p0) + 4
+                                  : reinterpret_cast<const float2*>(brick) + (d.t + d.trec * c0);
     float wo[8];
     if (!kParity) corner_weights(fx, fy, fz, wo);
 #pragma unroll
@@ -296,14 +306,15 @@ __device__ __forceinline__ void derived_channels(const float4* __restrict__ bric
         const int dx = px ^ (c & 1), dy = py ^ ((c >> 1) & 1), dz = pz ^ ((c >> 2) & 1);
         const float w =
             kParity ? (dx ? fx : 1.0f - fx) * (dy ? fy : 1.0f - fy) * (dz ? fz : 1.0f - fz) : wo[c];
-        const float4* p = brick + 3 * (base + (dz * E + dy) * E + dx);
+        const int r = dz * d.slice + dy * d.row + dx;
         if (kFirst == 0) {
-            const float4 a = ldg_l2_256(p);
+            const float4 a = ldg_l2_256(p0 + d.rec * r);
             fma2(w, a.x, a.y, out[0], out[1]);
             fma2(w, a.z, a.w, out[2], out[3]);
         }
         if (kFirst + kCount > 4) {
-            const float4 m = ldg_l2_256(p + 1), t = ldg_l2_256(p + 2);
+            const float4 m = ldg_l2_256(p0 + d.m + d.rec * r);
+            const float2 t = ldg_l2_256(t0 + d.trec * r);
             float* o = out + (4 - kFirst);
             fma2(w, m.x, m.y, o[0], o[1]);
             fma2(w, m.z, m.w, o[2], o[3]);
@@ -314,23 +325,24 @@ __device__ __forceinline__ void derived_channels(const float4* __restrict__ bric
 
 // derived_channels over a derived brick staged in shared memory (plain loads).
 template <int kFirst, int kCount>
-__device__ __forceinline__ void derived_channels_smem(const float4* brick, int E, int lx, int ly, int lz, float fx,
+__device__ __forceinline__ void derived_channels_smem(const float4* brick, const DerLayout& d, int lx, int ly, int lz, float fx,
                                                       float fy, float fz, float* out) {
-    const int base = (lz * E + ly) * E + lx;
 #pragma unroll
     for (int q = 0; q < kCount; ++q) out[q] = 0.0f;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         const int dx = c & 1, dy = (c >> 1) & 1, dz = (c >> 2) & 1;
         const float w = (dx ? fx : 1.0f - fx) * (dy ? fy : 1.0f - fy) * (dz ? fz : 1.0f - fz);
-        const float4* p = brick + 3 * (base + (dz * E + dy) * E + dx);
+        const int r = (lz + dz) * d.slice + (ly + dy) * d.row + lx + dx;
+        const float4* p = brick + d.rec * r;
         if (kFirst == 0) {
             const float4 a = p[0];
             fma2(w, a.x, a.y, out[0], out[1]);
             fma2(w, a.z, a.w, out[2], out[3]);
         }
         if (kFirst + kCount > 4) {
-            const float4 m = p[1], t = p[2];
+            const float4 m = p[d.m];
+            const float2 t = reinterpret_cast<const float2*>(brick)[d.t + d.trec * r];
             float* o = out + (4 - kFirst);
             fma2(w, m.x, m.y, o[0], o[1]);
             fma2(w, m.z, m.w, o[2], o[3]);
@@ -344,10 +356,10 @@ __device__ __forceinline__ void derived_channels_smem(const float4* brick, int E
 // fma(0, kappa, 1) = 1 for any kappa, and every Hessian gradient carries the factor
 // gamma), so results are unchanged and its 16 loads per sample are saved.
 template <bool kParity>
-__device__ __forceinline__ void load_hessian(const TissueDev& tp, const float4* __restrict__ brick, int E, int lx,
+__device__ __forceinline__ void load_hessian(const TissueDev& tp, const float4* __restrict__ brick, const DerLayout& d, int lx,
                                              int ly, int lz, const float f[3], float fld[10]) {
     if (tp.gk != 0.0f) {
-        derived_channels<kParity, 4, 6>(brick, E, lx, ly, lz, f[0], f[1], f[2], fld + 4);
+        derived_channels<kParity, 4, 6>(brick, d, lx, ly, lz, f[0], f[1], f[2], fld + 4);
     } else {
 #pragma unroll
         for (int q = 4; q < 10; ++q) fld[q] = 0.0f;

@@ -164,12 +164,13 @@ __global__ void __launch_bounds__(256) k_make_bricks(const float* __restrict__ n
 // One CTA per skip brick: the voxel-wise intensity, central-difference gradient
 // (Eq. 2) and second/mixed differences (Sec. 2.3) of the brick's (B+1)^3 corner
 // voxels, with clamp-to-edge neighbours, divided by the spacing -- the per-voxel
-// morphology the paper's compute shader produces, laid out for 16-byte loads.
-// A warp passes its 32 corners' records (48 bytes each) through shared memory and stores
-// them as 1536 consecutive bytes: stored straight from the threads that computed them, a
-// warp's store wrote 16 of every 48 bytes
-// (181x217x181 at B = 8, 518 MB: 136 -> 116 us; 256x256x176, 788 MB: 213 -> 192 us). kBS
-// (log2 B) at compile time keeps the divisions by the edges out.
+// morphology the paper's compute shader produces, laid out as der_layout says. Stores are
+// whole lines: in the planes a warp writes 32 consecutive pieces, the padding (zeros)
+// among them (without it the rows' last sectors are half written: 181x217x181 at B = 8,
+// whole precompute 213 us, with it 145; as records 159); the 48-byte records of B = 4 go through shared
+// memory (stored straight from the threads that computed them, a warp's store wrote 16 of
+// every 48 bytes: 322 us, staged 267). kBS (log2 B) at compile time keeps the divisions by
+// the edges out.
 template <int kBS>
 __global__ void __launch_bounds__(256) k_make_derived(const float* __restrict__ norm, int nx, int ny, int nz, int nbx,
                                                       int nby, float hx, float hy, float hz, float* __restrict__ out) {
@@ -177,7 +178,8 @@ __global__ void __launch_bounds__(256) k_make_derived(const float* __restrict__ 
     // clamped to the volume (so neighbour i +- 1 of a corner is tile entry t +- 1)
     constexpr int B = 1 << kBS, E = B + 1, T = B + 3;
     __shared__ float tile[T * T * T];
-    __shared__ float4 stage[8][96];
+    constexpr bool kRecords = kBS == 2;
+    __shared__ float4 stage[kRecords ? 8 : 1][96];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int b = blockIdx.x;
     const int bx = b % nbx, by = (b / nbx) % nby, bz = b / (nbx * nby);
@@ -188,17 +190,21 @@ __global__ void __launch_bounds__(256) k_make_derived(const float* __restrict__ 
         tile[e] = __ldg(norm + ((long long)z * ny + y) * nx + x);
     }
     __syncthreads();
+    constexpr DerLayout d = der_layout(kBS);
     float4* dst = reinterpret_cast<float4*>(out + (size_t)(unsigned)b * (unsigned)der_brick_floats(kBS));
-    for (int e0 = wid * 32; e0 < E * E * E; e0 += 256) {
-        const int e = min(e0 + lane, E * E * E - 1);
-        const int lx = e % E, ly = (e / E) % E, lz = e / (E * E);
+    constexpr int R = kRecords ? E : d.row, S = kRecords ? E * E : d.slice, N = kRecords ? E * E * E : d.m;
+    for (int e0 = wid * 32; e0 < N; e0 += 256) {
+        const int e = min(e0 + lane, N - 1);
+        const int lz = e / S, ly = min(e % S / R, E - 1), lx = min(e % S % R, E - 1);
+        const bool pad = lx + R * ly + S * lz != e;
         // the corner voxel (clamped as in the per-voxel definition) in tile coordinates
         const int tx = min(B * bx + lx, nx - 1) - x0, ty = min(B * by + ly, ny - 1) - y0,
                   tz = min(B * bz + lz, nz - 1) - z0;
         const float* t0 = tile + (tz * T + ty) * T + tx;
         auto at = [&](int dx, int dy, int dz) { return t0[(dz * T + dy) * T + dx]; };
         const float c = at(0, 0, 0), c2 = 2.0f * c;
-        float4 a, m, t;
+        float4 a, m;
+        float2 t;
         a.x = c;
         a.y = (at(1, 0, 0) - at(-1, 0, 0)) * (0.5f * hx);
         a.z = (at(0, 1, 0) - at(0, -1, 0)) * (0.5f * hy);
@@ -209,18 +215,23 @@ __global__ void __launch_bounds__(256) k_make_derived(const float* __restrict__ 
         m.w = ((at(1, 1, 0) - at(1, -1, 0)) - (at(-1, 1, 0) - at(-1, -1, 0))) * (0.25f * hx * hy);
         t.x = ((at(1, 0, 1) - at(1, 0, -1)) - (at(-1, 0, 1) - at(-1, 0, -1))) * (0.25f * hx * hz);
         t.y = ((at(0, 1, 1) - at(0, 1, -1)) - (at(0, -1, 1) - at(0, -1, -1))) * (0.25f * hy * hz);
-        t.z = 0.0f;
-        t.w = 0.0f;
-        float4* sp = stage[wid];
-        sp[3 * lane] = a;
-        sp[3 * lane + 1] = m;
-        sp[3 * lane + 2] = t;
-        __syncwarp();
-        const int left = 3 * (E * E * E - e0);  // pieces from e0 on
+        if (kRecords) {
+            float4* sp = stage[kRecords ? wid : 0];
+            sp[3 * lane] = a;
+            sp[3 * lane + 1] = m;
+            sp[3 * lane + 2] = make_float4(t.x, t.y, 0.0f, 0.0f);
+            __syncwarp();
+            const int left = 3 * (N - e0);  // pieces from e0 on
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (lane + 32 * q < left) dst[3 * e0 + lane + 32 * q] = sp[lane + 32 * q];
-        __syncwarp();
+            for (int q = 0; q < 3; ++q)
+                if (lane + 32 * q < left) dst[3 * e0 + lane + 32 * q] = sp[lane + 32 * q];
+            __syncwarp();
+        } else if (e0 + lane < N) {
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            dst[e] = pad ? zero : a;
+            dst[d.m + e] = pad ? zero : m;
+            reinterpret_cast<float2*>(dst)[d.t + e] = pad ? make_float2(0.f, 0.f) : t;
+        }
     }
 }
 
