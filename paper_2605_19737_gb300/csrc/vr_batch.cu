@@ -44,12 +44,20 @@ __device__ __forceinline__ void batch_body(const BatchLaunch& B) {
         float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
         unsigned dense = 0, evald = 0, shaded = 0, interp = 0;
         if (!hit) r.ns = 0;
-        if (kAllDerived || v.dbricks)
-            march_gather<true, false, kCount, kBS>(v, vw.tp, reinterpret_cast<const float4*>(vw.tf), r, B.skip,
-                                                       inv_gmax, is, out, dense, evald, shaded, interp);
-        else
-            march_gather<false, false, kCount, kBS>(v, vw.tp, reinterpret_cast<const float4*>(vw.tf), r, B.skip,
-                                                        inv_gmax, is, out, dense, evald, shaded, interp);
+        const float4* tf = reinterpret_cast<const float4*>(vw.tf);
+        if (kAllDerived || v.dbricks) {
+            if (kCount)
+                march_gather<true, false, true, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out, dense, evald, shaded,
+                                                     interp);
+            else
+                march_ahead<true, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out);
+        } else {
+            if (kCount)
+                march_gather<false, false, true, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out, dense, evald, shaded,
+                                                      interp);
+            else
+                march_ahead<false, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out);
+        }
         if (inside) reinterpret_cast<float4*>(vw.out)[(long long)j * vw.W + i] = out;
         if (kCount) {
             rays_hit += hit ? 1u : 0u;
