@@ -9,7 +9,7 @@
 //    4-tap stencils of a cell (voxels i0-1 .. i0+2) fall inside it; 6912 bytes
 //    (a multiple of 16), one bulk copy moves it;
 //  * skip bricks of B^3 cells (B = 2^bs, 4, 8 or 16; 8 by default) carry the
-//    quantised min/max grid, the empty flags, the per-cell empty bits and the
+//    quantised min/max grid, the empty flags and the
 //    derived bricks of the voxel-wise derivatives, (B+1)^3 corners each.
 #pragma once
 

@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(256) k_render_staged(const __grid_constant__ R
 // warp picks the front-most brick any live lane needs, one lane pulls it in with a
 // bulk copy completing on an mbarrier (bounded wait), and the lanes whose next sample
 // lies in it march through it reading the 8 corners of their cells from shared
-// memory (cell bits and the transfer function still through L1). The warp leaves
+// memory (skip field and transfer function still through L1). The warp leaves
 // when a vote finds no live lane. Each lane walks its own samples front to back with
 // the gather kernel's arithmetic (offset-order corner sums), so the image is the
 // same bit for bit. No vesselness channel (mode 2 uses the gather kernels).
