@@ -49,6 +49,14 @@ __device__ __forceinline__ const float4* derived_brick(const VolumeDev& v, int b
         v.dbricks + (size_t)(unsigned)bi * (unsigned)(kBS ? der_brick_floats(kBS) : v.der_stride));
 }
 
+// Whether a sweep reads a cell's corners in parity order (derived_channels). The table's
+// gradient is continuous in the sample's field, so a sweep for the table alone takes the
+// faster offset order (fit step of 8 views 6.64 -> 6.07 ms; not at edge 4, whose corners
+// share L1 columns). Voxel and uniform gradients jump at table knots and at |g| = 0, and a
+// sum in another order puts single samples on the other side: there the order of the
+// corners stays as it has been (it costs 2 % of the 1080p gradient).
+__host__ __device__ constexpr bool parity_order(bool table_only, int bs) { return !table_only || bs == 2; }
+
 // The sample field, from the derived bricks (voxel-wise derivatives) or by the
 // per-sample stencils -- the same linear map of the voxels, either way. kHessian:
 // the Hessian channels are read even without a curvature term (gamma = 0): the
@@ -56,7 +64,7 @@ __device__ __forceinline__ const float4* derived_brick(const VolumeDev& v, int b
 // does.
 // bi: the skip brick of the sample's cell (derived bricks); sbi, base: its storage
 // brick and the stencil origin in it (intensity bricks).
-template <bool kDerived, bool kHessian, int kBS>
+template <bool kDerived, bool kHessian, bool kParity, int kBS>
 __device__ __forceinline__ void eval_field(const VolumeDev& v, const TissueDev& tp, int bi, long long sbi,
                                            const int i0[3], int base, const float f[3], const float is[3],
                                            float fld[10]) {
@@ -64,11 +72,11 @@ __device__ __forceinline__ void eval_field(const VolumeDev& v, const TissueDev& 
         const float4* brick = derived_brick<kBS>(v, bi);
         const int m = (1 << (kBS ? kBS : v.bs)) - 1;
         const DerLayout d = kBS ? der_layout(kBS) : v.der;
-        derived_channels<kBS == 2, 0, 4>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
+        derived_channels<kParity, 0, 4>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
         if (kHessian)
-            derived_channels<kBS == 2, 4, 6>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
+            derived_channels<kParity, 4, 6>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
         else
-            load_hessian<kBS == 2>(tp, brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f, fld);
+            load_hessian<kParity>(tp, brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f, fld);
     } else {
         field_eval(GLoad{v.bricks + sbi * kBrickVox}, base, f[0], f[1], f[2], fld);
         scale_field(fld, is);
@@ -280,7 +288,7 @@ __global__ void __launch_bounds__(256) k_channels_to_voxels(const float* __restr
 // The sample of the reverse sweep at fractions f of cell i0: its field and optics. No
 // skipping: a sample in empty space has alpha = 0, but its lookup still gives the opacity
 // entries it reads a non-zero gradient. bs: log2 of the skip-brick edge.
-template <bool kDerived, bool kLazyHessian, bool kNoHessian, bool k2D, int kBS>
+template <bool kDerived, bool kLazyHessian, bool kNoHessian, bool k2D, bool kParity, int kBS>
 __device__ __forceinline__ void sweep_eval(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
                                            const int i0[3], const float f[3], const float dir[3], const float is[3],
                                            float inv_gmax, float fld[10], SampleOptics& so) {
@@ -296,17 +304,17 @@ __device__ __forceinline__ void sweep_eval(const VolumeDev& v, const TissueDev& 
         const float4* brick = derived_brick<kBS>(v, bi);
         const int m = (1 << bs) - 1;
         const DerLayout d = kBS ? der_layout(kBS) : v.der;
-        derived_channels<kBS == 2, 0, 4>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
+        derived_channels<kParity, 0, 4>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld);
         optics_tf<k2D ? 2 : 1>(fld, vval, tp, tf, inv_gmax, so);
         if (!kNoHessian && so.c.w != 0.0f) {
-            derived_channels<kBS == 2, 4, 6>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
+            derived_channels<kParity, 4, 6>(brick, d, i0[0] & m, i0[1] & m, i0[2] & m, f[0], f[1], f[2], fld + 4);
         } else {
 #pragma unroll
             for (int q = 4; q < 10; ++q) fld[q] = 0.0f;
         }
         optics_rest(fld, dir, tp, so);
     } else {
-        eval_field<kDerived, true, kBS>(v, tp, bi, sbi, i0, base, f, is, fld);
+        eval_field<kDerived, true, kParity, kBS>(v, tp, bi, sbi, i0, base, f, is, fld);
         optics_core<k2D ? 2 : 1>(fld, vval, dir, tp, tf, inv_gmax, so);
     }
 }
@@ -457,7 +465,7 @@ __global__ void __launch_bounds__(128, kTfOnly && !k2D ? 5 : 4) k_render_backwar
                 int base;
                 const long long sbi = storage_brick(v, i0, base);
                 float fld[10];
-                eval_field<kDerived, false, kBS>(v, L.tp, bi, sbi, i0, base, f, is, fld);
+                eval_field<kDerived, false, parity_order(kTfOnly, kBS), kBS>(v, L.tp, bi, sbi, i0, base, f, is, fld);
                 const float vval =
                     v.vbricks ? value_eval(GLoad{v.vbricks + sbi * kBrickVox}, base, f[0], f[1], f[2]) : 0.f;
                 float alpha, col[3];
@@ -498,8 +506,8 @@ __global__ void __launch_bounds__(128, kTfOnly && !k2D ? 5 : 4) k_render_backwar
                     continue;
                 float fld[10];
                 SampleOptics so;
-                sweep_eval<kDerived, kLazyHessian, kNoHessian, k2D, kBS>(v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld,
-                                                                         so);
+                sweep_eval<kDerived, kLazyHessian, kNoHessian, k2D, parity_order(kTfOnly, kBS), kBS>(
+                    v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld, so);
                 const float alpha = so.alpha;
                 // T_k = T_{k+1} / (1 - alpha_k); Tk still holds T_{k+1} here, which a zero
                 // alpha leaves unchanged (x / 1 = x), so the division is skipped then
@@ -580,7 +588,8 @@ __global__ void __launch_bounds__(128, kTfOnly ? 4 : 3) k_backward_lanes(const _
                                            (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
                                            (unsigned)i0[2] <= (unsigned)(v.n[2] - 2));
             if (on)
-                sweep_eval<true, kLazyHessian, kNoHessian, k2D, kBS>(v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld, so);
+                sweep_eval<true, kLazyHessian, kNoHessian, k2D, parity_order(kTfOnly, kBS), kBS>(
+                    v, L.tp, tf, i0, f, r.dir, is, inv_gmax, fld, so);
         }
         const unsigned shaded = __ballot_sync(0xffffffffu, on && so.c.w != 0.0f);
         // the recurrences over the samples kb, kb - 1, ...; a sample of zero opacity entry

@@ -217,10 +217,9 @@ __device__ __forceinline__ void field_eval(const Load& load, int base, float fx,
 // voxel index per axis) rather than of their offset from the cell, so that lanes in
 // neighbouring cells read the same record in the same instruction; each lane picks the
 // matching weight, ~30 instructions per sample. The adjoint sweep gained 3 % by it while
-// neighbouring corners shared L1 columns, and still takes it with skip bricks of edge 4
-//; with the padded planes it costs 1-9 % (fit step of 8 views 6.08 ms in
-// offset order, 6.64 in parity order). The forward kernels keep the offset order
-// everywhere, so that single-view and batched renders stay bit-identical.
+// neighbouring corners shared L1 columns; with the padded planes it costs 2-9 %. The sweep
+// takes it where parity_order says so. The forward kernels keep the offset order everywhere,
+// so that single-view and batched renders stay bit-identical.
 // Read-only 16- and 8-byte loads that ask L2 to fetch the surrounding 256 bytes from DRAM
 // (neighbouring corner records of the same brick rows).
 __device__ __forceinline__ float4 ldg_l2_256(const float4* p) {
