@@ -99,7 +99,6 @@ struct vr_ctx {
     };
     std::unordered_map<void*, Held> allocs;  // device buffers in use
     size_t mem_used = 0;                     // their bytes
-    bool streams_mixed = false;              // vr_set_stream has changed the stream
     size_t mem_limit = 0;                      // 0: no limit beyond the device's
     long long fail_after = -1;                 // >= 0: allocations left before an injected failure
 };
@@ -139,9 +138,8 @@ vr_status cuda_fail(vr_ctx* c, cudaError_t e, const char* what) {
 // device: opening a study makes eleven allocations and closing it eleven frees, each of
 // which waits for the device (181x217x181, load to first 720p frame and close: 0.35 ms of
 // cudaMalloc, 0.64 ms of cudaFree, 2.44 -> 1.45 ms).
-// The pool holds idle buffers only: whoever frees has waited for the work that uses them
-// (on the context's stream; a context that changed streams waits for the device, as
-// cudaFree does), so any context, stream or thread may take them. It is bounded, the
+// The pool holds idle buffers only: whoever frees has waited for the whole device, as
+// cudaFree does (Freeing), so any context, stream or thread may take them. It is bounded, the
 // oldest given up first, and is given back when the device runs out of memory and when
 // the last context on the device is destroyed. A context with a memory limit frees at
 // once. Buffers belong to one CUDA context: after a device reset none is offered again.
@@ -233,55 +231,73 @@ cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
     return cudaSuccess;
 }
 
-// Callers have waited for everything on the context's stream that uses the buffer.
-void dfree(vr_ctx* ctx, void* p) {
-    if (!p) return;
-    size_t cap = 0;
-    auto it = ctx->allocs.find(p);
-    if (it != ctx->allocs.end()) {
-        cap = it->second.cap;
-        ctx->mem_used -= it->second.bytes;
-        ctx->allocs.erase(it);
+// Frees buffers of a context: Freeing fr(ctx); fr(p); fr(q); or, for one, dfree(ctx, p).
+// It first waits, once, for everything queued on the device. The context's stream alone would
+// not do: a caller's graph may hold a batch launch and be replayed on any stream. A buffer goes
+// to the pool only after that wait succeeded (it fails on a stream under capture, for
+// instance); otherwise cudaFree does its own.
+class Freeing {
+  public:
+    explicit Freeing(vr_ctx* ctx) : ctx_(ctx), idle_(cudaDeviceSynchronize() == cudaSuccess) {
+        if (!idle_) (void)cudaGetLastError();
     }
-    const unsigned long long cuda_ctx = current_cuda_context();
-    if (cap == 0 || ctx->mem_limit || cuda_ctx == 0 || cuda_ctx != ctx->cuda_ctx || cap > SparePool::kBytes) {
-        cudaFree(p);
-        return;
-    }
-    if (ctx->streams_mixed && cudaDeviceSynchronize() != cudaSuccess) {
-        cudaFree(p);
-        return;
-    }
-    SparePool& pool = spare_pool();
-    std::lock_guard<std::mutex> lock(pool.mu);
-    if (pool.n == SparePool::kEntries) {
-        if (pool.e[0].device == ctx->device && pool.e[0].cuda_ctx == cuda_ctx) cudaFree(pool.e[0].p);
-        else if (pool.e[0].cuda_ctx != cuda_ctx) {
-            cudaFree(p);  // another device's buffer is not given back from here
+    void operator()(void* p) {
+        if (!p) return;
+        size_t cap = 0;
+        auto it = ctx_->allocs.find(p);
+        if (it != ctx_->allocs.end()) {
+            cap = it->second.cap;
+            ctx_->mem_used -= it->second.bytes;
+            ctx_->allocs.erase(it);
+        }
+        const unsigned long long cuda_ctx = current_cuda_context();
+        if (!idle_ || cap == 0 || ctx_->mem_limit || cuda_ctx == 0 || cuda_ctx != ctx_->cuda_ctx ||
+            cap > SparePool::kBytes) {
+            cudaFree(p);
             return;
         }
-        pool.remove(0);
+        SparePool& pool = spare_pool();
+        std::lock_guard<std::mutex> lock(pool.mu);
+        if (pool.n == SparePool::kEntries) {
+            if (pool.e[0].device == ctx_->device && pool.e[0].cuda_ctx == cuda_ctx) cudaFree(pool.e[0].p);
+            else if (pool.e[0].cuda_ctx != cuda_ctx) {
+                cudaFree(p);  // another device's buffer is not given back from here
+                return;
+            }
+            pool.remove(0);
+        }
+        pool.e[pool.n++] = {p, cap, cuda_ctx, ctx_->device};
+        pool.trim(ctx_->device, cuda_ctx, SparePool::kBytes);
     }
-    pool.e[pool.n++] = {p, cap, cuda_ctx, ctx->device};
-    pool.trim(ctx->device, cuda_ctx, SparePool::kBytes);
+
+  private:
+    vr_ctx* ctx_;
+    bool idle_;
+};
+
+void dfree(vr_ctx* ctx, void* p) {
+    if (!p) return;
+    Freeing fr(ctx);
+    fr(p);
 }
 
 void free_volume(vr_ctx* ctx, Volume* v) {
-    dfree(ctx, v->d_norm);
-    dfree(ctx, v->d_bricks);
-    dfree(ctx, v->d_grid);
-    dfree(ctx, v->d_empty);
-    dfree(ctx, v->d_vc);
-    dfree(ctx, v->d_minmax);
-    dfree(ctx, v->d_vessel);
-    dfree(ctx, v->d_vbricks);
-    dfree(ctx, v->d_dbricks);
-    dfree(ctx, v->d_cellq);
-    dfree(ctx, v->d_skip);
-    dfree(ctx, v->d_smax);
-    dfree(ctx, v->d_ch2);
-    dfree(ctx, v->d_tf);
-    dfree(ctx, v->d_prefix);
+    Freeing fr(ctx);
+    fr(v->d_norm);
+    fr(v->d_bricks);
+    fr(v->d_grid);
+    fr(v->d_empty);
+    fr(v->d_vc);
+    fr(v->d_minmax);
+    fr(v->d_vessel);
+    fr(v->d_vbricks);
+    fr(v->d_dbricks);
+    fr(v->d_cellq);
+    fr(v->d_skip);
+    fr(v->d_smax);
+    fr(v->d_ch2);
+    fr(v->d_tf);
+    fr(v->d_prefix);
     delete v;
 }
 
@@ -431,23 +447,23 @@ vr_status vr_create(vr_ctx** out, int device, void* cuda_stream) {
 vr_status vr_destroy(vr_ctx* ctx) {
     if (!ctx) return VR_OK;
     DeviceGuard g(ctx->device);
-    cudaStreamSynchronize(ctx->stream);
+    Freeing fr(ctx);
     for (auto& kv : ctx->batches) {
         for (auto& g : kv.second->graphs) cudaGraphExecDestroy(g.second);
-        dfree(ctx, kv.second->d_views);
-        dfree(ctx, kv.second->d_prefix);
+        fr(kv.second->d_views);
+        fr(kv.second->d_prefix);
         delete kv.second;
     }
     for (auto& kv : ctx->vols) free_volume(ctx, kv.second);
     if (ctx->graph_stream) cudaStreamDestroy(ctx->graph_stream);
     if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
     if (ctx->ev_out) cudaEventDestroy(ctx->ev_out);
-    dfree(ctx, ctx->d_partials);
-    dfree(ctx, ctx->d_stage);
-    dfree(ctx, ctx->d_scratch);
-    dfree(ctx, ctx->d_tfgrad);
-    dfree(ctx, ctx->d_dgrad);
-    dfree(ctx, ctx->d_work);
+    fr(ctx->d_partials);
+    fr(ctx->d_stage);
+    fr(ctx->d_scratch);
+    fr(ctx->d_tfgrad);
+    fr(ctx->d_dgrad);
+    fr(ctx->d_work);
     {
         std::lock_guard<std::mutex> lock(spare_pool().mu);
         if (--spare_pool().contexts[ctx->device] == 0)
@@ -460,7 +476,6 @@ vr_status vr_destroy(vr_ctx* ctx) {
 
 vr_status vr_set_stream(vr_ctx* ctx, void* cuda_stream) {
     if (!ctx) return VR_ERR_INVALID_ARG;
-    if (ctx->stream != (cudaStream_t)cuda_stream) ctx->streams_mixed = true;
     ctx->stream = (cudaStream_t)cuda_stream;
     return VR_OK;
 }
@@ -538,7 +553,6 @@ vr_status vr_load_volume(vr_ctx* ctx, const void* data, int on_device, vr_dtype 
     const void* raw = data;
     if (e == cudaSuccess) e = device_input(ctx, data, on_device, esz * v->nvox, &raw);
     if (e != cudaSuccess) {
-        cudaStreamSynchronize(ctx->stream);
         free_volume(ctx, v);
         return cuda_fail(ctx, e, "load_volume: allocate/copy");
     }
@@ -560,7 +574,6 @@ vr_status vr_load_volume(vr_ctx* ctx, const void* data, int on_device, vr_dtype 
     if (st == VR_OK && !(isfinite(mm[0]) && isfinite(mm[1])))
         st = fail(ctx, VR_ERR_INVALID_ARG, "load_volume: non-finite intensities");
     if (st != VR_OK) {
-        cudaStreamSynchronize(ctx->stream);
         free_volume(ctx, v);
         return st;
     }
@@ -575,7 +588,6 @@ vr_status vr_free_volume(vr_ctx* ctx, int vol_id) {
     Volume* v = get_vol(ctx, vol_id);
     if (!v) return fail(ctx, VR_ERR_INVALID_ARG, "free_volume: unknown id %d", vol_id);
     DeviceGuard g(ctx->device);
-    cudaStreamSynchronize(ctx->stream);
     free_volume(ctx, v);
     ctx->vols.erase(vol_id);
     return VR_OK;
@@ -829,9 +841,10 @@ vr_status vr_set_brick_size(vr_ctx* ctx, int vol_id, int cells) {
     // field do not depend on it); the derived bricks are rebuilt by the next
     // vr_precompute_morphology
     v->morph_ready = false;
-    dfree(ctx, v->d_grid);
-    dfree(ctx, v->d_empty);
-    dfree(ctx, v->d_dbricks);
+    Freeing fr(ctx);
+    fr(v->d_grid);
+    fr(v->d_empty);
+    fr(v->d_dbricks);
     v->d_grid = nullptr, v->d_empty = nullptr, v->d_dbricks = nullptr;
     v->bs = bs;
     for (int a = 0; a < 3; ++a) v->nb[a] = (v->n[a] - 1 + (1 << bs) - 1) >> bs;
@@ -1254,9 +1267,9 @@ vr_status vr_batch_create(vr_ctx* ctx, const vr_view* views, int n_views, int* b
     }
     vr_status st = batch_upload(ctx, b);
     if (st != VR_OK) {
-        cudaStreamSynchronize(ctx->stream);
-        dfree(ctx, b->d_views);
-        dfree(ctx, b->d_prefix);
+        Freeing fr(ctx);
+        fr(b->d_views);
+        fr(b->d_prefix);
         delete b;
         return st;
     }
@@ -1337,11 +1350,10 @@ vr_status vr_batch_free(vr_ctx* ctx, int batch_id) {
     auto it = ctx->batches.find(batch_id);
     if (it == ctx->batches.end()) return fail(ctx, VR_ERR_INVALID_ARG, "batch_free: unknown batch %d", batch_id);
     DeviceGuard g(ctx->device);
-    cudaStreamSynchronize(ctx->stream);
-    if (ctx->graph_stream) cudaStreamSynchronize(ctx->graph_stream);
+    Freeing fr(ctx);
     for (auto& gx : it->second->graphs) cudaGraphExecDestroy(gx.second);
-    dfree(ctx, it->second->d_views);
-    dfree(ctx, it->second->d_prefix);
+    fr(it->second->d_views);
+    fr(it->second->d_prefix);
     delete it->second;
     ctx->batches.erase(it);
     return VR_OK;
@@ -1373,7 +1385,6 @@ vr_status vr_fma_peak(vr_ctx* ctx, int blocks, int iters, int reps, float* h_ms,
         ms.push_back(t);
     }
     for (int q = 0; q < made; ++q) cudaEventDestroy(ev[q]);
-    if (e != cudaSuccess) cudaStreamSynchronize(ctx->stream);
     dfree(ctx, out);
     if (e != cudaSuccess) return fail(ctx, VR_ERR_CUDA, "fma_peak: %s", cudaGetErrorString(e));
     std::sort(ms.begin(), ms.end());
