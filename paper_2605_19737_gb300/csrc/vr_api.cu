@@ -66,6 +66,7 @@ struct Batch {
 
 }  // namespace
 
+constexpr size_t kMarkerBytes = 256;
 constexpr int kParamSums = 32;  // words into vr_ctx::d_work (64 words, 8-byte aligned)
 
 struct vr_ctx {
@@ -98,7 +99,8 @@ struct vr_ctx {
         size_t bytes, cap;  // asked for, and the allocation's size
     };
     std::unordered_map<void*, Held> allocs;  // device buffers in use
-    size_t mem_used = 0;                     // their bytes
+    size_t mem_used = 0;                     // their bytes, and the marker's
+    void* marker = nullptr;                  // freed and allocated anew as a wait for the device (Freeing)
     size_t mem_limit = 0;                      // 0: no limit beyond the device's
     long long fail_after = -1;                 // >= 0: allocations left before an injected failure
 };
@@ -234,12 +236,22 @@ cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
 // Frees buffers of a context: Freeing fr(ctx); fr(p); fr(q); or, for one, dfree(ctx, p).
 // It first waits, once, for everything queued on the device. The context's stream alone would
 // not do: a caller's graph may hold a batch launch and be replayed on any stream. A buffer goes
-// to the pool only after that wait succeeded (it fails on a stream under capture, for
-// instance); otherwise cudaFree does its own.
+// to the pool only after that wait succeeded; otherwise cudaFree does its own.
+// The wait is the one that cudaFree makes, on a small buffer kept for it (measured: it ends
+// with the kernels and graph replays of every stream; 2 us with the next cudaMalloc when the
+// device is idle). cudaDeviceSynchronize fails, and invalidates the capture, while any thread
+// captures any stream; cudaFree only where that capture forbids it to this thread.
 class Freeing {
   public:
-    explicit Freeing(vr_ctx* ctx) : ctx_(ctx), idle_(cudaDeviceSynchronize() == cudaSuccess) {
-        if (!idle_) (void)cudaGetLastError();
+    explicit Freeing(vr_ctx* ctx) : ctx_(ctx) {
+        if (ctx->marker) {
+            idle_ = cudaFree(ctx->marker) == cudaSuccess;
+            if (idle_) ctx->marker = nullptr;
+        } else {
+            idle_ = cudaDeviceSynchronize() == cudaSuccess;
+        }
+        if (!ctx->marker && cudaMalloc(&ctx->marker, kMarkerBytes) != cudaSuccess) ctx->marker = nullptr;
+        (void)cudaGetLastError();
     }
     void operator()(void* p) {
         if (!p) return;
@@ -428,10 +440,15 @@ vr_status vr_create(vr_ctx** out, int device, void* cuda_stream) {
     DeviceGuard g(device);
     cudaFree(nullptr);  // the CUDA context exists from here on
     ctx->cuda_ctx = current_cuda_context();
-    cudaError_t e = dalloc(ctx, &ctx->d_work, 64 * sizeof(unsigned));
+    cudaError_t e = cudaMalloc(&ctx->marker, kMarkerBytes);
+    if (e == cudaSuccess) {
+        ctx->mem_used += kMarkerBytes;
+        e = dalloc(ctx, &ctx->d_work, 64 * sizeof(unsigned));
+    }
     if (e == cudaSuccess) e = cudaMemset(ctx->d_work, 0, 64 * sizeof(unsigned));
     if (e != cudaSuccess) {
         dfree(ctx, ctx->d_work);
+        cudaFree(ctx->marker);
         delete ctx;
         (void)cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? VR_ERR_OOM : VR_ERR_CUDA;
@@ -464,6 +481,7 @@ vr_status vr_destroy(vr_ctx* ctx) {
     fr(ctx->d_tfgrad);
     fr(ctx->d_dgrad);
     fr(ctx->d_work);
+    cudaFree(ctx->marker);
     {
         std::lock_guard<std::mutex> lock(spare_pool().mu);
         if (--spare_pool().contexts[ctx->device] == 0)

@@ -7,6 +7,9 @@
 // allocated at that moment. It lasts until something waits for the whole device:
 // cudaDeviceSynchronize or cudaFree. Until then, a write into one of those buffers on behalf
 // of a new object counts as a violation.
+// fake_capture() stands for a capture by another thread that forbids this one nothing
+// (cudaStreamCaptureModeThreadLocal): cudaFree works, but cudaDeviceSynchronize fails and
+// invalidates the capture, as on the device.
 #include <cuda_runtime_api.h>
 
 #include <stdint.h>
@@ -22,8 +25,8 @@ namespace {
 
 std::map<char*, size_t> g_live;    // allocations by address
 std::set<char*> g_replayed;        // those the unknown work uses
-bool g_busy = false, g_fail_waits = false;
-int g_violations = 0, g_device_waits = 0;
+bool g_busy = false, g_fail_waits = false, g_capture = false, g_capture_valid = false;
+int g_violations = 0;
 
 void device_done() {
     g_busy = false;
@@ -53,7 +56,8 @@ void fake_replay() {
 }
 void fake_fail_waits(int on) { g_fail_waits = on != 0; }
 int fake_violations() { return g_violations; }
-int fake_device_waits() { return g_device_waits; }
+void fake_capture(int on) { g_capture = on != 0, g_capture_valid = true; }
+int fake_capture_valid() { return g_capture_valid; }
 long long fake_live_bytes() {
     long long s = 0;
     for (auto& kv : g_live) s += (long long)kv.second;
@@ -68,13 +72,17 @@ cudaError_t cudaMalloc(void** p, size_t n) {
 }
 cudaError_t cudaFree(void* p) {
     if (!p) return cudaSuccess;
+    if (g_fail_waits) return cudaErrorStreamCaptureUnsupported;
     device_done();  // the real call waits for the device
     g_live.erase(static_cast<char*>(p));
     free(p);
     return cudaSuccess;
 }
 cudaError_t cudaDeviceSynchronize() {
-    ++g_device_waits;
+    if (g_capture) {
+        g_capture_valid = false;
+        return cudaErrorStreamCaptureUnsupported;
+    }
     const cudaError_t e = wait();
     if (e == cudaSuccess) device_done();
     return e;

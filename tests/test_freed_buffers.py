@@ -137,6 +137,22 @@ def test_no_buffer_in_use_is_handed_out(lib, scene, fail_waits):
     c.close()
 
 
+def test_capture_on_another_thread_stays_valid(lib):
+    """Another thread captures a stream of its own in thread-local mode, which cudaFree has no
+    part in: buffers are freed, none in use is handed out, and the capture stays valid."""
+    c = Lib(lib)
+    before = lib.fake_violations()
+    lib.fake_capture(1)
+    try:
+        for scene in (_free_volume, _free_batch, _destroy, _wider_table):
+            scene(c)
+        assert lib.fake_capture_valid()
+    finally:
+        lib.fake_capture(0)
+    assert lib.fake_violations() == before
+    c.close()
+
+
 def test_everything_is_given_back(lib):
     base = lib.fake_live_bytes()
     a, b = Lib(lib), Lib(lib)
