@@ -69,9 +69,13 @@ struct Batch {
 constexpr size_t kMarkerBytes = 256;
 constexpr int kParamSums = 32;  // words into vr_ctx::d_work (64 words, 8-byte aligned)
 
+namespace {
+struct DevicePool;
+}
+
 struct vr_ctx {
     int device = 0;
-    unsigned long long cuda_ctx = 0;  // id of the CUDA context the buffers belong to
+    DevicePool* pool = nullptr;  // where its buffers come from, NULL: cudaMalloc
     cudaStream_t stream = nullptr;
     std::string err;
     std::map<int, Volume*> vols;
@@ -96,9 +100,11 @@ struct vr_ctx {
     cudaStream_t graph_stream = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     struct Held {
-        size_t bytes, cap;  // asked for, and the allocation's size
+        size_t bytes;
+        bool pooled;  // from the pool, not cudaMalloc
     };
-    std::unordered_map<void*, Held> allocs;  // device buffers in use
+    std::unordered_map<void*, Held> allocs;  // device buffers
+    std::vector<void*> held;                 // those to be freed after a wait that succeeds (Freeing)
     size_t mem_used = 0;                     // their bytes, and the marker's
     void* marker = nullptr;                  // freed and allocated anew as a wait for the device (Freeing)
     size_t mem_limit = 0;                      // 0: no limit beyond the device's
@@ -136,65 +142,72 @@ vr_status cuda_fail(vr_ctx* c, cudaError_t e, const char* what) {
 // knows what it holds (vr_memory_used), can refuse to grow past a limit
 // (vr_set_memory_limit) and can be made to see an allocation fail (vr_debug_fail_alloc).
 // A refused allocation returns cudaErrorMemoryAllocation like a failed cudaMalloc.
-// Freed buffers are kept for the next allocation of about their size, by any context on the
-// device: opening a study makes eleven allocations and closing it eleven frees, each of
-// which waits for the device (181x217x181, load to first 720p frame and close: 0.35 ms of
-// cudaMalloc, 0.64 ms of cudaFree, 2.44 -> 1.45 ms).
-// The pool holds idle buffers only: whoever frees has waited for the whole device, as
-// cudaFree does (Freeing), so any context, stream or thread may take them. It is bounded, the
-// oldest given up first, and is given back when the device runs out of memory and when
-// the last context on the device is destroyed. A context with a memory limit frees at
-// once. Buffers belong to one CUDA context: after a device reset none is offered again.
-struct SparePool {
-    static constexpr size_t kBytes = (size_t)2 << 30;
-    static constexpr int kEntries = 64;
-    struct Entry {
-        void* p;
-        size_t cap;
-        unsigned long long cuda_ctx;
-        int device;
-    };
-    std::mutex mu;
-    Entry e[kEntries];  // oldest first
-    int n = 0;
-    std::map<int, int> contexts;  // live contexts per device
-
-    void remove(int i) {
-        memmove(e + i, e + i + 1, sizeof(Entry) * (size_t)(n - i - 1));
-        --n;
-    }
-    // Give back the device's oldest buffers until the others take at most `keep` bytes;
-    // those of another (destroyed) CUDA context are only forgotten.
-    void trim(int device, unsigned long long cuda_ctx, size_t keep) {
-        size_t sum = 0;
-        for (int i = 0; i < n; ++i) sum += e[i].device == device ? e[i].cap : 0;
-        for (int i = 0; i < n && sum > keep;) {
-            if (e[i].device != device) {
-                ++i;
-                continue;
-            }
-            sum -= e[i].cap;
-            if (e[i].cuda_ctx == cuda_ctx) cudaFree(e[i].p);
-            remove(i);
-        }
-    }
-    // The smallest buffer that fits with little waste, or NULL.
-    void* take(int device, unsigned long long cuda_ctx, size_t bytes, size_t* cap) {
-        int best = -1;
-        for (int i = 0; i < n; ++i)
-            if (e[i].device == device && e[i].cuda_ctx == cuda_ctx && e[i].cap >= bytes &&
-                e[i].cap - bytes <= std::max<size_t>(4096, bytes / 16) && (best < 0 || e[i].cap < e[best].cap))
-                best = i;
-        if (best < 0) return nullptr;
-        void* p = e[best].p;
-        *cap = e[best].cap;
-        remove(best);
-        return p;
-    }
+// They come from a CUDA memory pool that the contexts on a device share and that keeps what is
+// freed for the next allocation: opening a study makes eleven allocations and closing it eleven
+// frees (181x217x181: cudaMalloc 251 us and cudaFree 656 us, from the pool 4 and 5; load to
+// first 720p frame and close 2.44 -> 1.45 ms).
+// What the pool keeps is bounded, and is not lost to others: the driver takes it back for any
+// cudaMalloc of the process that finds the device full, and the library when the last context
+// on the device is destroyed. A context with a memory limit has it released at once.
+struct DevicePool {
+    static constexpr size_t kSpareBytes = (size_t)2 << 30;
+    int device;
+    unsigned long long cuda_ctx;  // id of the CUDA context whose stream it is
+    cudaMemPool_t pool;
+    cudaStream_t stream;  // orders allocations and frees, and runs nothing
+    int users;            // library contexts
 };
-SparePool& spare_pool() {
-    static SparePool* pool = new SparePool();  // never destroyed: contexts may outlive static objects
-    return *pool;
+std::mutex g_pools_mu;
+std::vector<DevicePool*>& device_pools() {
+    static auto* pools = new std::vector<DevicePool*>();  // never destroyed: contexts may outlive static objects
+    return *pools;
+}
+
+// The pool of the current CUDA context's device, NULL where there can be none (allocations
+// are then cudaMalloc's).
+DevicePool* acquire_pool(int device, unsigned long long cuda_ctx) {
+    if (cuda_ctx == 0) return nullptr;
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    for (DevicePool* p : device_pools())
+        if (p->device == device && p->cuda_ctx == cuda_ctx) {
+            ++p->users;
+            return p;
+        }
+    DevicePool n{device, cuda_ctx, nullptr, nullptr, 1};
+    int supported = 0;
+    cudaDeviceGetAttribute(&supported, cudaDevAttrMemoryPoolsSupported, device);
+    cudaMemPoolProps props;
+    memset(&props, 0, sizeof props);
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    unsigned long long all = ~0ull;  // Freeing bounds what is kept
+    if (!supported || cudaMemPoolCreate(&n.pool, &props) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    if (cudaMemPoolSetAttribute(n.pool, cudaMemPoolAttrReleaseThreshold, &all) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&n.stream, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaMemPoolDestroy(n.pool);
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    device_pools().push_back(new DevicePool(n));
+    return device_pools().back();
+}
+
+// Buffers still out (held back because no wait succeeded) stay valid past the pool's handle.
+void release_pool(DevicePool* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    if (--p->users) return;
+    auto& pools = device_pools();
+    pools.erase(std::find(pools.begin(), pools.end(), p));
+    if (current_cuda_context() == p->cuda_ctx) {  // else it went with its CUDA context
+        cudaMemPoolDestroy(p->pool);
+        cudaStreamDestroy(p->stream);
+    }
+    delete p;
 }
 
 template <class T>
@@ -207,27 +220,18 @@ cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
     if (ctx->fail_after > 0) --ctx->fail_after;
     if (ctx->mem_limit && bytes > ctx->mem_limit - std::min(ctx->mem_limit, ctx->mem_used))
         return cudaErrorMemoryAllocation;
-    SparePool& pool = spare_pool();
-    const unsigned long long cuda_ctx = current_cuda_context();
     void* q = nullptr;
-    size_t cap = bytes;
-    if (cuda_ctx) {
-        std::lock_guard<std::mutex> lock(pool.mu);
-        q = pool.take(ctx->device, cuda_ctx, bytes, &cap);
+    const bool pooled = ctx->pool && current_cuda_context() == ctx->pool->cuda_ctx;
+    cudaError_t e;
+    if (pooled) {
+        e = cudaMallocFromPoolAsync(&q, bytes, ctx->pool->pool, ctx->pool->stream);
+        if (e == cudaSuccess && (e = cudaStreamSynchronize(ctx->pool->stream)) != cudaSuccess)  // for every stream
+            cudaFreeAsync(q, ctx->pool->stream);
+    } else {
+        e = cudaMalloc(&q, bytes);
     }
-    if (!q) {
-        cudaError_t e = cudaMalloc(&q, bytes);
-        if (e == cudaErrorMemoryAllocation) {
-            (void)cudaGetLastError();
-            {
-                std::lock_guard<std::mutex> lock(pool.mu);
-                pool.trim(ctx->device, cuda_ctx, 0);
-            }
-            e = cudaMalloc(&q, bytes);
-        }
-        if (e != cudaSuccess) return e;
-    }
-    ctx->allocs[q] = {bytes, cap};
+    if (e != cudaSuccess) return e;
+    ctx->allocs[q] = {bytes, pooled};
     ctx->mem_used += bytes;
     *p = static_cast<T*>(q);
     return cudaSuccess;
@@ -236,7 +240,8 @@ cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
 // Frees buffers of a context: Freeing fr(ctx); fr(p); fr(q); or, for one, dfree(ctx, p).
 // It first waits, once, for everything queued on the device. The context's stream alone would
 // not do: a caller's graph may hold a batch launch and be replayed on any stream. A buffer goes
-// to the pool only after that wait succeeded; otherwise cudaFree does its own.
+// back to the pool only after that wait succeeded; otherwise the context holds on to it, as
+// used, until one does.
 // The wait is the one that cudaFree makes, on a small buffer kept for it (measured: it ends
 // with the kernels and graph replays of every stream; 2 us with the next cudaMalloc when the
 // device is idle). cudaDeviceSynchronize fails, and invalidates the capture, while any thread
@@ -251,40 +256,43 @@ class Freeing {
             idle_ = cudaDeviceSynchronize() == cudaSuccess;
         }
         if (!ctx->marker && cudaMalloc(&ctx->marker, kMarkerBytes) != cudaSuccess) ctx->marker = nullptr;
+        idle_ = idle_ && ctx->pool && current_cuda_context() == ctx->pool->cuda_ctx;
         (void)cudaGetLastError();
+        if (idle_) {
+            std::vector<void*> held;
+            held.swap(ctx->held);
+            for (void* p : held) (*this)(p);
+        }
     }
     void operator()(void* p) {
         if (!p) return;
-        size_t cap = 0;
-        auto it = ctx_->allocs.find(p);
-        if (it != ctx_->allocs.end()) {
-            cap = it->second.cap;
-            ctx_->mem_used -= it->second.bytes;
-            ctx_->allocs.erase(it);
-        }
-        const unsigned long long cuda_ctx = current_cuda_context();
-        if (!idle_ || cap == 0 || ctx_->mem_limit || cuda_ctx == 0 || cuda_ctx != ctx_->cuda_ctx ||
-            cap > SparePool::kBytes) {
-            cudaFree(p);
+        const auto it = ctx_->allocs.find(p);  // everything was dalloc's
+        if (it->second.pooled && !idle_) {
+            ctx_->held.push_back(p);
             return;
         }
-        SparePool& pool = spare_pool();
-        std::lock_guard<std::mutex> lock(pool.mu);
-        if (pool.n == SparePool::kEntries) {
-            if (pool.e[0].device == ctx_->device && pool.e[0].cuda_ctx == cuda_ctx) cudaFree(pool.e[0].p);
-            else if (pool.e[0].cuda_ctx != cuda_ctx) {
-                cudaFree(p);  // another device's buffer is not given back from here
-                return;
-            }
-            pool.remove(0);
+        if (it->second.pooled) {
+            cudaFreeAsync(p, ctx_->pool->stream);
+            trim_ = true;
+        } else {
+            cudaFree(p);
         }
-        pool.e[pool.n++] = {p, cap, cuda_ctx, ctx_->device};
-        pool.trim(ctx_->device, cuda_ctx, SparePool::kBytes);
+        ctx_->mem_used -= it->second.bytes;
+        ctx_->allocs.erase(it);
+    }
+    ~Freeing() {
+        if (!trim_) return;
+        const DevicePool& d = *ctx_->pool;
+        unsigned long long used = 0;
+        if (cudaStreamSynchronize(d.stream) == cudaSuccess &&
+            cudaMemPoolGetAttribute(d.pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+            cudaMemPoolTrimTo(d.pool, (size_t)used + (ctx_->mem_limit ? 0 : DevicePool::kSpareBytes));
+        (void)cudaGetLastError();
     }
 
   private:
     vr_ctx* ctx_;
-    bool idle_;
+    bool idle_, trim_ = false;
 };
 
 void dfree(vr_ctx* ctx, void* p) {
@@ -293,8 +301,7 @@ void dfree(vr_ctx* ctx, void* p) {
     fr(p);
 }
 
-void free_volume(vr_ctx* ctx, Volume* v) {
-    Freeing fr(ctx);
+void free_volume(Freeing& fr, Volume* v) {
     fr(v->d_norm);
     fr(v->d_bricks);
     fr(v->d_grid);
@@ -311,6 +318,11 @@ void free_volume(vr_ctx* ctx, Volume* v) {
     fr(v->d_tf);
     fr(v->d_prefix);
     delete v;
+}
+
+void free_volume(vr_ctx* ctx, Volume* v) {
+    Freeing fr(ctx);
+    free_volume(fr, v);
 }
 
 Volume* get_vol(vr_ctx* ctx, int id) {
@@ -439,23 +451,22 @@ vr_status vr_create(vr_ctx** out, int device, void* cuda_stream) {
     ctx->stream = (cudaStream_t)cuda_stream;
     DeviceGuard g(device);
     cudaFree(nullptr);  // the CUDA context exists from here on
-    ctx->cuda_ctx = current_cuda_context();
     cudaError_t e = cudaMalloc(&ctx->marker, kMarkerBytes);
     if (e == cudaSuccess) {
+        // d_work next to it, not from the pool: freeing the marker would else give its page
+        // back and take 40 us, allocating it again 55
         ctx->mem_used += kMarkerBytes;
         e = dalloc(ctx, &ctx->d_work, 64 * sizeof(unsigned));
+        ctx->pool = acquire_pool(device, current_cuda_context());
     }
     if (e == cudaSuccess) e = cudaMemset(ctx->d_work, 0, 64 * sizeof(unsigned));
     if (e != cudaSuccess) {
         dfree(ctx, ctx->d_work);
         cudaFree(ctx->marker);
+        release_pool(ctx->pool);
         delete ctx;
         (void)cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? VR_ERR_OOM : VR_ERR_CUDA;
-    }
-    {
-        std::lock_guard<std::mutex> lock(spare_pool().mu);
-        ++spare_pool().contexts[device];
     }
     *out = ctx;
     return VR_OK;
@@ -464,29 +475,27 @@ vr_status vr_create(vr_ctx** out, int device, void* cuda_stream) {
 vr_status vr_destroy(vr_ctx* ctx) {
     if (!ctx) return VR_OK;
     DeviceGuard g(ctx->device);
-    Freeing fr(ctx);
-    for (auto& kv : ctx->batches) {
-        for (auto& g : kv.second->graphs) cudaGraphExecDestroy(g.second);
-        fr(kv.second->d_views);
-        fr(kv.second->d_prefix);
-        delete kv.second;
-    }
-    for (auto& kv : ctx->vols) free_volume(ctx, kv.second);
-    if (ctx->graph_stream) cudaStreamDestroy(ctx->graph_stream);
-    if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
-    if (ctx->ev_out) cudaEventDestroy(ctx->ev_out);
-    fr(ctx->d_partials);
-    fr(ctx->d_stage);
-    fr(ctx->d_scratch);
-    fr(ctx->d_tfgrad);
-    fr(ctx->d_dgrad);
-    fr(ctx->d_work);
-    cudaFree(ctx->marker);
     {
-        std::lock_guard<std::mutex> lock(spare_pool().mu);
-        if (--spare_pool().contexts[ctx->device] == 0)
-            spare_pool().trim(ctx->device, current_cuda_context(), 0);  // the last context gives everything back
+        Freeing fr(ctx);
+        for (auto& kv : ctx->batches) {
+            for (auto& g : kv.second->graphs) cudaGraphExecDestroy(g.second);
+            fr(kv.second->d_views);
+            fr(kv.second->d_prefix);
+            delete kv.second;
+        }
+        for (auto& kv : ctx->vols) free_volume(fr, kv.second);
+        if (ctx->graph_stream) cudaStreamDestroy(ctx->graph_stream);
+        if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
+        if (ctx->ev_out) cudaEventDestroy(ctx->ev_out);
+        fr(ctx->d_partials);
+        fr(ctx->d_stage);
+        fr(ctx->d_scratch);
+        fr(ctx->d_tfgrad);
+        fr(ctx->d_dgrad);
+        fr(ctx->d_work);
     }
+    cudaFree(ctx->marker);
+    release_pool(ctx->pool);
     (void)cudaGetLastError();
     delete ctx;
     return VR_OK;

@@ -18,12 +18,16 @@
 
 #include <map>
 #include <set>
+#include <utility>
+#include <vector>
 
 #include "vr.h"
 
 namespace {
 
 std::map<char*, size_t> g_live;    // allocations by address
+std::vector<std::pair<char*, size_t>> g_spare;  // freed into the memory pool, the oldest first
+size_t g_capacity = ~(size_t)0;    // of the device
 std::set<char*> g_replayed;        // those the unknown work uses
 bool g_busy = false, g_fail_waits = false, g_capture = false, g_capture_valid = false;
 int g_violations = 0;
@@ -42,6 +46,27 @@ void written(const void* p) {
     if (c < it->first + it->second && g_replayed.count(it->first)) ++g_violations;
 }
 
+size_t held() {
+    size_t s = 0;
+    for (auto& kv : g_live) s += kv.second;
+    for (auto& e : g_spare) s += e.second;
+    return s;
+}
+
+// The pool gives its oldest spare memory back until the device holds at most `keep` bytes.
+void trim(size_t keep) {
+    while (!g_spare.empty() && held() > keep) {
+        free(g_spare.front().first);
+        g_spare.erase(g_spare.begin());
+    }
+}
+
+bool room(size_t n) {
+    if (n > g_capacity) return false;
+    trim(g_capacity - n);  // as the driver does for any allocation of the process
+    return held() <= g_capacity - n;
+}
+
 cudaError_t wait() { return g_fail_waits ? cudaErrorStreamCaptureUnsupported : cudaSuccess; }
 
 }  // namespace
@@ -58,14 +83,12 @@ void fake_fail_waits(int on) { g_fail_waits = on != 0; }
 int fake_violations() { return g_violations; }
 void fake_capture(int on) { g_capture = on != 0, g_capture_valid = true; }
 int fake_capture_valid() { return g_capture_valid; }
-long long fake_live_bytes() {
-    long long s = 0;
-    for (auto& kv : g_live) s += (long long)kv.second;
-    return s;
-}
+long long fake_held_bytes() { return (long long)held(); }
+void fake_capacity(long long n) { g_capacity = n < 0 ? ~(size_t)0 : (size_t)n; }
 
 // ---- the runtime
 cudaError_t cudaMalloc(void** p, size_t n) {
+    if (!room(n)) return cudaErrorMemoryAllocation;
     *p = calloc(n ? n : 1, 1);
     g_live[static_cast<char*>(*p)] = n;
     return cudaSuccess;
@@ -76,6 +99,42 @@ cudaError_t cudaFree(void* p) {
     device_done();  // the real call waits for the device
     g_live.erase(static_cast<char*>(p));
     free(p);
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) {
+    *p = reinterpret_cast<cudaMemPool_t>(3);
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolDestroy(cudaMemPool_t) {
+    trim(0);
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
+cudaError_t cudaMemPoolGetAttribute(cudaMemPool_t, cudaMemPoolAttr, void* v) {
+    size_t used = 0;
+    for (auto& kv : g_live) used += kv.second;
+    *static_cast<unsigned long long*>(v) = used;
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t keep) {
+    trim(keep);
+    return cudaSuccess;
+}
+cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) {
+    for (size_t i = g_spare.size(); i-- > 0;)
+        if (g_spare[i].second == n) {
+            *p = g_spare[i].first;
+            g_live[g_spare[i].first] = n;
+            g_spare.erase(g_spare.begin() + (long)i);
+            return cudaSuccess;
+        }
+    return cudaMalloc(p, n);
+}
+cudaError_t cudaFreeAsync(void* p, cudaStream_t) {  // waits for nothing
+    char* c = static_cast<char*>(p);
+    if (g_busy && g_replayed.count(c)) ++g_violations;
+    g_spare.emplace_back(c, g_live[c]);
+    g_live.erase(c);
     return cudaSuccess;
 }
 cudaError_t cudaDeviceSynchronize() {

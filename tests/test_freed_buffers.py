@@ -30,7 +30,7 @@ def lib(tmp_path_factory):
                     os.path.join(HERE, "native", "fake_cuda.cpp"), os.path.join(native.BUILD, "vr_api.o"), "-ldl",
                     "-o", out], check=True)
     lib = ctypes.CDLL(out)
-    lib.fake_live_bytes.restype = ctypes.c_longlong
+    lib.fake_held_bytes.restype = ctypes.c_longlong
     lib.vr_last_error.restype = ctypes.c_char_p
     return lib
 
@@ -82,6 +82,11 @@ class Lib:
         bid = ctypes.c_int()
         self.ok(self.lib.vr_batch_create(self.h, arr, views, ctypes.byref(bid)))
         return bid.value
+
+    def used(self):
+        n = ctypes.c_ulonglong()
+        self.ok(self.lib.vr_memory_used(self.h, ctypes.byref(n)))
+        return n.value
 
     def close(self):
         if self.h:
@@ -154,7 +159,7 @@ def test_capture_on_another_thread_stays_valid(lib):
 
 
 def test_everything_is_given_back(lib):
-    base = lib.fake_live_bytes()
+    base = lib.fake_held_bytes()
     a, b = Lib(lib), Lib(lib)
     for _ in range(3):
         for c in (a, b):
@@ -162,4 +167,39 @@ def test_everything_is_given_back(lib):
             c.open(17)
     a.close()
     b.close()
-    assert lib.fake_live_bytes() == base
+    assert lib.fake_held_bytes() == base
+
+
+def test_freed_memory_is_there_for_others(lib):
+    """Another allocator of the process finds room for what a freed volume took, while the
+    context lives."""
+    c = Lib(lib)
+    vid = c.open(40)
+    held, used = lib.fake_held_bytes(), c.used()
+    c.ok(lib.vr_free_volume(c.h, vid))
+    taken = used - c.used()
+    p = ctypes.c_void_p()
+    lib.fake_capacity(ctypes.c_longlong(held))
+    try:
+        assert lib.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(taken)) == 0
+    finally:
+        lib.fake_capacity(ctypes.c_longlong(-1))
+    lib.cudaFree(p)
+    c.open(40)
+    c.close()
+
+
+def test_what_is_kept_is_bounded(lib):
+    """A volume above the bound is given back at once, and so is everything of a context with a
+    memory limit."""
+    c = Lib(lib)
+    base = lib.fake_held_bytes()
+    big = c.load(320)
+    c.ok(lib.vr_precompute_morphology(c.h, big, None, 0))
+    assert lib.fake_held_bytes() - base > 2 << 30
+    c.ok(lib.vr_free_volume(c.h, big))
+    assert lib.fake_held_bytes() - base <= 2 << 30
+    c.ok(lib.vr_set_memory_limit(c.h, ctypes.c_ulonglong(1 << 40)))
+    c.ok(lib.vr_free_volume(c.h, c.load(20)))
+    assert lib.fake_held_bytes() <= base + (1 << 20)
+    c.close()

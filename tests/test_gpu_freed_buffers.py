@@ -95,3 +95,23 @@ def test_capture_on_another_thread_stays_valid(torch):
     graph.replay()
     torch.cuda.synchronize()
     assert float(x[0]) == 2.0
+
+
+def test_freed_memory_is_there_for_torch(torch):
+    """After a volume is freed torch can have all the memory that is free and part of what the
+    library kept, while the context lives; the context then works as before."""
+    import paper_2605_19737_gb300 as pkg
+    dims = (200, 200, 200)
+    cams = camera_array([orbit_camera(dims, (1, 1, 1), 20.0, 10.0, width=64, height=48)])
+    with pkg.Context(0) as ctx:
+        vid = _open(ctx, 0, dims)
+        want = ctx.render(vid, cams, 64, 48).cpu()
+        used = ctx.memory_used()
+        ctx.free_volume(vid)
+        taken = used - ctx.memory_used()
+        assert taken > 500 << 20
+        torch.cuda.empty_cache()
+        big = torch.empty(torch.cuda.mem_get_info()[0] + taken // 2, dtype=torch.uint8, device="cuda")
+        del big
+        torch.cuda.empty_cache()
+        assert torch.equal(ctx.render(_open(ctx, 0, dims), cams, 64, 48).cpu(), want)
