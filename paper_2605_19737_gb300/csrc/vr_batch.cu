@@ -47,14 +47,12 @@ __device__ __forceinline__ void batch_body(const BatchLaunch& B) {
         const float4* tf = reinterpret_cast<const float4*>(vw.tf);
         if (kAllDerived || v.dbricks) {
             if (kCount)
-                march_gather<true, false, true, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out, dense, evald, shaded,
-                                                     interp);
+                march_count<true, false, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out, dense, evald, shaded, interp);
             else
                 march_ahead<true, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out);
         } else {
             if (kCount)
-                march_gather<false, false, true, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out, dense, evald, shaded,
-                                                      interp);
+                march_count<false, false, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out, dense, evald, shaded, interp);
             else
                 march_ahead<false, kBS>(v, vw.tp, tf, r, B.skip, inv_gmax, is, out);
         }
@@ -106,11 +104,13 @@ cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, int* per_sm
 cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, bool all_derived, int bs,
                                 cudaStream_t st) {
     const int t = warps_per_block * 32;
-    if (all_derived && B.counters)
+    // without skipping there is nothing to look ahead for either
+    const bool count = B.counters || !B.skip;
+    if (all_derived && count)
         launch_derived<true>(B, ctas, t, bs, st);
     else if (all_derived)
         launch_derived<false>(B, ctas, t, bs, st);
-    else if (B.counters)
+    else if (count)
         k_render_batch_mixed<true><<<ctas, t, 0, st>>>(B);
     else
         k_render_batch_mixed<false><<<ctas, t, 0, st>>>(B);

@@ -82,7 +82,7 @@ __device__ __forceinline__ bool eval_sample(const VolumeDev& v, const TissueDev&
 // exactly 0 (its intensity lies in the range of the cell's 8 corners) and adds nothing.
 // The skip field holds, per cell, the distance to the nearest cell that may have
 // opacity, so one byte load both tests the cell and leaps over empty space; it needs no
-// brick state in registers.
+// brick state in registers. With skip the volume has a field.
 // The lanes of a warp walk in step: all at the same sample index k, advancing together
 // by the smallest leap any lane may take. Neighbouring rays then sit at the same
 // depth and their corner loads share cells; a lane that leapt alone would lose step for
@@ -91,9 +91,6 @@ __device__ __forceinline__ bool eval_sample(const VolumeDev& v, const TissueDev&
 // 0.811 ms, each lane leaping for itself 2.16 / 0.134 / 0.90, warps in step 1.81 / 0.130
 // / 0.72. Bound by latency: ~0.45 issue slots used, two L1 round trips (byte, corners)
 // and the table's per sample.
-// kCount: the launch wants sample counters. Evaluated samples are defined by the
-// skip bricks (samples outside bricks classified empty), so this variant walks brick by
-// brick and sample by sample instead of leaping; the image is the same.
 // With kState it also returns the ray's last sample index (kstop) and the
 // transmittance in front of that sample (t_last), which the adjoint sweep starts from.
 // kBS: log2 of the skip-brick edge in cells, fixed at compile time (2, 3, 4), or 0 to
@@ -102,19 +99,16 @@ __device__ __forceinline__ bool eval_sample(const VolumeDev& v, const TissueDev&
 // slower).
 // Called by whole warps; a lane without a ray passes r.ns = 0.
 constexpr unsigned kRayEnded = 0x7fffffffu;  // above any advance
-template <bool kDerived, bool kState, bool kCount, int kBS>
+template <bool kDerived, bool kState, int kBS>
 __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
                                              const RayDev& r, int skip, float inv_gmax, const float is[3],
-                                             float4& out, unsigned& dense, unsigned& evald, unsigned& shaded,
-                                             unsigned& interp, int* klast_out = nullptr, float* t_last = nullptr) {
+                                             float4& out, int* klast_out, float* t_last) {
     float C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f;
     float A_prev = 0.f;  // kState: A before the last evaluated sample
     int klast = -1;      // kState: last evaluated sample
     int k1 = -1;         // kState: first sample with A >= 1 (where the adjoint sweep must start
     float T1 = 1.f;      // when early termination is off) and the transmittance in front of it
     int k = 0;
-    unsigned ne = 0, nsh = 0, nip = 0;
-    const int bs = kBS ? kBS : v.bs;
     // the position of sample k, u0 + k du, carried by exact integer additions
     long long U[3] = {r.u0[0], r.u0[1], r.u0[2]};
     auto step = [&]() {
@@ -137,47 +131,28 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
             adv = 0u;
             if (!VR_CHECK(tp.status, (unsigned)i0[0] <= (unsigned)(v.n[0] - 2) &&
                                          (unsigned)i0[1] <= (unsigned)(v.n[1] - 2) &&
-                                         (unsigned)i0[2] <= (unsigned)(v.n[2] - 2))) {
+                                         (unsigned)i0[2] <= (unsigned)(v.n[2] - 2)))
                 adv = 1u;
-            } else if (skip) {
-                bool out = false;
-                if (kCount || !v.skipf) {
-                    const int bc[3] = {i0[0] >> bs, i0[1] >> bs, i0[2] >> bs};
-                    if (__ldg(v.empty + brick_index(v, bc))) {
-                        out = true;
-                        adv = (unsigned)(brick_exit_k_at(r, U, bc, 1 << bs, k, ns) - k);
-                    }
-                }
-                if (!out && v.skipf) {
-                    adv = __ldg(v.skipf + skip_index(i0[0], i0[1], i0[2], v.skip_cx, v.skip_by));
-                    if (kCount && adv) {
-                        ++ne;
-                        adv = 1u;
-                    }
-                }
-            }
+            else if (skip)
+                adv = __ldg(v.skipf + skip_index(i0[0], i0[1], i0[2], v.skip_cx, v.skip_by));
         }
-        // without counters adv is a distance in cells (samples when there is no field)
-        const unsigned m = __reduce_min_sync(0xffffffffu, adv);
+        const unsigned m = __reduce_min_sync(0xffffffffu, adv);  // a distance in cells
         if (m) {
             if (m == kRayEnded) break;
-            leap(kCount || !v.skipf ? (int)m : (int)((float)(m - 1u) * tp.leap_per_cell) + 1);
+            leap((int)((float)(m - 1u) * tp.leap_per_cell) + 1);
             continue;
         }
         if (adv) {
             step();
             continue;
         }
-        if (kCount) ++nip;
         float alpha, col[3], f[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) f[q] = cell_frac_at(U[q], v.n[q]);
         if (!eval_sample<kDerived, kBS>(v, tp, tf, f, i0, r.dir, inv_gmax, is, alpha, col)) {
-            if (kCount) ++ne;
             step();
             continue;
         }
-        if (kCount) ++nsh;
         const float wgt = (1.0f - A) * alpha;  // Eqs. 5-6
         fma2v(col[0], col[1], wgt, wgt, C0, C1);
         C2 = fmaf(col[2], wgt, C2);
@@ -190,23 +165,103 @@ __device__ __forceinline__ void march_gather(const VolumeDev& v, const TissueDev
             k1 = k;
             T1 = 1.0f - A_prev;
         }
-        if (kCount) ++ne;
         if (A >= tp.et_threshold) {
             ns = k + 1;
         }
         step();
     }
     out = make_float4(C0, C1, C2, A);
+    if (kState) {
+        // the adjoint sweep starts at the first sample with A >= min(et, 1): the stopping
+        // sample, or (early termination off) the first that made A reach 1
+        const int kl = ns - 1;
+        *klast_out = k1 >= 0 ? k1 : kl;
+        *t_last = k1 >= 0 ? T1 : ((klast == kl) ? 1.0f - A_prev : 1.0f - A);  // samples after klast: alpha 0
+    }
+}
+
+// The same march, the same image and ray state, for launches that want sample counters or
+// whose volume has no skip field. Evaluated samples are defined by the skip bricks (samples
+// outside bricks classified empty), so a lane walks brick by brick and sample by sample; in
+// step with the others it would stop at every brick any of them has to enter
+// (1080p of a 128^3 head 732 us in step, 629 each for itself).
+template <bool kDerived, bool kState, int kBS>
+__device__ __forceinline__ void march_count(const VolumeDev& v, const TissueDev& tp, const float4* __restrict__ tf,
+                                            const RayDev& r, int skip, float inv_gmax, const float is[3], float4& out,
+                                            unsigned& dense, unsigned& evald, unsigned& shaded, unsigned& interp,
+                                            int* klast_out = nullptr, float* t_last = nullptr) {
+    float C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f, A_prev = 0.f, T1 = 1.f;
+    int klast = -1, k1 = -1, k = 0, ns = r.ns;
+    unsigned ne = 0, nsh = 0, nip = 0;
+    const int bs = kBS ? kBS : v.bs;
+    int cur = -1;  // the brick whose flag `empty` is
+    bool empty = false;
+    long long U[3] = {r.u0[0], r.u0[1], r.u0[2]};
+    auto advance = [&](int m) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) U[q] += m == 1 ? r.du[q] : (long long)m * r.du[q];
+        k += m;
+    };
+    while (k < ns) {
+        int i0[3], bc[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            i0[q] = cell_index_at(U[q], v.n[q]);
+            bc[q] = i0[q] >> bs;
+        }
+        if (!VR_CHECK(tp.status, (unsigned)bc[0] < (unsigned)v.nb[0] && (unsigned)bc[1] < (unsigned)v.nb[1] &&
+                                     (unsigned)bc[2] < (unsigned)v.nb[2])) {
+            advance(1);
+            continue;
+        }
+        if (skip) {
+            const int bi = brick_index(v, bc);
+            if (bi != cur) {
+                cur = bi;
+                empty = __ldg(v.empty + bi) != 0;
+            }
+            if (empty) {
+                advance(brick_exit_k_at(r, U, bc, 1 << bs, k, ns) - k);
+                continue;
+            }
+            if (v.skipf && __ldg(v.skipf + skip_index(i0[0], i0[1], i0[2], v.skip_cx, v.skip_by))) {
+                ++ne;
+                advance(1);
+                continue;
+            }
+        }
+        ++nip;
+        ++ne;
+        float alpha, col[3], f[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) f[q] = cell_frac_at(U[q], v.n[q]);
+        if (eval_sample<kDerived, kBS>(v, tp, tf, f, i0, r.dir, inv_gmax, is, alpha, col)) {
+            ++nsh;
+            const float wgt = (1.0f - A) * alpha;  // Eqs. 5-6
+            fma2v(col[0], col[1], wgt, wgt, C0, C1);
+            C2 = fmaf(col[2], wgt, C2);
+            if (kState) {
+                A_prev = A;
+                klast = k;
+            }
+            A += wgt;
+            if (kState && k1 < 0 && A >= 1.0f) {
+                k1 = k;
+                T1 = 1.0f - A_prev;
+            }
+            if (A >= tp.et_threshold) ns = k + 1;
+        }
+        advance(1);
+    }
+    out = make_float4(C0, C1, C2, A);
     dense = (unsigned)ns;
     evald = ne;
     shaded = nsh;
     interp = nip;
-    if (kState) {
-        // the adjoint sweep starts at the first sample with A >= min(et, 1): the stopping
-        // sample, or (early termination off) the first that made A reach 1
-        const int kl = (int)dense - 1;
+    if (kState) {  // as march_gather
+        const int kl = ns - 1;
         *klast_out = k1 >= 0 ? k1 : kl;
-        *t_last = k1 >= 0 ? T1 : ((klast == kl) ? 1.0f - A_prev : 1.0f - A);  // samples after klast: alpha 0
+        *t_last = k1 >= 0 ? T1 : ((klast == kl) ? 1.0f - A_prev : 1.0f - A);
     }
 }
 

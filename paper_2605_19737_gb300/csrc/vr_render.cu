@@ -19,9 +19,17 @@ namespace {
 // Registers per thread: 64 for the derived-brick path (8 CTAs of 4 warps per SM:
 // equal at 1080p, 2.5 % faster on the 8-view 512^2 workload than 72), 72 when it also
 // records the ray state (CTAs of at most 4 warps, 7 per SM: 1.5 % faster than 80 at 6;
-// 64 spills ~100 bytes), 80 for the stencils. CTAs of 2, 4 or 8 warps (tile_pixel).
-template <bool kDerived, bool kState, bool kCount, int kBS>
-__global__ void __launch_bounds__(kState ? 128 : 256, kDerived ? (kState ? 7 : 4) : (kState ? 6 : 3))
+// 64 spills ~100 bytes), 80 for the stencils. CTAs of 2, 4 or 8 warps (tile_pixel), or of one.
+// kCount: 0 leaps, 1 counts (march_count), 2 counts with 128 registers, for launches of so few
+// rays that loads in flight per warp count more than warps (181x217x181 head with / without
+// curvature, us at 64 -> 128 registers: 64^2 1616 -> 785 / 421 -> 333, 256^2 824 -> 567 / 385 ->
+// 331, 400x300 811 -> 624 / 419 -> 345, 430^2 745 -> 748 / 428 -> 518: the line lies between the
+// last two).
+constexpr long long kFewRays = 28ll * 32 * kSMs;
+template <bool kDerived, bool kState, int kCount, int kBS>
+__global__ void __launch_bounds__(kState ? 128 : 256,
+                                  kCount == 2 ? (kState ? 4 : 2)
+                                              : kDerived ? (kState ? 7 : 4) : (kState ? 6 : 3))
     k_render_gather(const __grid_constant__ RenderLaunch L) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     int di, dj;
@@ -43,8 +51,11 @@ __global__ void __launch_bounds__(kState ? 128 : 256, kDerived ? (kState ? 7 : 4
     int kl = -1;
     float tl = 1.0f;
     if (!hit) r.ns = 0;
-    march_gather<kDerived, kState, kCount, kBS>(v, L.tp, tf, r, L.skip, inv_gmax, is, px, dense, evald, shaded,
-                                                    interp, &kl, &tl);
+    if (kCount)
+        march_count<kDerived, kState, kBS>(v, L.tp, tf, r, L.skip, inv_gmax, is, px, dense, evald, shaded, interp, &kl,
+                                           &tl);
+    else
+        march_gather<kDerived, kState, kBS>(v, L.tp, tf, r, L.skip, inv_gmax, is, px, &kl, &tl);
     if (inside) {
         const long long pix = ((long long)(L.cam_offset + cam) * L.H + j) * L.W + i;
         reinterpret_cast<float4*>(L.out)[pix] = px;
@@ -110,10 +121,12 @@ void launch_lanes_derived(const RenderLaunch& L, dim3 grid, cudaStream_t st) {
 
 template <bool kDerived, bool kState, int kBS>
 void launch_gather_count(const RenderLaunch& L, dim3 grid, int threads, cudaStream_t st) {
-    if (L.counters || L.ray_samples)
-        k_render_gather<kDerived, kState, true, kBS><<<grid, threads, 0, st>>>(L);
+    if (!(L.counters || L.ray_samples || (L.skip && !L.vol.skipf)))
+        k_render_gather<kDerived, kState, 0, kBS><<<grid, threads, 0, st>>>(L);
+    else if ((long long)L.W * L.H * L.n_cams > kFewRays)
+        k_render_gather<kDerived, kState, 1, kBS><<<grid, threads, 0, st>>>(L);
     else
-        k_render_gather<kDerived, kState, false, kBS><<<grid, threads, 0, st>>>(L);
+        k_render_gather<kDerived, kState, 2, kBS><<<grid, threads, 0, st>>>(L);
 }
 
 }  // namespace
@@ -164,6 +177,9 @@ cudaError_t launch_render_gather(const RenderLaunch& L0, int warps, cudaStream_t
     // the state-recording kernels are built for CTAs of at most 4 warps (72 registers,
     // 7 CTAs per SM); the image and the state do not depend on the CTA shape
     if (L.ray_state && warps > 4) warps = 4;
+    // launches of fewer CTAs than SMs (those with counters; the others had several lanes) get
+    // smaller ones (32^2 940 -> 741 us at 64 registers)
+    while (warps > 1 && (long long)L.W * L.H * L.n_cams < 32ll * warps * kSMs) warps >>= 1;
     const int tx = tile_packets_x(L.packet_w, warps);
     L.tile_w = tx * L.packet_w;
     L.tile_h = (warps / tx) * L.packet_h;
