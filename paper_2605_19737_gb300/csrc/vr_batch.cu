@@ -69,51 +69,61 @@ __device__ __forceinline__ void batch_body(const BatchLaunch& B) {
 }
 
 // kBS: the skip-brick size shared by every view, or 0 when the views mix sizes.
-template <bool kCount, int kBS>
-__global__ void __maxnreg__(72) k_render_batch_derived(const __grid_constant__ BatchLaunch B) {
+// kFew: a batch of few packets takes 128 registers, for more loads in flight per warp: the
+// three planes of the derived bricks cost a sparse ray twice the lines that records did, and a
+// small batch waits for them (one view of the 181x217x181 head with / without curvature, us at
+// 72 -> 128 registers: 64^2 1686 -> 770 / 478 -> 347, 256^2 867 -> 586 / 427 -> 360, 400x300
+// 791 -> 550 / 408 -> 348, 430^2 746 -> 716 / 422 -> 486: the line lies between the last two).
+template <bool kCount, bool kFew, int kBS>
+__global__ void __maxnreg__(kFew ? 128 : 72) k_render_batch_derived(const __grid_constant__ BatchLaunch B) {
     batch_body<true, kCount, kBS>(B);
 }
 
-template <bool kCount>
-__global__ void __launch_bounds__(256, 3) k_render_batch_mixed(const __grid_constant__ BatchLaunch B) {
+template <bool kCount, bool kFew>
+__global__ void __launch_bounds__(256, kFew ? 2 : 3) k_render_batch_mixed(const __grid_constant__ BatchLaunch B) {
     batch_body<false, kCount, 0>(B);
 }
 
-template <bool kCount>
-void launch_derived(const BatchLaunch& B, int ctas, int threads, int bs, cudaStream_t st) {
-    if (bs == 2)
-        k_render_batch_derived<kCount, 2><<<ctas, threads, 0, st>>>(B);
+template <bool kCount, bool kFew>
+void launch_variant(const BatchLaunch& B, int ctas, int threads, bool all_derived, int bs, cudaStream_t st) {
+    if (!all_derived)
+        k_render_batch_mixed<kCount, kFew><<<ctas, threads, 0, st>>>(B);
+    else if (bs == 2)
+        k_render_batch_derived<kCount, kFew, 2><<<ctas, threads, 0, st>>>(B);
     else if (bs == 3)
-        k_render_batch_derived<kCount, 3><<<ctas, threads, 0, st>>>(B);
+        k_render_batch_derived<kCount, kFew, 3><<<ctas, threads, 0, st>>>(B);
     else if (bs == 4)
-        k_render_batch_derived<kCount, 4><<<ctas, threads, 0, st>>>(B);
+        k_render_batch_derived<kCount, kFew, 4><<<ctas, threads, 0, st>>>(B);
     else
-        k_render_batch_derived<kCount, 0><<<ctas, threads, 0, st>>>(B);
+        k_render_batch_derived<kCount, kFew, 0><<<ctas, threads, 0, st>>>(B);
 }
 
 }  // namespace
 
-cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, int* per_sm) {
+bool batch_few(int packets) { return packets <= 28 * kSMs; }
+
+cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, bool few, int* per_sm) {
     // every variant of a family is held to the same registers, so one answers for all
-    return all_derived ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_render_batch_derived<false, 3>,
-                                                                       warps_per_block * 32, 0)
-                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_render_batch_mixed<false>,
-                                                                       warps_per_block * 32, 0);
+    auto kernel = all_derived ? (few ? k_render_batch_derived<false, true, 3> : k_render_batch_derived<false, false, 3>)
+                              : (few ? k_render_batch_mixed<false, true> : k_render_batch_mixed<false, false>);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, warps_per_block * 32, 0);
 }
 
 cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, bool all_derived, int bs,
                                 cudaStream_t st) {
     const int t = warps_per_block * 32;
-    // without skipping there is nothing to look ahead for either
-    const bool count = B.counters || !B.skip;
-    if (all_derived && count)
-        launch_derived<true>(B, ctas, t, bs, st);
-    else if (all_derived)
-        launch_derived<false>(B, ctas, t, bs, st);
-    else if (count)
-        k_render_batch_mixed<true><<<ctas, t, 0, st>>>(B);
-    else
-        k_render_batch_mixed<false><<<ctas, t, 0, st>>>(B);
+    const bool few = batch_few(B.n_work);
+    if (B.counters || !B.skip) {  // without skipping there is nothing to look ahead for either
+        if (few)
+            launch_variant<true, true>(B, ctas, t, all_derived, bs, st);
+        else
+            launch_variant<true, false>(B, ctas, t, all_derived, bs, st);
+    } else {
+        if (few)
+            launch_variant<false, true>(B, ctas, t, all_derived, bs, st);
+        else
+            launch_variant<false, false>(B, ctas, t, all_derived, bs, st);
+    }
     return cudaGetLastError();
 }
 

@@ -351,7 +351,10 @@ cudaError_t launch_channels_to_voxels(const float* dgrad, const int n[3], const 
 // bs: the skip-brick size (log2 cells) every view shares, or 0 when they differ.
 cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, bool all_derived, int bs,
                                 cudaStream_t st);
-cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, int* per_sm);
+// Whether a batch of that many packets takes the kernels for few rays, and the CTAs of a
+// kernel that an SM holds.
+bool batch_few(int packets);
+cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, bool few, int* per_sm);
 cudaError_t launch_render_staged(const RenderLaunch& L, int warps_per_block, int ctas, cudaStream_t st);
 // The staged design on the derived bricks (skip bricks of 4^3 or 8^3 cells, bs 2 or 3).
 cudaError_t launch_render_staged_derived(const RenderLaunch& L, int warps_per_block, int ctas, cudaStream_t st);

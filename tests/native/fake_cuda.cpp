@@ -283,7 +283,8 @@ cudaError_t launch_channels_to_voxels(const float*, const int*, const float*, fl
     return cudaSuccess;
 }
 cudaError_t launch_render_batch(const BatchLaunch&, int, int, bool, int, cudaStream_t) { return cudaSuccess; }
-cudaError_t batch_ctas_per_sm(int, bool, int* n) {
+bool batch_few(int) { return true; }
+cudaError_t batch_ctas_per_sm(int, bool, bool, int* n) {
     *n = 1;
     return cudaSuccess;
 }
