@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <string>
@@ -75,7 +76,7 @@ struct DevicePool;
 
 struct vr_ctx {
     int device = 0;
-    DevicePool* pool = nullptr;  // where its buffers come from, NULL: cudaMalloc
+    DevicePool* pool = nullptr;  // where its buffers may come from
     cudaStream_t stream = nullptr;
     std::string err;
     std::map<int, Volume*> vols;
@@ -142,20 +143,25 @@ vr_status cuda_fail(vr_ctx* c, cudaError_t e, const char* what) {
 // knows what it holds (vr_memory_used), can refuse to grow past a limit
 // (vr_set_memory_limit) and can be made to see an allocation fail (vr_debug_fail_alloc).
 // A refused allocation returns cudaErrorMemoryAllocation like a failed cudaMalloc.
-// They come from a CUDA memory pool that the contexts on a device share and that keeps what is
-// freed for the next allocation: opening a study makes eleven allocations and closing it eleven
-// frees (181x217x181: cudaMalloc 251 us and cudaFree 656 us, from the pool 4 and 5; load to
-// first 720p frame and close 2.44 -> 1.45 ms).
+// A process that opens study after study makes eleven allocations and eleven frees for each:
+// once a volume has been freed, they come from a CUDA memory pool that the contexts on a device
+// share while there are any, and that keeps what is freed for the next allocation (181x217x181: cudaMalloc 251 us and
+// cudaFree 656, from the pool 9 and 4; load to first 720p frame and close 2.44 -> 1.44 ms). A
+// first study is cudaMalloc's: the pool would grow for it in 600 us and shrink in 900 (2.3 ms
+// more for the first growth in a process).
 // What the pool keeps is bounded, and is not lost to others: the driver takes it back for any
 // cudaMalloc of the process that finds the device full, and the library when the last context
-// on the device is destroyed. A context with a memory limit has it released at once.
+// on the device is destroyed. A context with a memory limit does without.
 struct DevicePool {
     static constexpr size_t kSpareBytes = (size_t)2 << 30;
-    int device;
-    unsigned long long cuda_ctx;  // id of the CUDA context whose stream it is
-    cudaMemPool_t pool;
-    cudaStream_t stream;  // orders allocations and frees, and runs nothing
-    int users;            // library contexts
+    const int device;
+    const unsigned long long cuda_ctx;  // id of the CUDA context whose stream it is
+    int users = 1;                      // library contexts
+    std::atomic<bool> wanted{false};    // a volume has been freed
+    std::atomic<bool> ready{false};     // the rest is there
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t stream = nullptr;  // orders allocations and frees, and runs nothing
+    DevicePool(int d, unsigned long long c) : device(d), cuda_ctx(c) {}
 };
 std::mutex g_pools_mu;
 std::vector<DevicePool*>& device_pools() {
@@ -163,8 +169,7 @@ std::vector<DevicePool*>& device_pools() {
     return *pools;
 }
 
-// The pool of the current CUDA context's device, NULL where there can be none (allocations
-// are then cudaMalloc's).
+// The entry of the current CUDA context's device, NULL when that cannot be told.
 DevicePool* acquire_pool(int device, unsigned long long cuda_ctx) {
     if (cuda_ctx == 0) return nullptr;
     std::lock_guard<std::mutex> lock(g_pools_mu);
@@ -173,27 +178,44 @@ DevicePool* acquire_pool(int device, unsigned long long cuda_ctx) {
             ++p->users;
             return p;
         }
-    DevicePool n{device, cuda_ctx, nullptr, nullptr, 1};
+    device_pools().push_back(new DevicePool(device, cuda_ctx));
+    return device_pools().back();
+}
+
+// Makes the pool itself, or gives it up where there can be none: allocations then stay
+// cudaMalloc's.
+void start_pool(DevicePool* p) {
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    if (p->ready || !p->wanted) return;
+    p->wanted = false;
     int supported = 0;
-    cudaDeviceGetAttribute(&supported, cudaDevAttrMemoryPoolsSupported, device);
+    cudaDeviceGetAttribute(&supported, cudaDevAttrMemoryPoolsSupported, p->device);
     cudaMemPoolProps props;
     memset(&props, 0, sizeof props);
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = device;
+    props.location.id = p->device;
     unsigned long long all = ~0ull;  // Freeing bounds what is kept
-    if (!supported || cudaMemPoolCreate(&n.pool, &props) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
+    cudaMemPool_t pool = nullptr;
+    if (supported && cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &all) == cudaSuccess &&
+            cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) == cudaSuccess) {
+            p->pool = pool;
+            p->ready = true;
+        } else {
+            cudaMemPoolDestroy(pool);
+        }
     }
-    if (cudaMemPoolSetAttribute(n.pool, cudaMemPoolAttrReleaseThreshold, &all) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&n.stream, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaMemPoolDestroy(n.pool);
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    device_pools().push_back(new DevicePool(n));
-    return device_pools().back();
+    (void)cudaGetLastError();
+}
+
+// Gives back what the pool keeps beyond `spare` bytes.
+void trim_pool(const DevicePool& d, size_t spare) {
+    unsigned long long used = 0;
+    if (cudaStreamSynchronize(d.stream) == cudaSuccess &&
+        cudaMemPoolGetAttribute(d.pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+        cudaMemPoolTrimTo(d.pool, (size_t)used + spare);
+    (void)cudaGetLastError();
 }
 
 // Buffers still out (held back because no wait succeeded) stay valid past the pool's handle.
@@ -203,7 +225,7 @@ void release_pool(DevicePool* p) {
     if (--p->users) return;
     auto& pools = device_pools();
     pools.erase(std::find(pools.begin(), pools.end(), p));
-    if (current_cuda_context() == p->cuda_ctx) {  // else it went with its CUDA context
+    if (p->ready && current_cuda_context() == p->cuda_ctx) {  // else it went with its CUDA context
         cudaMemPoolDestroy(p->pool);
         cudaStreamDestroy(p->stream);
     }
@@ -221,7 +243,12 @@ cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
     if (ctx->mem_limit && bytes > ctx->mem_limit - std::min(ctx->mem_limit, ctx->mem_used))
         return cudaErrorMemoryAllocation;
     void* q = nullptr;
-    const bool pooled = ctx->pool && current_cuda_context() == ctx->pool->cuda_ctx;
+    bool pooled = ctx->pool && !ctx->mem_limit && (ctx->pool->ready || ctx->pool->wanted) &&
+                  current_cuda_context() == ctx->pool->cuda_ctx;
+    if (pooled && !ctx->pool->ready) {
+        start_pool(ctx->pool);
+        pooled = ctx->pool->ready;
+    }
     cudaError_t e;
     if (pooled) {
         e = cudaMallocFromPoolAsync(&q, bytes, ctx->pool->pool, ctx->pool->stream);
@@ -239,9 +266,8 @@ cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
 
 // Frees buffers of a context: Freeing fr(ctx); fr(p); fr(q); or, for one, dfree(ctx, p).
 // It first waits, once, for everything queued on the device. The context's stream alone would
-// not do: a caller's graph may hold a batch launch and be replayed on any stream. A buffer goes
-// back to the pool only after that wait succeeded; otherwise the context holds on to it, as
-// used, until one does.
+// not do: a caller's graph may hold a batch launch and be replayed on any stream. When the wait
+// fails the context holds on to the buffers, as used, until one succeeds.
 // The wait is the one that cudaFree makes, on a small buffer kept for it (measured: it ends
 // with the kernels and graph replays of every stream; 2 us with the next cudaMalloc when the
 // device is idle). cudaDeviceSynchronize fails, and invalidates the capture, while any thread
@@ -256,8 +282,9 @@ class Freeing {
             idle_ = cudaDeviceSynchronize() == cudaSuccess;
         }
         if (!ctx->marker && cudaMalloc(&ctx->marker, kMarkerBytes) != cudaSuccess) ctx->marker = nullptr;
-        idle_ = idle_ && ctx->pool && current_cuda_context() == ctx->pool->cuda_ctx;
         (void)cudaGetLastError();
+        // (a buffer of another CUDA context than the current one is held back too)
+        pool_ = idle_ && ctx->pool && ctx->pool->ready && current_cuda_context() == ctx->pool->cuda_ctx;
         if (idle_) {
             std::vector<void*> held;
             held.swap(ctx->held);
@@ -267,32 +294,28 @@ class Freeing {
     void operator()(void* p) {
         if (!p) return;
         const auto it = ctx_->allocs.find(p);  // everything was dalloc's
-        if (it->second.pooled && !idle_) {
+        const bool pooled = it->second.pooled;
+        if (!idle_ || (pooled && !pool_)) {
             ctx_->held.push_back(p);
             return;
         }
-        if (it->second.pooled) {
-            cudaFreeAsync(p, ctx_->pool->stream);
-            trim_ = true;
-        } else {
-            cudaFree(p);
-        }
+        if (pooled) cudaFreeAsync(p, ctx_->pool->stream);
+        else cudaFree(p);
+        trim_ = trim_ || pooled;
         ctx_->mem_used -= it->second.bytes;
         ctx_->allocs.erase(it);
     }
+    // A volume has been freed: the next one's buffers come from the pool.
+    void reopens() {
+        if (ctx_->pool && !ctx_->pool->ready && !ctx_->mem_limit) ctx_->pool->wanted = true;
+    }
     ~Freeing() {
-        if (!trim_) return;
-        const DevicePool& d = *ctx_->pool;
-        unsigned long long used = 0;
-        if (cudaStreamSynchronize(d.stream) == cudaSuccess &&
-            cudaMemPoolGetAttribute(d.pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
-            cudaMemPoolTrimTo(d.pool, (size_t)used + (ctx_->mem_limit ? 0 : DevicePool::kSpareBytes));
-        (void)cudaGetLastError();
+        if (trim_) trim_pool(*ctx_->pool, ctx_->mem_limit ? 0 : DevicePool::kSpareBytes);
     }
 
   private:
     vr_ctx* ctx_;
-    bool idle_, trim_ = false;
+    bool idle_, pool_, trim_ = false;
 };
 
 void dfree(vr_ctx* ctx, void* p) {
@@ -318,6 +341,7 @@ void free_volume(Freeing& fr, Volume* v) {
     fr(v->d_tf);
     fr(v->d_prefix);
     delete v;
+    fr.reopens();
 }
 
 void free_volume(vr_ctx* ctx, Volume* v) {

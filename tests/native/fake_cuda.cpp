@@ -30,7 +30,7 @@ std::vector<std::pair<char*, size_t>> g_spare;  // freed into the memory pool, t
 size_t g_capacity = ~(size_t)0;    // of the device
 std::set<char*> g_replayed;        // those the unknown work uses
 bool g_busy = false, g_fail_waits = false, g_capture = false, g_capture_valid = false;
-int g_violations = 0;
+int g_violations = 0, g_pool_allocs = 0;
 
 void device_done() {
     g_busy = false;
@@ -81,6 +81,7 @@ void fake_replay() {
 }
 void fake_fail_waits(int on) { g_fail_waits = on != 0; }
 int fake_violations() { return g_violations; }
+int fake_pool_allocs() { return g_pool_allocs; }
 void fake_capture(int on) { g_capture = on != 0, g_capture_valid = true; }
 int fake_capture_valid() { return g_capture_valid; }
 long long fake_held_bytes() { return (long long)held(); }
@@ -121,6 +122,7 @@ cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t keep) {
     return cudaSuccess;
 }
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) {
+    ++g_pool_allocs;
     for (size_t i = g_spare.size(); i-- > 0;)
         if (g_spare[i].second == n) {
             *p = g_spare[i].first;

@@ -39,9 +39,12 @@ class Lib:
     """One context of the fake library. fail_waits: every wait fails during the calls made
     through `freeing` (as on a stream under capture, or one that the caller has destroyed)."""
 
-    def __init__(self, lib, fail_waits=False):
+    def __init__(self, lib, fail_waits=False, reopens=True):
+        """reopens: a volume has been freed, after which buffers come from the pool."""
         self.lib, self.h, self.fail_waits = lib, ctypes.c_void_p(), fail_waits
         assert lib.vr_create(ctypes.byref(self.h), 0, None) == 0
+        if reopens:
+            self.ok(lib.vr_free_volume(self.h, self.load(3)))
 
     def ok(self, status):
         assert status == 0, self.lib.vr_last_error(self.h)
@@ -190,8 +193,8 @@ def test_freed_memory_is_there_for_others(lib):
 
 
 def test_what_is_kept_is_bounded(lib):
-    """A volume above the bound is given back at once, and so is everything of a context with a
-    memory limit."""
+    """A volume above the bound is given back at once; with a memory limit set, all of a volume
+    is, also one opened before."""
     c = Lib(lib)
     base = lib.fake_held_bytes()
     big = c.load(320)
@@ -199,7 +202,37 @@ def test_what_is_kept_is_bounded(lib):
     assert lib.fake_held_bytes() - base > 2 << 30
     c.ok(lib.vr_free_volume(c.h, big))
     assert lib.fake_held_bytes() - base <= 2 << 30
+    vid = c.load(20)
     c.ok(lib.vr_set_memory_limit(c.h, ctypes.c_ulonglong(1 << 40)))
-    c.ok(lib.vr_free_volume(c.h, c.load(20)))
+    c.ok(lib.vr_free_volume(c.h, vid))
     assert lib.fake_held_bytes() <= base + (1 << 20)
     c.close()
+
+
+def test_pool_from_the_second_study_on(lib):
+    """A context that opens one study allocates as without a pool; one that opens another, and
+    any beside it, from the pool; one with a memory limit never."""
+    before = lib.fake_pool_allocs()
+    c, d = Lib(lib, reopens=False), Lib(lib, reopens=False)
+    vid = c.open(20)
+    c.batch(vid)
+    assert lib.fake_pool_allocs() == before
+    c.ok(lib.vr_free_volume(c.h, vid))
+    assert lib.fake_pool_allocs() == before
+    c.open(20)
+    one = lib.fake_pool_allocs()
+    assert one > before
+    d.open(20)
+    assert lib.fake_pool_allocs() > one
+    e = Lib(lib, reopens=False)
+    e.ok(lib.vr_set_memory_limit(e.h, ctypes.c_ulonglong(1 << 40)))
+    two = lib.fake_pool_allocs()
+    e.ok(lib.vr_free_volume(e.h, e.open(20)))
+    e.open(20)
+    assert lib.fake_pool_allocs() == two
+    for x in (c, d, e):
+        x.close()
+    f = Lib(lib, reopens=False)  # the last context has ended: as in a new process
+    f.open(20)
+    assert lib.fake_pool_allocs() == two
+    f.close()

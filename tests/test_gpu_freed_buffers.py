@@ -35,6 +35,7 @@ def test_replay_on_another_stream_outlives_its_volume(torch):
     cams = camera_array([orbit_camera(DIMS, (1, 1, 1), 15.0 * k, 10.0, width=W, height=H) for k in range(n)])
     side, elsewhere = torch.cuda.Stream(), torch.cuda.Stream()
     with pkg.Context(0) as ctx, pkg.Context(0, stream=side) as other:
+        ctx.free_volume(_open(ctx, 0))  # the library keeps freed memory from here on
         vid = _open(ctx, 0)
         outs = [torch.zeros((H, W, 4), device="cuda") for _ in range(n)]
         bid = ctx.batch_create([(vid, cams[k], outs[k], W, H) for k in range(n)])
@@ -81,6 +82,7 @@ def test_capture_on_another_thread_stays_valid(torch):
 
     stream = torch.cuda.Stream()
     with pkg.Context(0, stream=stream) as ctx:
+        ctx.free_volume(_open(ctx, 0))  # the library keeps freed memory from here on
         vid = _open(ctx, 0)
         t = threading.Thread(target=capture)
         t.start()
@@ -104,6 +106,7 @@ def test_freed_memory_is_there_for_torch(torch):
     dims = (200, 200, 200)
     cams = camera_array([orbit_camera(dims, (1, 1, 1), 20.0, 10.0, width=64, height=48)])
     with pkg.Context(0) as ctx:
+        ctx.free_volume(_open(ctx, 0))  # the library keeps freed memory from here on
         vid = _open(ctx, 0, dims)
         want = ctx.render(vid, cams, 64, 48).cpu()
         used = ctx.memory_used()
