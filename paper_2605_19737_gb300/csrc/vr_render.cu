@@ -439,6 +439,8 @@ __global__ void __launch_bounds__(256, 3) k_render_staged_derived(const __grid_c
         int k = 0, kstop = -1, cur = -1, bc[3] = {0, 0, 0};
         float C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f;
         unsigned ne = 0, nsh = 0, nip = 0;
+        // the position of sample k, u0 + k du, carried by exact integer additions
+        long long U[3] = {r.u0[0], r.u0[1], r.u0[2]};
         while (true) {
             while (live && cur < 0) {  // this lane's next sample outside empty bricks
                 if (k >= r.ns) {
@@ -446,22 +448,21 @@ __global__ void __launch_bounds__(256, 3) k_render_staged_derived(const __grid_c
                     break;
                 }
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    int i0;
-                    float f;
-                    sample_cell(r, q, k, v.n[q], i0, f);
-                    bc[q] = i0 >> kBS;
-                }
+                for (int q = 0; q < 3; ++q) bc[q] = cell_index_at(U[q], v.n[q]) >> kBS;
                 if (!VR_CHECK(tp.status, (unsigned)bc[0] < (unsigned)v.nb[0] && (unsigned)bc[1] < (unsigned)v.nb[1] &&
                                              (unsigned)bc[2] < (unsigned)v.nb[2])) {
                     live = false;
                     break;
                 }
                 const int bi = brick_index(v, bc);
-                if (L.skip && __ldg(v.empty + bi))
-                    k = brick_exit_k(r, bc, B, k, r.ns);
-                else
+                if (L.skip && __ldg(v.empty + bi)) {
+                    const int to = brick_exit_k_at(r, U, bc, B, k, r.ns);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) U[q] += (long long)(to - k) * r.du[q];
+                    k = to;
+                } else {
                     cur = bi;
+                }
             }
             const unsigned key = live ? brick_key(bc, eb) : 0xffffffffu;
             const unsigned mk = __reduce_min_sync(0xffffffffu, key);
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(256, 3) k_render_staged_derived(const __grid_c
                     float f[3];
 #pragma unroll
                     for (int q = 0; q < 3; ++q) {
-                        sample_cell(r, q, k, v.n[q], i0[q], f[q]);
+                        i0[q] = cell_index_at(U[q], v.n[q]);
                         b2[q] = i0[q] >> kBS;
                     }
                     if (b2[0] != sc[0] || b2[1] != sc[1] || b2[2] != sc[2]) {
@@ -505,6 +506,8 @@ __global__ void __launch_bounds__(256, 3) k_render_staged_derived(const __grid_c
                         done_sample = __ldg(v.skipf + skip_index(i0[0], i0[1], i0[2], v.skip_cx, v.skip_by)) != 0;
                     if (!done_sample) {
                         ++nip;
+#pragma unroll
+                        for (int q = 0; q < 3; ++q) f[q] = cell_frac_at(U[q], v.n[q]);
                         float fld[10];
                         derived_channels_smem<0, 4>(sbrick, der_layout(kBS), lx, ly, lz, f[0], f[1], f[2], fld);
                         if (tp.gk != 0.0f) {
@@ -535,6 +538,8 @@ __global__ void __launch_bounds__(256, 3) k_render_staged_derived(const __grid_c
                         live = false;
                         break;
                     }
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) U[q] += r.du[q];
                 }
             }
         }
