@@ -483,7 +483,11 @@ vr_status vr_memory_used(vr_ctx* ctx, unsigned long long* bytes);
  * would: the call that needed it returns VR_ERR_OOM and releases nothing it did
  * not allocate. Derived bricks are optional: a precompute that cannot get them
  * under the cap renders from the per-sample stencils instead (same images within
- * rounding). Lowering the cap below the current use frees nothing. */
+ * rounding). So are the skip fields (5 bytes per cell with what they are made from): a
+ * precompute that cannot get one renders by the brick flags, and any other allocation
+ * that finds no room, under a cap or on a full device, takes theirs until the volumes'
+ * next precompute (same images, slower). Lowering the cap below the current use frees
+ * nothing. */
 vr_status vr_set_memory_limit(vr_ctx* ctx, unsigned long long bytes);
 
 /* Fault injection for the out-of-memory paths (host side; nothing faults on the

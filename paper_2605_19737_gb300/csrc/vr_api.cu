@@ -42,7 +42,8 @@ struct Volume {
     float* d_vbricks = nullptr;
     float* d_dbricks = nullptr;  // derived bricks (voxel-wise I, gradient, Hessian) or nullptr
     uint32_t* d_cellq = nullptr;  // after the morphology precompute: per-cell quantised min/max
-    uint8_t* d_skip = nullptr;    // and the skip field under the current transfer function, with its scratch
+    uint8_t* d_skip = nullptr;    // and the skip field under the current transfer function, with its scratch;
+                                  // both or neither
     float* d_smax = nullptr;  // per-scale max Hessian norm (8 floats)
     float* d_ch2 = nullptr;   // second channel: [0, 2) its I_min, I_max, [4, 8) its VolConst
     bool v_ready = false;     // d_vessel holds a complete second channel (vesselness or a modality)
@@ -106,8 +107,9 @@ struct vr_ctx {
     };
     std::unordered_map<void*, Held> allocs;  // device buffers
     std::vector<void*> held;                 // those to be freed after a wait that succeeds (Freeing)
-    size_t mem_used = 0;                     // their bytes, and the marker's
-    void* marker = nullptr;                  // freed and allocated anew as a wait for the device (Freeing)
+    size_t mem_used = 0;                     // their bytes
+    void* marker = nullptr;                  // freed and allocated anew as a wait for the device (Freeing),
+                                             // not counted
     size_t mem_limit = 0;                      // 0: no limit beyond the device's
     long long fail_after = -1;                 // >= 0: allocations left before an injected failure
 };
@@ -232,23 +234,16 @@ void release_pool(DevicePool* p) {
     delete p;
 }
 
-template <class T>
-cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
-    *p = nullptr;
-    if (ctx->fail_after == 0) {
-        ctx->fail_after = -1;  // one injected failure, then allocation behaves normally
-        return cudaErrorMemoryAllocation;
-    }
-    if (ctx->fail_after > 0) --ctx->fail_after;
+cudaError_t allocate(vr_ctx* ctx, void** p, size_t bytes) {
     if (ctx->mem_limit && bytes > ctx->mem_limit - std::min(ctx->mem_limit, ctx->mem_used))
         return cudaErrorMemoryAllocation;
-    void* q = nullptr;
     bool pooled = ctx->pool && !ctx->mem_limit && (ctx->pool->ready || ctx->pool->wanted) &&
                   current_cuda_context() == ctx->pool->cuda_ctx;
     if (pooled && !ctx->pool->ready) {
         start_pool(ctx->pool);
         pooled = ctx->pool->ready;
     }
+    void* q = nullptr;
     cudaError_t e;
     if (pooled) {
         e = cudaMallocFromPoolAsync(&q, bytes, ctx->pool->pool, ctx->pool->stream);
@@ -260,8 +255,30 @@ cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes) {
     if (e != cudaSuccess) return e;
     ctx->allocs[q] = {bytes, pooled};
     ctx->mem_used += bytes;
-    *p = static_cast<T*>(q);
+    *p = q;
     return cudaSuccess;
+}
+
+bool drop_skip_fields(vr_ctx* ctx, size_t bytes);
+
+// optional: the caller does without the buffer when it is refused; for another, skip fields
+// make room.
+template <class T>
+cudaError_t dalloc(vr_ctx* ctx, T** p, size_t bytes, bool optional = false) {
+    *p = nullptr;
+    if (ctx->fail_after == 0) {
+        ctx->fail_after = -1;  // one injected failure, then allocation behaves normally
+        return cudaErrorMemoryAllocation;
+    }
+    if (ctx->fail_after > 0) --ctx->fail_after;
+    void* q = nullptr;
+    cudaError_t e = allocate(ctx, &q, bytes);
+    if (e == cudaErrorMemoryAllocation && !optional) {
+        (void)cudaGetLastError();
+        if (drop_skip_fields(ctx, bytes)) e = allocate(ctx, &q, bytes);
+    }
+    if (e == cudaSuccess) *p = static_cast<T*>(q);
+    return e;
 }
 
 // Frees buffers of a context: Freeing fr(ctx); fr(p); fr(q); or, for one, dfree(ctx, p).
@@ -309,6 +326,7 @@ class Freeing {
     void reopens() {
         if (ctx_->pool && !ctx_->pool->ready && !ctx_->mem_limit) ctx_->pool->wanted = true;
     }
+    bool idle() const { return idle_; }
     ~Freeing() {
         if (trim_) trim_pool(*ctx_->pool, ctx_->mem_limit ? 0 : DevicePool::kSpareBytes);
     }
@@ -347,6 +365,38 @@ void free_volume(Freeing& fr, Volume* v) {
 void free_volume(vr_ctx* ctx, Volume* v) {
     Freeing fr(ctx);
     free_volume(fr, v);
+}
+
+// Gives up every skip field of the context, and the cell ranges they are made from: the images
+// do not need them, and a context at its memory limit, or on a full device, held less before
+// there were fields (1 byte per cell and scratch). Renders then skip by the brick flags until the
+// volume's next precompute. Batches see it in their view tables. False when there was none, or
+// when `bytes` would not fit under the limit all the same.
+bool drop_skip_fields(vr_ctx* ctx, size_t bytes) {
+    size_t held = 0;
+    for (auto& kv : ctx->vols)
+        if (kv.second->d_skip)
+            held += ctx->allocs[kv.second->d_skip].bytes + ctx->allocs[kv.second->d_cellq].bytes;
+    if (!held || (ctx->mem_limit && ctx->mem_used - held + bytes > ctx->mem_limit)) return false;
+    Freeing fr(ctx);  // (a batch launch may be under way)
+    if (!fr.idle()) return false;
+    for (auto& kv : ctx->batches) {
+        Batch* b = kv.second;
+        for (ViewDev& v : b->table) v.vol.skipf = nullptr;
+        if (cudaMemcpyAsync(b->d_views, b->table.data(), sizeof(ViewDev) * b->table.size(), cudaMemcpyHostToDevice,
+                            ctx->stream) != cudaSuccess ||
+            cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+    }
+    for (auto& kv : ctx->vols) {
+        Volume* v = kv.second;
+        fr(v->d_cellq);
+        fr(v->d_skip);
+        v->d_cellq = nullptr, v->d_skip = nullptr;
+    }
+    return true;
 }
 
 Volume* get_vol(vr_ctx* ctx, int id) {
@@ -434,14 +484,12 @@ vr_status rebuild_bricks(vr_ctx* ctx, Volume* v) {
     return VR_OK;
 }
 
-// Brick skip flags and (once the morphology is precomputed) the per-cell skip field
-// under the volume's current transfer function. Scratch: tf_w + 1 prefix counts, then
-// tf_w column limits.
+// Brick skip flags and (once the morphology is precomputed, if it has one) the per-cell skip
+// field under the volume's current transfer function.
 vr_status classify_volume(vr_ctx* ctx, Volume* v) {
-    int* limits = v->d_prefix + v->tp.tf_w + 1;
     if (v->d_skip)
         CK(launch_skip_field(v->d_cellq, v->n, v->d_grid, v->nbricks, v->d_tf, v->tp.tf_w, v->tp.tf_h, v->d_prefix,
-                             limits, v->d_empty, skip_store(v->d_skip, v->n), ctx->stream),
+                             v->d_empty, skip_store(v->d_skip, v->n), ctx->stream),
            "classify bricks and cells");
     else
         CK(launch_classify(v->d_grid, v->nbricks, v->d_tf, v->tp.tf_w, v->tp.tf_h, v->d_empty, v->d_prefix,
@@ -479,7 +527,6 @@ vr_status vr_create(vr_ctx** out, int device, void* cuda_stream) {
     if (e == cudaSuccess) {
         // d_work next to it, not from the pool: freeing the marker would else give its page
         // back and take 40 us, allocating it again 55
-        ctx->mem_used += kMarkerBytes;
         e = dalloc(ctx, &ctx->d_work, 64 * sizeof(unsigned));
         ctx->pool = acquire_pool(device, current_cuda_context());
     }
@@ -671,12 +718,23 @@ vr_status vr_precompute_morphology(vr_ctx* ctx, int vol_id, const float* h_sigma
             v->d_dbricks = nullptr;  // fall back to the per-sample stencils
         }
     }
-    // per-cell min/max (4 B per cell) and the skip field (1 B per cell + scratch), for either path
-    if (!v->d_cellq) CK(dalloc(ctx, &v->d_cellq, sizeof(uint32_t) * cellq_cells(v->n)), "cell grid");
-    if (!v->d_skip) CK(dalloc(ctx, &v->d_skip, skip_store_bytes(v->n)), "skip field");
+    // per-cell min/max (4 B per cell) and the skip field (1 B per cell + scratch), for either
+    // path; without room for both, renders skip by the brick flags
+    if (!v->d_cellq) {
+        cudaError_t e = dalloc(ctx, &v->d_cellq, sizeof(uint32_t) * cellq_cells(v->n), true);
+        if (e == cudaSuccess) {
+            e = dalloc(ctx, &v->d_skip, skip_store_bytes(v->n), true);
+            if (e != cudaSuccess) {
+                dfree(ctx, v->d_cellq);
+                v->d_cellq = nullptr;
+            }
+        }
+        if (e != cudaSuccess && e != cudaErrorMemoryAllocation) CK(e, "skip field");
+        (void)cudaGetLastError();
+    }
     if (v->d_dbricks)
         CK(launch_make_derived(v->d_norm, v->n, v->nb, v->bs, v->s, v->d_dbricks, ctx->stream), "derived bricks");
-    CK(launch_cell_minmax(v->d_norm, v->n, v->d_cellq, ctx->stream), "cell min/max");
+    if (v->d_cellq) CK(launch_cell_minmax(v->d_norm, v->n, v->d_cellq, ctx->stream), "cell min/max");
     if (v->params_ready) {
         vr_status cs = classify_volume(ctx, v);
         if (cs != VR_OK) return cs;
@@ -745,7 +803,7 @@ vr_status vr_set_tissue_params(vr_ctx* ctx, int vol_id, const vr_tissue_params* 
         dfree(ctx, v->d_prefix);
         v->d_prefix = nullptr;
         v->prefix_cap = 0;
-        CK(dalloc(ctx, &v->d_prefix, sizeof(int) * (2 * (size_t)tp->tf_w + 1)), "classification scratch");
+        CK(dalloc(ctx, &v->d_prefix, sizeof(int) * ((size_t)tp->tf_w + 1)), "classification scratch");
         v->prefix_cap = tp->tf_w + 1;
     }
     CK(cudaMemcpyAsync(v->d_tf, tp->tf, bytes, tp->tf_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -1126,6 +1184,7 @@ vr_status vr_render_backward(vr_ctx* ctx, int vol_id, const vr_camera* h_cams, i
     BackwardLaunch B;
     memset(&B, 0, sizeof B);
     fill_launch(B.r, v, W, H, skip);
+    B.r.vol.skipf = nullptr;  // not read, and an allocation below may give the fields up
     const bool staged = opts && opts->kernel == VR_KERNEL_STAGED;
     if (staged || (opts && opts->kernel == VR_KERNEL_GATHER_STENCIL)) B.r.vol.dbricks = nullptr;
     B.r.packet_w = opts ? opts->packet_w : 4;

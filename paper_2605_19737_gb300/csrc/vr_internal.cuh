@@ -99,13 +99,15 @@ struct SkipStore {
     uint32_t* block_bits; // [bz][by][bwx], bit set = 4^3 block empty
     uint4* block_dist;    // [bz][by][bwx] distance in blocks to the nearest non-empty block, capped,
                           // as four bit planes of 32 blocks
+    int* limits;          // [kMaxTableWidth] the table's column limits
 };
+constexpr int kMaxTableWidth = 4096;
 inline size_t skip_store_bytes(const int n[3]) {
     const SkipDims d = skip_dims(n);
     const size_t f = (size_t)d.bz * d.by * d.cx * 16;
     const size_t c = ((size_t)d.cz * d.cy * d.wx * 4 + 15) & ~(size_t)15;
     const size_t b = ((size_t)d.bz * d.by * d.bwx * 4 + 15) & ~(size_t)15;
-    return f + c + b + (size_t)d.bz * d.by * d.bwx * 16;
+    return f + c + b + (size_t)d.bz * d.by * d.bwx * 16 + sizeof(int) * kMaxTableWidth;
 }
 inline SkipStore skip_store(uint8_t* p, const int n[3]) {
     const SkipDims d = skip_dims(n);
@@ -117,6 +119,8 @@ inline SkipStore skip_store(uint8_t* p, const int n[3]) {
     s.block_bits = reinterpret_cast<uint32_t*>(p);
     p += ((size_t)d.bz * d.by * d.bwx * 4 + 15) & ~(size_t)15;
     s.block_dist = reinterpret_cast<uint4*>(p);
+    p += (size_t)d.bz * d.by * d.bwx * 16;
+    s.limits = reinterpret_cast<int*>(p);
     return s;
 }
 constexpr int kSMs = 152;
@@ -316,10 +320,10 @@ cudaError_t launch_classify(const uint16_t* grid, long long nbricks, const float
 // 16 bits: [nz - 1][ny - 1][cellq_pitch(nx)].
 cudaError_t launch_cell_minmax(const float* norm, const int n[3], uint32_t* cellq, cudaStream_t st);
 // The skip field, and the brick flags of launch_classify, under a transfer function
-// (scratch: tf_w + 1 and tf_w ints).
+// (prefix_scratch: tf_w + 1 ints).
 cudaError_t launch_skip_field(const uint32_t* cellq, const int n[3], const uint16_t* grid, long long nbricks,
-                              const float* tf, int tf_w, int tf_h, int* prefix_scratch, int* limit_scratch,
-                              uint8_t* empty, const SkipStore& s, cudaStream_t st);
+                              const float* tf, int tf_w, int tf_h, int* prefix_scratch, uint8_t* empty,
+                              const SkipStore& s, cudaStream_t st);
 
 // Multi-scale vesselness of `norm` into V (both nvox floats); tmp_a and tmp_b are
 // nvox floats of scratch each, smax receives each scale's max Hessian norm.

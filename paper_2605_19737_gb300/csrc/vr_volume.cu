@@ -760,17 +760,17 @@ cudaError_t launch_cell_minmax(const float* norm, const int n[3], uint32_t* cell
 }
 
 cudaError_t launch_skip_field(const uint32_t* cellq, const int n[3], const uint16_t* grid, long long nbricks,
-                              const float* tf, int tf_w, int tf_h, int* prefix_scratch, int* limit_scratch,
-                              uint8_t* empty, const SkipStore& s, cudaStream_t st) {
+                              const float* tf, int tf_w, int tf_h, int* prefix_scratch, uint8_t* empty,
+                              const SkipStore& s, cudaStream_t st) {
     const SkipDims d = skip_dims(n);
     constexpr int TC = 32 - 2 * kCellErosions, TB = 32 - 2 * kBlockErosions;
     const float* tf1 = tf_h == 1 && tf_w <= 1024 ? tf : nullptr;
-    if (!tf1) k_tf_alpha_prefix<<<1, 1024, 0, st>>>(tf, tf_w, tf_h, prefix_scratch, limit_scratch);
+    if (!tf1) k_tf_alpha_prefix<<<1, 1024, 0, st>>>(tf, tf_w, tf_h, prefix_scratch, s.limits);
     const int layers = (d.cz + 15) / 16;
     const long long per_layer = (long long)d.wx * d.by * 256;
     const long long more = (nbricks + per_layer - 1) / per_layer;
     k_cell_bits<<<dim3(d.wx, d.by, layers + (unsigned)(more < 4 ? more : 4)), 256, 0, st>>>(
-        cellq, d, cellq_pitch(n[0]), limit_scratch, tf1, tf_w, s.cell_bits, reinterpret_cast<uint8_t*>(s.block_bits),
+        cellq, d, cellq_pitch(n[0]), s.limits, tf1, tf_w, s.cell_bits, reinterpret_cast<uint8_t*>(s.block_bits),
         layers, grid, nbricks, empty);
     const dim3 tiles(d.wx, (d.cy + TC - 1) / TC, (d.cz + TC - 1) / TC);
     if ((long long)tiles.x * tiles.y * tiles.z <= kSMs) {

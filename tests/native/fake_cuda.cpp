@@ -255,7 +255,7 @@ cudaError_t launch_cell_minmax(const float*, const int*, uint32_t* cellq, cudaSt
     written(cellq);
     return cudaSuccess;
 }
-cudaError_t launch_skip_field(const uint32_t*, const int*, const uint16_t*, long long, const float*, int, int, int*, int*,
+cudaError_t launch_skip_field(const uint32_t*, const int*, const uint16_t*, long long, const float*, int, int, int*,
                               uint8_t*, const SkipStore&, cudaStream_t) {
     return cudaSuccess;
 }
