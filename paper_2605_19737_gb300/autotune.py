@@ -6,13 +6,14 @@ Times candidates on the caller's own workload with CUDA events (median of
 
 * tune_render: one vr_render call (a view or several cameras of one volume) over
   skip-brick edges of 4, 8 or 16 cells (vr_set_brick_size), warp packets of 4x8,
-  8x4 or 16x2 rays and CTAs of 2, 4 or 8 warps (the CTA tile: 8x8 .. 16x16 pixels).
+  8x4 or 16x2 rays and CTAs of 2, 4 or 8 warps (the CTA tile: 8x8 .. 16x16 pixels);
+  over the edges alone where a launch has so few rays that it takes a shape of its own.
 * tune_batch: the batched persistent renderer over packet shapes 4x8, 8x4, 16x2
   and 32x1, 2, 4 or 8 warps per CTA, and optionally the skip-brick edge of the
   batch's volumes; the grid always fills the SMs at the kernel's resident-CTA
   occupancy.
 
-Changing the brick size rebuilds a volume's grid, cell grid and derived bricks;
+Changing the brick size rebuilds a volume's grid and derived bricks;
 the caller passes `prepare(cells)`, which sets the size on its volumes and
 re-runs their precompute and tissue parameters (and vr_batch_update for a batch).
 The images do not depend on any of these choices.
@@ -24,6 +25,10 @@ import os
 DEFAULT_CANDIDATES = [(pw, w) for pw in (4, 8, 16, 32) for w in (2, 4, 8)]
 RENDER_CANDIDATES = [(pw, w) for pw in (4, 8, 16) for w in (2, 4, 8)]
 BRICK_SIZES = (4, 8, 16)
+DEFAULT_SHAPE = (4, 4)
+# vr_render gives each ray several lanes, whatever the launch shape asked for, in launches of up
+# to this many rays (and of up to 64 cameras)
+SHAPELESS_RAYS, LAUNCH_CAMERAS = 200000, 64
 
 
 def default_cache_path():
@@ -105,10 +110,13 @@ def tune_render(ctx, vol, cams, W, H, key, prepare=None, bricks=BRICK_SIZES, can
     out = out if out is not None else torch.empty((n, H, W, 4), device="cuda:%d" % ctx.device)
     if prepare is None:
         bricks = (None,)
+    if not candidates:
+        shapeless = W * H * min(n, LAUNCH_CAMERAS) <= SHAPELESS_RAYS
+        candidates = [DEFAULT_SHAPE] if shapeless else RENDER_CANDIDATES
 
     def launch(pw, w):
         ctx.render(vol, cams, W, H, out=out, kernel=VR_KERNEL_GATHER, packet_w=pw, warps_per_block=w)
-    return _search(ctx, key, cache_path, force, bricks, prepare, candidates or RENDER_CANDIDATES, launch, reps)
+    return _search(ctx, key, cache_path, force, bricks, prepare, candidates, launch, reps)
 
 
 def tune_batch(ctx, batch, key, candidates=None, reps=5, cache_path=None, force=False, prepare=None,
