@@ -62,6 +62,7 @@ struct Batch {
     int* d_prefix = nullptr;        // 4 packet shapes x n_views
     int n_work[4] = {0, 0, 0, 0};   // packets per packet shape (packet_w = 4, 8, 16, 32)
     bool all_derived = false;       // every view's volume has derived bricks
+    bool curved = false;            // some view has a curvature term
     int bs = 3;                     // the skip-brick size all views share, 0 when they differ
     std::map<std::pair<int, int>, cudaGraphExec_t> graphs;  // (packet_w, warps) -> graph
 };
@@ -95,7 +96,7 @@ struct vr_ctx {
     unsigned* d_work = nullptr;   // [0]: staged-kernel work counter, [1]: status word, [kParamSums..]:
                                   // five doubles, the uniform gradients' sums of a backward
     int staged_ctas[2][17] = {};   // resident CTAs per SM by (vesselness, warps per block)
-    int batch_ctas[2][2][17] = {}; // resident batch-kernel CTAs per SM by (all derived, few rays, warps per block)
+    int batch_ctas[3][17] = {};    // resident batch-kernel CTAs per SM by (kind, warps per block)
     size_t derived_budget = kDerivedBudgetBytes;  // largest derived-brick store precompute builds
     std::map<int, Batch*> batches;
     int next_batch = 1;
@@ -1276,7 +1277,7 @@ vr_status batch_upload(vr_ctx* ctx, Batch* b) {
         }
         b->n_work[si] = acc;
     }
-    bool all_derived = true;
+    bool all_derived = true, curved = false;
     int bs = -1;
     for (int i = 0; i < n; ++i) {
         const vr_view& vw = b->views[i];
@@ -1296,14 +1297,16 @@ vr_status batch_upload(vr_ctx* ctx, Batch* b) {
         d.H = vw.H;
         d.rc = L.rc;
         all_derived = all_derived && L.vol.dbricks != nullptr;
+        curved = curved || L.tp.gk != 0.0f;
         bs = (bs < 0 || bs == v->bs) ? v->bs : 0;
     }
-    if (all_derived != b->all_derived || bs != b->bs) {
+    if (all_derived != b->all_derived || curved != b->curved || bs != b->bs) {
         // the captured graphs launch another kernel variant
         if (ctx->graph_stream) CK(cudaStreamSynchronize(ctx->graph_stream), "batch: graph sync");
         for (auto& gx : b->graphs) cudaGraphExecDestroy(gx.second);
         b->graphs.clear();
         b->all_derived = all_derived;
+        b->curved = curved;
         b->bs = bs;
     }
     CK(cudaMemcpyAsync(b->d_views, b->table.data(), sizeof(ViewDev) * n, cudaMemcpyHostToDevice, ctx->stream),
@@ -1327,9 +1330,9 @@ vr_status batch_enqueue(vr_ctx* ctx, Batch* b, const vr_render_opts& o, vr_count
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device), "batch: SM count");
     const int warps = batch_warps(b->n_work[si], o.warps_per_block, sms);
-    const bool few = batch_few(b->n_work[si]);
-    int& per_sm = ctx->batch_ctas[b->all_derived][few][warps];
-    if (per_sm == 0) CK(batch_ctas_per_sm(warps, b->all_derived, few, &per_sm), "batch: occupancy");
+    const BatchKind kind = batch_kind(b->n_work[si], b->all_derived, b->curved);
+    int& per_sm = ctx->batch_ctas[(int)kind][warps];
+    if (per_sm == 0) CK(batch_ctas_per_sm(warps, kind, &per_sm), "batch: occupancy");
     if (per_sm < 1) return fail(ctx, VR_ERR_INVALID_ARG, "batch: kernel does not fit on an SM");
     BatchLaunch B;
     memset(&B, 0, sizeof B);
@@ -1347,7 +1350,7 @@ vr_status batch_enqueue(vr_ctx* ctx, Batch* b, const vr_render_opts& o, vr_count
     if (ctas > need) ctas = need;
     if (ctas < 1) ctas = 1;
     CK(cudaMemsetAsync(ctx->d_work + 2, 0, sizeof(unsigned), st), "batch: reset work counter");
-    CK(launch_render_batch(B, warps, ctas, b->all_derived, b->bs, st), "batch kernel");
+    CK(launch_render_batch(B, warps, ctas, kind, b->bs, st), "batch kernel");
     return VR_OK;
 }
 
@@ -1442,9 +1445,9 @@ vr_status vr_batch_render_graph(vr_ctx* ctx, int batch_id, const vr_render_opts*
         int sms = 0;
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device), "batch: SM count");
         const int work = b->n_work[shape_index(o.packet_w)], warps = batch_warps(work, o.warps_per_block, sms);
-        const bool few = batch_few(work);
-        int& per_sm = ctx->batch_ctas[b->all_derived][few][warps];
-        if (per_sm == 0) CK(batch_ctas_per_sm(warps, b->all_derived, few, &per_sm), "batch: occupancy");
+        const BatchKind kind = batch_kind(work, b->all_derived, b->curved);
+        int& per_sm = ctx->batch_ctas[(int)kind][warps];
+        if (per_sm == 0) CK(batch_ctas_per_sm(warps, kind, &per_sm), "batch: occupancy");
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(ctx->graph_stream, cudaStreamCaptureModeThreadLocal), "graph capture begin");
         vr_status es = batch_enqueue(ctx, b, o, nullptr, ctx->graph_stream);

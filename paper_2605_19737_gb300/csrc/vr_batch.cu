@@ -70,25 +70,25 @@ __device__ __forceinline__ void batch_body(const BatchLaunch& B) {
 
 // kBS: the skip-brick size shared by every view, or 0 when the views mix sizes.
 // kFew: a batch of few packets takes 128 registers, for more loads in flight per warp: the
-// three planes of the derived bricks cost a sparse ray twice the lines that records did, and a
-// small batch waits for them (one view of the 181x217x181 head with / without curvature, us at
-// 72 -> 128 registers: 64^2 1686 -> 770 / 478 -> 347, 256^2 867 -> 586 / 427 -> 360, 400x300
-// 791 -> 550 / 408 -> 348, 430^2 746 -> 716 / 422 -> 486: the line lies between the last two).
+// three planes of the derived bricks cost a sparse ray twice the lines that records did, and
+// the warps wait for them. The line (batch_few) lies at 28 packets per SM without curvature,
+// which reads one plane of the three, and at 170 with it (181x217x181 head, us at 72 -> 128
+// registers, by packets per SM; with curvature 64^2 (0.8) 1686 -> 770, 400x300 (25) 791 -> 550,
+// 16 views of 130x100 (43) 2062 -> 1275, of 260x200 (171) 2849 -> 2583, of 400x300 (395) 4150 ->
+// 4270; without 64^2 478 -> 347, 400x300 408 -> 348, 430^2 (38) 422 -> 486).
 template <bool kCount, bool kFew, int kBS>
 __global__ void __maxnreg__(kFew ? 128 : 72) k_render_batch_derived(const __grid_constant__ BatchLaunch B) {
     batch_body<true, kCount, kBS>(B);
 }
 
-template <bool kCount, bool kFew>
-__global__ void __launch_bounds__(256, kFew ? 2 : 3) k_render_batch_mixed(const __grid_constant__ BatchLaunch B) {
+template <bool kCount>
+__global__ void __launch_bounds__(256, 3) k_render_batch_mixed(const __grid_constant__ BatchLaunch B) {
     batch_body<false, kCount, 0>(B);
 }
 
 template <bool kCount, bool kFew>
-void launch_variant(const BatchLaunch& B, int ctas, int threads, bool all_derived, int bs, cudaStream_t st) {
-    if (!all_derived)
-        k_render_batch_mixed<kCount, kFew><<<ctas, threads, 0, st>>>(B);
-    else if (bs == 2)
+void launch_derived(const BatchLaunch& B, int ctas, int threads, int bs, cudaStream_t st) {
+    if (bs == 2)
         k_render_batch_derived<kCount, kFew, 2><<<ctas, threads, 0, st>>>(B);
     else if (bs == 3)
         k_render_batch_derived<kCount, kFew, 3><<<ctas, threads, 0, st>>>(B);
@@ -98,32 +98,37 @@ void launch_variant(const BatchLaunch& B, int ctas, int threads, bool all_derive
         k_render_batch_derived<kCount, kFew, 0><<<ctas, threads, 0, st>>>(B);
 }
 
+template <bool kCount>
+void launch_variant(const BatchLaunch& B, int ctas, int threads, BatchKind kind, int bs, cudaStream_t st) {
+    if (kind == BatchKind::kMixed)
+        k_render_batch_mixed<kCount><<<ctas, threads, 0, st>>>(B);
+    else if (kind == BatchKind::kFew)
+        launch_derived<kCount, true>(B, ctas, threads, bs, st);
+    else
+        launch_derived<kCount, false>(B, ctas, threads, bs, st);
+}
+
 }  // namespace
 
-bool batch_few(int packets) { return packets <= 28 * kSMs; }
+BatchKind batch_kind(int packets, bool all_derived, bool curved) {
+    if (!all_derived) return BatchKind::kMixed;
+    return packets <= (curved ? 170 : 28) * kSMs ? BatchKind::kFew : BatchKind::kMany;
+}
 
-cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, bool few, int* per_sm) {
-    // every variant of a family is held to the same registers, so one answers for all
-    auto kernel = all_derived ? (few ? k_render_batch_derived<false, true, 3> : k_render_batch_derived<false, false, 3>)
-                              : (few ? k_render_batch_mixed<false, true> : k_render_batch_mixed<false, false>);
+cudaError_t batch_ctas_per_sm(int warps_per_block, BatchKind kind, int* per_sm) {
+    // every variant of a kind is held to the same registers, so one answers for all
+    auto kernel = kind == BatchKind::kMixed ? k_render_batch_mixed<false>
+                  : kind == BatchKind::kFew ? k_render_batch_derived<false, true, 3>
+                                            : k_render_batch_derived<false, false, 3>;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, warps_per_block * 32, 0);
 }
 
-cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, bool all_derived, int bs,
+cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, BatchKind kind, int bs,
                                 cudaStream_t st) {
-    const int t = warps_per_block * 32;
-    const bool few = batch_few(B.n_work);
-    if (B.counters || !B.skip) {  // without skipping there is nothing to look ahead for either
-        if (few)
-            launch_variant<true, true>(B, ctas, t, all_derived, bs, st);
-        else
-            launch_variant<true, false>(B, ctas, t, all_derived, bs, st);
-    } else {
-        if (few)
-            launch_variant<false, true>(B, ctas, t, all_derived, bs, st);
-        else
-            launch_variant<false, false>(B, ctas, t, all_derived, bs, st);
-    }
+    if (B.counters || !B.skip)  // without skipping there is nothing to look ahead for either
+        launch_variant<true>(B, ctas, warps_per_block * 32, kind, bs, st);
+    else
+        launch_variant<false>(B, ctas, warps_per_block * 32, kind, bs, st);
     return cudaGetLastError();
 }
 

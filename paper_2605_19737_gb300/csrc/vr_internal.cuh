@@ -352,13 +352,15 @@ cudaError_t launch_wait_probe(unsigned* status, long long budget_cycles, cudaStr
 cudaError_t launch_check_probe(unsigned* status, cudaStream_t st);
 cudaError_t launch_channels_to_voxels(const float* dgrad, const int n[3], const float s[3], float* dvol,
                                       cudaStream_t st);
+// The kernels of a batch: some volume without derived bricks; few packets (curved: some view has
+// a curvature term); any other.
+enum class BatchKind { kMixed, kFew, kMany };
+BatchKind batch_kind(int packets, bool all_derived, bool curved);
+// CTAs of a kind's kernels that an SM holds.
+cudaError_t batch_ctas_per_sm(int warps_per_block, BatchKind kind, int* per_sm);
 // bs: the skip-brick size (log2 cells) every view shares, or 0 when they differ.
-cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, bool all_derived, int bs,
+cudaError_t launch_render_batch(const BatchLaunch& B, int warps_per_block, int ctas, BatchKind kind, int bs,
                                 cudaStream_t st);
-// Whether a batch of that many packets takes the kernels for few rays, and the CTAs of a
-// kernel that an SM holds.
-bool batch_few(int packets);
-cudaError_t batch_ctas_per_sm(int warps_per_block, bool all_derived, bool few, int* per_sm);
 cudaError_t launch_render_staged(const RenderLaunch& L, int warps_per_block, int ctas, cudaStream_t st);
 // The staged design on the derived bricks (skip bricks of 4^3 or 8^3 cells, bs 2 or 3).
 cudaError_t launch_render_staged_derived(const RenderLaunch& L, int warps_per_block, int ctas, cudaStream_t st);

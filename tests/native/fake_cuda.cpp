@@ -284,9 +284,10 @@ cudaError_t launch_check_probe(unsigned*, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_channels_to_voxels(const float*, const int*, const float*, float*, cudaStream_t) {
     return cudaSuccess;
 }
-cudaError_t launch_render_batch(const BatchLaunch&, int, int, bool, int, cudaStream_t) { return cudaSuccess; }
-bool batch_few(int) { return true; }
-cudaError_t batch_ctas_per_sm(int, bool, bool, int* n) {
+enum class BatchKind { kMixed, kFew, kMany };
+cudaError_t launch_render_batch(const BatchLaunch&, int, int, BatchKind, int, cudaStream_t) { return cudaSuccess; }
+BatchKind batch_kind(int, bool, bool) { return BatchKind::kFew; }
+cudaError_t batch_ctas_per_sm(int, BatchKind, int* n) {
     *n = 1;
     return cudaSuccess;
 }

@@ -64,3 +64,29 @@ def test_few_rays(torch, derived, brick, W, H):
                 ctx.synchronize()
                 assert torch.equal(out, want[0])
             assert torch.equal(kw["counters"], ctr)
+
+
+@pytest.mark.parametrize("gamma,W,H", [(0.0, 400, 340), (0.0, 400, 344), (0.4, 896, 920), (0.4, 896, 928)])
+def test_batch_line(torch, gamma, W, H):
+    """Batches on both sides of the line between their kernels: 28 packets of 8 x 4 rays per SM
+    (4256) without a curvature term, 170 (25840) with one; and one that crosses it by an update."""
+    import paper_2605_19737_gb300 as pkg
+    packets = -(-W // 8) * -(-H // 4)
+    line = 152 * (170 if gamma else 28)
+    assert abs(packets - line) < 300
+    cams = camera_array([orbit_camera(DIMS, SP, 40.0, 25.0, width=W, height=H)])
+    tf = np.zeros((1, 256, 4), np.float32)
+    tf[0, 128:] = (0.9, 0.5, 0.2, 0.02)
+    with pkg.Context(0) as ctx:
+        vid = _volume(ctx, True, 8)
+        out = torch.zeros((H, W, 4), device="cuda")
+        bid = ctx.batch_create([(vid, cams[0], out, W, H)])  # with a curvature term
+        for g in (0.4, gamma, 0.4):
+            ctx.set_tissue_params(vid, tf, shading=1, grad_mod=0, gamma=g, kappa_ref=0.05)
+            ctx.batch_update(bid)
+            want = ctx.render(vid, cams, W, H)[0]
+            for kw in (dict(), dict(graph=True), dict(graph=True, packet_w=4, warps_per_block=4)):
+                out.zero_()
+                ctx.batch_render(bid, **kw)
+                ctx.synchronize()
+                assert torch.equal(out, want)
