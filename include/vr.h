@@ -133,8 +133,9 @@ typedef struct {
                            at most 4 (8 is taken as 4: the image is the same); renders of
                            too few rays to fill the GPU (up to 200000, without counters) give
                            each ray several lanes and a shape of their own, whatever packet_w
-                           and warps_per_block say (again the same image); the staged
-                           kernel 1..8 */
+                           and warps_per_block say (again the same image); other renders
+                           and batches of fewer CTAs than the GPU has SMs run smaller ones;
+                           the staged kernel 1..8 */
     void* ray_state;    /* NULL, or device memory of n_cams*H*W x 8 bytes (per-lane kernels
                            only): vr_render writes, per pixel, the index of the ray's last
                            sample (int32; -1 for none) and the transmittance in front of it

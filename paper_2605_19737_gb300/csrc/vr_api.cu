@@ -148,10 +148,10 @@ vr_status cuda_fail(vr_ctx* c, cudaError_t e, const char* what) {
 // A refused allocation returns cudaErrorMemoryAllocation like a failed cudaMalloc.
 // A process that opens study after study makes eleven allocations and eleven frees for each:
 // once a volume has been freed, they come from a CUDA memory pool that the contexts on a device
-// share while there are any, and that keeps what is freed for the next allocation (181x217x181: cudaMalloc 251 us and
-// cudaFree 656, from the pool 9 and 4; load to first 720p frame and close 2.44 -> 1.44 ms). A
-// first study is cudaMalloc's: the pool would grow for it in 600 us and shrink in 900 (2.3 ms
-// more for the first growth in a process).
+// share while there are any, and that keeps what is freed for the next allocation (181x217x181:
+// cudaMalloc 251 us and cudaFree 656, from the pool 9 and 4; load to first 720p frame and close
+// 2.44 -> 1.45 ms). A first study is cudaMalloc's: the pool would grow for it in 600 us and
+// shrink in 900 (2.3 ms more for the first growth in a process).
 // What the pool keeps is bounded, and is not lost to others: the driver takes it back for any
 // cudaMalloc of the process that finds the device full, and the library when the last context
 // on the device is destroyed. A context with a memory limit does without.

@@ -54,7 +54,7 @@ __device__ __forceinline__ const float4* derived_brick(const VolumeDev& v, int b
 // faster offset order (fit step of 8 views 6.64 -> 6.07 ms; not at edge 4, whose corners
 // share L1 columns). Voxel and uniform gradients jump at table knots and at |g| = 0, and a
 // sum in another order puts single samples on the other side: there the order of the
-// corners stays as it has been (it costs 2 % of the 1080p gradient).
+// corners stays as it has been (about 2 % of the 1080p gradient, within what its runs differ).
 __host__ __device__ constexpr bool parity_order(bool table_only, int bs) { return !table_only || bs == 2; }
 
 // The sample field, from the derived bricks (voxel-wise derivatives) or by the
@@ -218,8 +218,9 @@ __device__ __forceinline__ void scatter_channels(float* __restrict__ dgrad, cons
 //   D = gz / 2sz + d_x(Hxz) / 4 sx sz + d_y(Hyz) / 4 sy sz,    S = Hzz / sz^2
 // the voxel is A + d_z(D) + s_z(S). A CTA owns 32 x 8 columns and walks a run of planes: the
 // ten channels of a plane (with their one-voxel border) go through shared memory once and D
-// and S of three planes stay in registers, so every channel is read from memory about 1.3
-// times instead of through 28 scattered loads per voxel (181x217x181: 291 -> 117 us, 312 MB).
+// and S of three planes stay in registers: 340 / 256 x (planes + 2) / planes loads per value, 1.55
+// in walks of twelve planes, most of the repeated ones from L2, instead of 28 scattered loads per
+// voxel (181x217x181: 291 -> 117 us; 312 MB is each value read and each voxel written once).
 constexpr int kVoxTileY = 8;
 __global__ void __launch_bounds__(256) k_channels_to_voxels(const float* __restrict__ G, int nx, int ny, int nz,
                                                             float sx, float sy, float sz, int planes,

@@ -169,8 +169,8 @@ void gauss_passes(const float* in, float* out, float* tmp, const int n[3], const
 // a CTA owns a 32 x 8 column of voxels and walks planes z0 .. z1 - 1. Each plane (with
 // its one-voxel border) is staged in shared memory once, loaded a plane ahead; a thread
 // reads the nine in-plane neighbours it needs and keeps those of the planes below and
-// above in registers: 9 shared reads and 1.3 global loads per voxel instead of 19 loads
-// (pass A of 256x256x176: 64 -> 36 us).
+// above in registers: 9 shared reads and 340 / 256 x (planes + 2) / planes global loads per voxel (1.5
+// in walks of 16 planes) instead of 19 loads (pass A of 256x256x176: 64 -> 36 us).
 // emit(z, H) is called by every thread of the CTA for every plane.
 // A short volume gets shorter walks (march_planes): with 16 planes per CTA 42x41x62 had 48
 // CTAs, each a chain of 18 plane loads, and took 162 us for two scales (now 94).

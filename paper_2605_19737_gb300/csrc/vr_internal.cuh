@@ -52,7 +52,10 @@ __host__ __device__ __forceinline__ constexpr long long der_brick_floats(int bs)
 // curvature term only the first plane is read, 16 of 16 bytes instead of 16 of 48.
 // Measured, records -> planes: 1080p frame of the 181x217x181 head 1.88 -> 1.82 ms, its
 // 540p at B = 16 0.84 -> 0.77, 32 views without curvature 8.88 -> 8.27, fit step of 8 views
-// 6.90 -> 6.07. B = 4 has no room for the padding (planes:
+// 6.90 -> 6.07. What a sparse ray with curvature reads lies on twice the lines that records did
+// (12-13 a sample instead of 6-7; 64x64 of the head at one lane per ray and 64 registers 1195 ->
+// 1645 us): launches of few rays give a ray several lanes or a warp more registers, after which
+// they are faster than with records. B = 4 has no room for the padding (planes:
 // 700x600 0.78 -> 0.81 ms) and keeps the records. Kernels take the layout of a fixed B: as
 // run-time values it cost the launches of several lanes per ray 3 %.
 struct DerLayout {

@@ -4,7 +4,7 @@
 // pixel packet (4 x 8 by default: 6 % faster than 8 x 4 or 16 x 2 at 1080p) and a
 // CTA a 16x8 tile. Each lane walks its own samples front to back; per sample it
 // reads its cell straight from HBM/L2 through L1 -- the 8 corners of the derived
-// bricks (voxel-wise I, gradient, Hessian: three 16-byte loads per corner) when
+// bricks (voxel-wise I, gradient, Hessian: a 16-, a 16- and an 8-byte load per corner) when
 // they were built, else the 56 weighted voxels of the 4x4x4 neighbourhood of the
 // intensity bricks with the separable stencils -- evaluates Eq. 4 and the
 // shading, and composites by Eqs. 5-6. Empty cells are leapt over by the skip
@@ -149,13 +149,25 @@ void launch_gather_bs(const RenderLaunch& L, dim3 grid, int threads, cudaStream_
 
 // Lanes per ray of a launch with that many rays. One lane per ray fills the chip at
 // 152 SMs x 32 warps x 32 = 156 k rays; below that the time is one ray's serial chain.
-// Measured us at 1 / 2 / 4 / 8 / 16 lanes (128^3 head; 181x217x181 head, 2D table):
-//   64 x 64     226 / 100 /  59 /  37 /  29
-//   128 x 128   203 /  96 /  64 /  49 /  59      990 / 326 / 186 / 127 / 141
-//   256 x 256   180 / 121 / 113 / 129 / 170      678 / 367 / 316 / 301 / 333
-//   400 x 300                                    677 / 414 / 394 / 388 / 449
-//   384 x 384   201 / 192 / 208 / 266 / 369
-//   512 x 512   272 / 294 / 342 / 459 / 649      728 / 700 / 780 / 966 / 1207
+// Measured us at 1 / 2 / 4 / 8 / 16 lanes, 128^3 head with a 1D table and 181x217x181 head with a
+// 2D table and curvature, derived bricks:
+//    90 x 90    113 /  62 /  39 /  27 /  29     1264 / 477 / 248 / 120 /   88
+//   128 x 128    96 /  60 /  39 /  37 /  43     1053 / 409 / 221 / 126 /  143
+//   180 x 150    92 /  59 /  43 /  45 /  56      949 / 370 / 211 / 171 /  176
+//   256 x 256    88 /  65 /  69 /  88 / 123      633 / 329 / 288 / 320 /  401
+//   400 x 300    97 /  85 /  88 / 123 / 181      635 / 352 / 340 / 417 /  539
+//   384 x 384   111 / 106 / 116 / 174 / 262      563 / 466 / 449 / 621 /  824
+//   440 x 440   130 / 127 / 145 / 222 / 341      622 / 530 / 540 / 782 / 1057
+//   512 x 512   153 / 157 / 184 / 295 / 458      660 / 628 / 678 / 1020 / 1394
+// and per-sample stencils:
+//    90 x 90    164 /  70 /  44 /  37 /  37      452 / 187 / 112 /  80 /   71
+//   180 x 150   129 /  70 /  55 /  56 /  68      386 / 195 / 164 / 131 /  143
+//   256 x 256   128 / 101 /  96 / 110 / 156      374 / 245 / 242 / 261 /  341
+//   400 x 300   150 / 119 / 124 / 151 / 224      468 / 324 / 303 / 345 /  467
+//   440 x 440   202 / 190 / 212 / 276 / 426      573 / 512 / 538 / 666 /  944
+//   512 x 512   238 / 239 / 272 / 365 / 572      671 / 640 / 702 / 884 / 1268
+// One set of lines serves the four columns: 36 % from the best of its row at 90 x 90 with
+// curvature, elsewhere 13 % at most.
 int render_lanes(long long rays) {
     return rays <= 6000 ? 16 : rays <= 28000 ? 8 : rays <= 100000 ? 4 : rays <= 200000 ? 2 : 1;
 }
