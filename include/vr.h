@@ -471,12 +471,12 @@ vr_status vr_debug_check_probe(vr_ctx* ctx);
 /* Device memory held by the context: every buffer the library allocates for it
  * (volumes, derived bricks, cell grids, vesselness, batches, scratch) is counted
  * in *bytes; caller-owned buffers (images, counters, ray state) are not, nor is freed memory
- * that the library keeps for later allocations of any context on the device, once a volume has
- * been freed there: at most 2 GiB per device, which the driver takes back for any cudaMalloc of
- * the process that finds the device full, and which is given back when the last context on the
- * device is destroyed; a context with a memory limit does without. Every call that frees
- * buffers waits for the device, as cudaFree does; where a capture forbids that, the buffers stay
- * with the context, counted, until a later such call. */
+ * that the library keeps for later allocations of any context on the device, once a volume (or
+ * its derived bricks, for another brick size) has been freed there: at most 2 GiB per device,
+ * which the driver takes back for any cudaMalloc of the process that finds the device full, and
+ * which is given back when the last context on the device is destroyed; a context with a memory
+ * limit does without. Every call that frees buffers waits for the device, as cudaFree does; where
+ * a capture forbids that, the buffers stay with the context, counted, until a later such call. */
 vr_status vr_memory_used(vr_ctx* ctx, unsigned long long* bytes);
 
 /* Cap on vr_memory_used (0, the default: no cap beyond the device's memory). An

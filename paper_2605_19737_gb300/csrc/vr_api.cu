@@ -147,11 +147,12 @@ vr_status cuda_fail(vr_ctx* c, cudaError_t e, const char* what) {
 // (vr_set_memory_limit) and can be made to see an allocation fail (vr_debug_fail_alloc).
 // A refused allocation returns cudaErrorMemoryAllocation like a failed cudaMalloc.
 // A process that opens study after study makes eleven allocations and eleven frees for each:
-// once a volume has been freed, they come from a CUDA memory pool that the contexts on a device
-// share while there are any, and that keeps what is freed for the next allocation (181x217x181:
-// cudaMalloc 251 us and cudaFree 656, from the pool 9 and 4; load to first 720p frame and close
-// 2.44 -> 1.45 ms). A first study is cudaMalloc's: the pool would grow for it in 600 us and
-// shrink in 900 (2.3 ms more for the first growth in a process).
+// once a volume has been freed (or its derived bricks, for another edge), they come from a CUDA
+// memory pool that the contexts on a device share while there are any, and that keeps what is
+// freed for the next allocation (181x217x181: cudaMalloc 251 us and cudaFree 656, from the pool 9
+// and 4; load to first 720p frame and close 2.44 -> 1.45 ms). A first study is cudaMalloc's: the
+// pool would grow for it in 600 us and shrink in 900 (2.3 ms more for the first growth in a
+// process).
 // What the pool keeps is bounded, and is not lost to others: the driver takes it back for any
 // cudaMalloc of the process that finds the device full, and the library when the last context
 // on the device is destroyed. A context with a memory limit does without.
@@ -160,7 +161,7 @@ struct DevicePool {
     const int device;
     const unsigned long long cuda_ctx;  // id of the CUDA context whose stream it is
     int users = 1;                      // library contexts
-    std::atomic<bool> wanted{false};    // a volume has been freed
+    std::atomic<bool> wanted{false};    // something large has been freed (Freeing::reopens)
     std::atomic<bool> ready{false};     // the rest is there
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;  // orders allocations and frees, and runs nothing
@@ -323,7 +324,7 @@ class Freeing {
         ctx_->mem_used -= it->second.bytes;
         ctx_->allocs.erase(it);
     }
-    // A volume has been freed: the next one's buffers come from the pool.
+    // A volume has been freed, or its derived bricks for others: the next ones come from the pool.
     void reopens() {
         if (ctx_->pool && !ctx_->pool->ready && !ctx_->mem_limit) ctx_->pool->wanted = true;
     }
@@ -955,6 +956,7 @@ vr_status vr_set_brick_size(vr_ctx* ctx, int vol_id, int cells) {
     fr(v->d_grid);
     fr(v->d_empty);
     fr(v->d_dbricks);
+    if (v->d_dbricks) fr.reopens();
     v->d_grid = nullptr, v->d_empty = nullptr, v->d_dbricks = nullptr;
     v->bs = bs;
     for (int a = 0; a < 3; ++a) v->nb[a] = (v->n[a] - 1 + (1 << bs) - 1) >> bs;

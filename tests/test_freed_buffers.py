@@ -211,7 +211,8 @@ def test_what_is_kept_is_bounded(lib):
 
 def test_pool_from_the_second_study_on(lib):
     """A context that opens one study allocates as without a pool; one that opens another, and
-    any beside it, from the pool; one with a memory limit never."""
+    any beside it, from the pool, as does one that changes its derived bricks; one with a memory
+    limit never."""
     before = lib.fake_pool_allocs()
     c, d = Lib(lib, reopens=False), Lib(lib, reopens=False)
     vid = c.open(20)
@@ -233,6 +234,11 @@ def test_pool_from_the_second_study_on(lib):
     for x in (c, d, e):
         x.close()
     f = Lib(lib, reopens=False)  # the last context has ended: as in a new process
-    f.open(20)
+    vid = f.load(20)
+    f.ok(lib.vr_set_brick_size(f.h, vid, 4))  # before there are derived bricks
+    f.ok(lib.vr_precompute_morphology(f.h, vid, None, 0))
     assert lib.fake_pool_allocs() == two
+    f.ok(lib.vr_set_brick_size(f.h, vid, 16))  # and in exchange for others
+    f.ok(lib.vr_precompute_morphology(f.h, vid, None, 0))
+    assert lib.fake_pool_allocs() > two
     f.close()
